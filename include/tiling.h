@@ -348,10 +348,11 @@ void tl_blob_free(tl_blob* b);
  * horizontal dominoes if it is below 2^31, else two vertical ones.  Writes
  * the canonical state of tl_domain_aztec(n) to `canon` (host or device, cap
  * >= 2 (2n+1)^2).  Synchronous.  The context keeps the device buffers
- * (about 20 n^2 bytes) and one captured graph of the whole sample
- * for the last order used, until tl_ctx_destroy or a call with another
- * order; calls on one context are serialised.  Errors: TL_EINVAL,
- * TL_ENOMEM, TL_ECUDA. */
+ * (n^2 bytes of packed rows, twice that for orders whose rows do not fit on
+ * chip, and 8 n^2 bytes once a result has gone to host memory) for the last
+ * order used, until tl_ctx_destroy or a call with another order; calls on one
+ * context are serialised.  Errors: TL_EINVAL, TL_ENOMEM, TL_ECUDA,
+ * TL_ETIMEOUT (a bounded device wait gave up). */
 int tl_aztec_shuffle(tl_ctx* ctx, int n, uint64_t seed, uint32_t stream_id, uint8_t* canon, size_t cap,
                      void* stream);
 

@@ -72,20 +72,22 @@ TL_API const char* tl_version(void) { return "tiling-gb300 0.1 (sm_103a)"; }
 // ---------------------------------------------------------------------------
 // Context
 // ---------------------------------------------------------------------------
-// Domino shuffling of one order n, kept per context: the device buffers and
-// one instantiated graph of the whole sample (zeroing, 2n + 1 kernels), so a
-// sample costs one graph launch instead of 2n + 1 host launches.  The key is
-// read by the kernels from `rng`, written before each launch.
+// Domino shuffling of one order n, kept per context: the packed rows of the
+// sample, and the stripes and exchange buffer of the resident kernel or, for
+// orders whose rows do not fit on chip, the second buffer of the per-step one.
 struct ShuffleCache {
     int n = 0;
-    uint8_t *A = nullptr, *B = nullptr, *F = nullptr, *canon = nullptr;
+    Geom g{};
+    uint32_t *rows = nullptr, *alt = nullptr;
+    uint8_t* canon = nullptr;   // staging of results read to host memory
+    int* stripe = nullptr;
+    unsigned long long* xbuf = nullptr;
     int* status = nullptr;
-    DevRng* rng = nullptr;
-    cudaGraphExec_t exec = nullptr;
+    std::vector<ShufflePlan> seg;   // empty: one launch per step
+    size_t xbuf_words = 0;
     void release()
     {
-        if (exec) cudaGraphExecDestroy(exec);
-        cudaFree(A); cudaFree(B); cudaFree(F); cudaFree(canon); cudaFree(status); cudaFree(rng);
+        cudaFree(rows); cudaFree(alt); cudaFree(canon); cudaFree(stripe); cudaFree(xbuf); cudaFree(status);
         *this = ShuffleCache();
     }
 };
@@ -2052,44 +2054,124 @@ TL_API int tl_state_hash(tl_chain* c, uint64_t* out, void* stream)
     return TL_OK;
 }
 
-// Buffers and graph of order n (rebuilt when n changes).
+// Stripes of a resident shuffling launch whose last step is K: bounds of the
+// rows n - K .. n + K that balance the work of that step, or an empty vector
+// if they do not fit the SMs' shared memory.
+//
+// A step costs a stripe about 4 warp instructions per word it looks at and
+// 2.4 per block it fills (a quarter of the blocks inside the inscribed
+// circle).  The stripe through the middle is the slowest at every step, so
+// balancing the last step balances them all.  Stripes are added while they
+// hold at least `kStripeWork` of it: below that a step is bound by its latency,
+// and a seam only adds exchanges.
+static std::vector<int> shuffle_stripes(const tl_ctx* ctx, int n, int K, int Kw, int h, size_t* smem)
+{
+    const int H = 2 * K + 1;
+    const int cap = (int)(((size_t)ctx->smem_optin - shuffle_static_smem()) / shuffle_smem_bytes(1, Kw));   // local rows that fit
+    std::vector<double> pre(H + 1, 0.0);
+    for (int y = 0; y < H; ++y) {
+        const double d = std::abs(y - K), chord = 0.5 * K * K - d * d;
+        pre[y + 1] = pre[y] + 4.0 * ((K - d) / 32 + 1) + 0.6 * std::sqrt(std::max(0.0, chord));
+    }
+    const double kStripeWork = 1000.0;
+    const int want = std::min(ctx->sms, std::max(1, (int)(pre[H] / kStripeWork)));
+    auto partition = [&](double T, std::vector<int>& lo) {
+        lo.assign(1, 0);
+        for (int a = 0; a < H;) {
+            int b = std::min(H, a + h);
+            auto local = [&](int e) { return (e < H ? e + h : H) - (a > 0 ? a - h : 0); };
+            if (local(b) > cap) return false;
+            while (b < H && pre[b + 1] - pre[a] <= T && local(b + 1) <= cap) ++b;
+            if (b < H && H - b < h) {
+                b = H - h;
+                if (b - a < h) return false;
+            }
+            lo.push_back(b);
+            a = b;
+            if ((int)lo.size() - 1 > want) return false;
+        }
+        return true;
+    };
+    std::vector<int> best, tmp;
+    if (cap < 1 || !partition(pre[H] + 1, best)) return {};
+    double tlo = 0, thi = pre[H] + 1;
+    for (int it = 0; it < 40; ++it) {
+        const double mid = 0.5 * (tlo + thi);
+        if (partition(mid, tmp)) {
+            thi = mid;
+            best = tmp;
+        } else {
+            tlo = mid;
+        }
+    }
+    const int C = (int)best.size() - 1;
+    int nloc = 0;
+    for (int k = 0; k < C; ++k)
+        nloc = std::max(nloc, (k < C - 1 ? best[k + 1] + h : H) - (k > 0 ? best[k] - h : 0));
+    *smem = shuffle_smem_bytes(nloc, Kw);
+    for (int& y : best) y += n - K;
+    return best;
+}
+
+// Buffers and stripes of order n (rebuilt when n changes).
 static int shuffle_prepare(tl_ctx* ctx, int n)
 {
     ShuffleCache& sc = ctx->shuffle;
-    if (sc.n == n && sc.exec) return TL_OK;
+    if (sc.n == n) return TL_OK;
     CUDA_TRY(cudaDeviceSynchronize());
     sc.release();
-    // cell buffers: 2n rows of 2n bytes rounded up to 4
-    const size_t W = 2 * (size_t)n + 1, ncanon = 2 * W * W,
-                 ncell = (size_t)2 * n * ((2 * (size_t)n + 3) & ~(size_t)3);
+    sc.g = make_geom(LAT_DOMINO, 2 * n + 1, 2 * n + 1, 0);
+    const int h = 4;
+    // launches: the last covers steps up to n; each one before it ends where
+    // the work of a step is half as much (the middle stripe of a launch's
+    // partition does up to its last step's share of it all the time)
+    std::vector<int> last(1, n);
+    while (last.back() > 560) last.push_back(last.back() * 5 / 7);
+    std::reverse(last.begin(), last.end());
+    std::vector<int> stripes;
+    std::vector<size_t> first;
+    size_t max_smem = 0;
+    for (int K : last) {
+        ShufflePlan sp{};
+        const std::vector<int> lo = shuffle_stripes(ctx, n, K, sc.g.K, h, &sp.smem_bytes);
+        if (lo.empty()) break;
+        sp.last = K;
+        sp.ctas = (int)lo.size() - 1;
+        sp.halo = h;
+        max_smem = std::max(max_smem, sp.smem_bytes);
+        sc.xbuf_words = std::max(sc.xbuf_words, (size_t)sp.ctas * 4 * h * (size_t)sc.g.row_words);
+        first.push_back(stripes.size());
+        stripes.insert(stripes.end(), lo.begin(), lo.end());
+        sc.seg.push_back(sp);
+    }
+    int bps = 0;
+    bool fits = sc.seg.size() == last.size() && shuffle_prepare_kernel(max_smem, &bps) == 0;
+    for (const ShufflePlan& sp : sc.seg) fits = fits && sp.ctas <= bps * ctx->sms;
     int rc;
-    if ((rc = dev_alloc(&sc.A, ncell, "shuffle cells")) || (rc = dev_alloc(&sc.B, ncell, "shuffle cells")) ||
-        (rc = dev_alloc(&sc.F, ncell, "shuffle cells")) || (rc = dev_alloc(&sc.canon, ncanon, "shuffle output")) ||
-        (rc = dev_alloc(&sc.status, 1, "status")) || (rc = dev_alloc(&sc.rng, 1, "shuffle key"))) {
+    if ((rc = dev_alloc(&sc.rows, (size_t)sc.g.total_words, "shuffle rows")) ||
+        (rc = dev_alloc(&sc.status, 1, "status"))) {
         sc.release();
         return rc;
     }
-    cudaStream_t cs = nullptr;
-    cudaGraph_t graph = nullptr;
-    cudaError_t e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
-    if (e == cudaSuccess) {
-        cudaError_t ec = cudaMemsetAsync(sc.A, 0, ncell, cs);
-        if (ec == cudaSuccess) ec = cudaMemsetAsync(sc.B, 0, ncell, cs);
-        if (ec == cudaSuccess) ec = cudaMemsetAsync(sc.F, 0, ncell, cs);
-        if (ec == cudaSuccess) ec = cudaMemsetAsync(sc.status, 0, sizeof(int), cs);
-        if (ec == cudaSuccess) ec = cudaMemsetAsync(sc.canon, 0, ncanon, cs);
-        if (ec == cudaSuccess) ec = (cudaError_t)launch_shuffle(n, sc.A, sc.B, sc.F, sc.rng, sc.status, sc.canon, cs);
-        e = cudaStreamEndCapture(cs, &graph);
-        if (e == cudaSuccess) e = ec;
+    if (!fits) {
+        sc.seg.clear();
+        rc = dev_alloc(&sc.alt, (size_t)sc.g.total_words, "shuffle rows");
+    } else {
+        if ((rc = dev_alloc(&sc.stripe, stripes.size(), "stripes")) == TL_OK)
+            rc = dev_alloc(&sc.xbuf, sc.xbuf_words, "exchange buffer");
+        if (rc == TL_OK &&
+            cudaMemcpy(sc.stripe, stripes.data(), sizeof(int) * stripes.size(), cudaMemcpyHostToDevice) != cudaSuccess)
+            rc = fail(TL_ECUDA, "tl_aztec_shuffle: stripes");
+        for (size_t i = 0; i < sc.seg.size(); ++i) {
+            sc.seg[i].stripe_lo = sc.stripe + first[i];
+            sc.seg[i].xbuf = sc.xbuf;
+            sc.seg[i].status = sc.status;
+        }
     }
-    if (e == cudaSuccess) e = cudaGraphInstantiate(&sc.exec, graph, 0);
-    if (graph) cudaGraphDestroy(graph);
-    if (cs) cudaStreamDestroy(cs);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
+    if (rc == TL_OK && cudaMemset(sc.status, 0, sizeof(int)) != cudaSuccess) rc = fail(TL_ECUDA, "tl_aztec_shuffle: memset");
+    if (rc != TL_OK) {
         sc.release();
-        return fail(TL_ECUDA, "tl_aztec_shuffle: graph of order %d: %s", n, cudaGetErrorString(e));
+        return rc;
     }
     sc.n = n;
     return TL_OK;
@@ -2108,16 +2190,23 @@ TL_API int tl_aztec_shuffle(tl_ctx* ctx, int n, uint64_t seed, uint32_t stream_i
     TL_TRY(shuffle_prepare(ctx, n));
     ShuffleCache& sc = ctx->shuffle;
     const DevRng rng{(uint32_t)seed, (uint32_t)(seed >> 32), stream_id};
+    const bool dev = is_device_ptr(canon);
+    if (!dev && !sc.canon) TL_TRY(dev_alloc(&sc.canon, ncanon, "shuffle output"));
     int hstatus = 0;
-    cudaError_t e = cudaMemcpyAsync(sc.rng, &rng, sizeof(rng), cudaMemcpyHostToDevice, SS(stream));
-    if (e == cudaSuccess) e = cudaGraphLaunch(sc.exec, SS(stream));
+    cudaError_t e =
+        (cudaError_t)(!sc.seg.empty()
+                          ? launch_shuffle(sc.seg.data(), (int)sc.seg.size(), n, sc.g.K, (size_t)sc.g.total_words,
+                                           sc.xbuf_words, sc.rows, rng, stream)
+                          : launch_shuffle_global(n, sc.g.K, (size_t)sc.g.total_words, sc.rows, sc.alt, rng, stream));
+    if (e == cudaSuccess) e = (cudaError_t)launch_unpack(sc.g, sc.rows, dev ? canon : sc.canon, stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&hstatus, sc.status, sizeof(int), cudaMemcpyDeviceToHost, SS(stream));
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(canon, sc.canon, ncanon, is_device_ptr(canon) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
-                            SS(stream));
+    if (e == cudaSuccess && !dev) e = cudaMemcpyAsync(canon, sc.canon, ncanon, cudaMemcpyDeviceToHost, SS(stream));
     if (e == cudaSuccess) e = cudaStreamSynchronize(SS(stream));
     if (e != cudaSuccess) return fail(TL_ECUDA, "tl_aztec_shuffle: %s", cudaGetErrorString(e));
-    if (hstatus) return fail(TL_ECUDA, "tl_aztec_shuffle: a created block was not a 2x2 hole");
+    if (hstatus) {
+        CUDA_TRY(cudaMemset(sc.status, 0, sizeof(int)));
+        return fail(TL_ETIMEOUT, "tl_aztec_shuffle: a bounded wait gave up");
+    }
     return TL_OK;
 }
 

@@ -78,12 +78,28 @@ int launch_density_read(const uint32_t* counts, uint64_t n, uint64_t samples, do
                         void* stream);
 int launch_nsew(const Geom& g, const uint32_t* counts, uint64_t samples, int kappa, double* out,
                 void* stream);
-// Domino shuffling of the Aztec diamond of order n: A, B, F are zeroed
-// device scratch of 2n rows of (2n rounded up to 4) bytes each, rng a device
-// copy of the key, canon the zeroed [2][2n+1][2n+1] output; status is raised
-// if a created block is not a 2x2 hole.  Capturable into a graph.
-int launch_shuffle(int n, uint8_t* A, uint8_t* B, uint8_t* F, const DevRng* rng, int* status, uint8_t* canon,
-                   void* stream);
+// Domino shuffling of the Aztec diamond of order n (tl_shuffle.cu) into
+// packed rows of the diamond's chain layout (Kw words per plane row).
+// Resident form: cooperative launches of consecutive steps, in each of which
+// stripe c holds the vertex rows [stripe_lo[c], stripe_lo[c + 1]) and `halo`
+// rows on each side.
+struct ShufflePlan {
+    int last;                      // last step of the launch
+    int ctas;
+    int halo;                      // = steps per exchange
+    size_t smem_bytes;             // dynamic shared memory per CTA
+    const int* stripe_lo;          // device [ctas + 1]
+    unsigned long long* xbuf;      // device [ctas][2][2][4 halo Kw] tagged words, shared by the launches
+    int* status;                   // device error word: 0 ok, 1 a bounded wait gave up
+};
+size_t shuffle_smem_bytes(int local_rows, int Kw);
+size_t shuffle_static_smem();
+int shuffle_prepare_kernel(size_t smem_bytes, int* blocks_per_sm);
+int launch_shuffle(const ShufflePlan* seg, int nseg, int n, int Kw, size_t total_words, size_t xbuf_words,
+                   uint32_t* rows, const DevRng& rng, void* stream);
+// One launch per step over two global buffers of total_words words each; the
+// sample ends in A.
+int launch_shuffle_global(int n, int Kw, size_t total_words, uint32_t* A, uint32_t* B, const DevRng& rng, void* stream);
 // seg: [nseg][6] height segments (y, lo, hi, parent, xs, dir); base_scratch: nseg ints.
 int launch_height(const Geom& g, const uint32_t* rows, const int* seg, int nseg, int hw, int hh,
                   int32_t* out, int* base_scratch, void* stream);

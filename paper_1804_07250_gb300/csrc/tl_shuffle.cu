@@ -1,232 +1,435 @@
 // Domino shuffling: exact uniform random tilings of the Aztec diamond (the
 // shuffling algorithms the paper names as an alternative exact sampler,
-// Sec. 3; Elkies, Kuperberg, Larsen and Propp).
+// Sec. 3; Elkies, Kuperberg, Larsen and Propp), in the face-local form of
+// Propp's generalized domino-shuffling.
 //
-// Cells are unit squares with lower-left corner (x, y), x, y in [-n, n); the
-// diamond of order k holds the cells with |x + 1/2| + |y + 1/2| <= k.  A
-// cell stores which part of a domino covers it (empty, left / right half of
-// a horizontal domino, bottom / top half of a vertical one), one byte per
-// cell, rows of S = 2n rounded up to 4 bytes.  In order k a horizontal
-// domino with left cell (x, y) goes north if x + y + k is even, else south;
-// a vertical one with bottom cell (x, y) goes east if x + y + k is even, else
-// west.  One step k -> k + 1 is two data-parallel kernels, each thread
-// taking the four cells of one 32-bit word:
-//  1. move (gather): every cell of order k + 1 looks at the four cells a
-//     domino could arrive from, and takes the part of the one that moves in,
-//     unless it is in a bad block (a north-going domino right below a
-//     south-going one, or an east-going one right left of a west-going one);
-//     all it reads lies in the 3 x 3 cells around it;
-//  2. fill: the cells left empty form disjoint 2x2 blocks whose lower-left
-//     cells have x + y + k + 1 odd, stacked from the bottom of every run of
-//     empty cells in a column.  An empty cell finds its block from its 3 x 3
-//     neighbourhood, or where that allows two blocks, from the parity of the
-//     run below it and that lower-left parity, and takes its
-//     part of the pair the block's Philox draw picks (two horizontal
-//     dominoes below 2^31, else two vertical ones).  The result goes to a
-//     third buffer, so no thread sees another's output.
+// Cells are unit squares with lower-left corner (x, y), x, y in [-n, n); in
+// order k a horizontal domino with left cell (x, y) goes north if x + y + k
+// is even, else south, a vertical one with bottom cell (x, y) east or west.
+// Seen from the 2x2 blocks of cells with x + y + K odd (K = k + 1), every
+// domino of order k lies along one side of exactly one such block of the
+// order-K diamond and moves to the opposite side of it; two dominoes of one
+// block destroy each other, and a block without any gets a new pair.  So a
+// step is one bitwise update of the four edges of every block of one colour
+// class, on the same packed edge planes as the chain's passes: with (X, Y)
+// the canonical vertex in the middle of the block (X = x + 1 + n, Y = y + 1 +
+// n), E = Hz(X, Y), W = Hz(X-1, Y), N = Vt(X, Y), S = Vt(X, Y-1):
+//   E' = W & ~E | v,  W' = E & ~W | v,  N' = S & ~N | h,  S' = N & ~S | h,
+// h and v the blocks with no edge whose draw picks a horizontal or a vertical
+// pair.  All K^2 blocks cover all edges of the diamond, so a step rewrites
+// every word in reach and the buffers alternate.
+//
+// Packed rows: planes He, Ho, Ve, Vo (edges at even and odd X), Kw words each.
+// A row's class alternates its parity p = (Y + K + 1) & 1 every step.  At
+// p = 0 the W edges are the odd plane moved up by one site; the step leaves
+// them there (word j of Ho then holds the odd edges left of its sites), and
+// the next step of the row, at p = 1, moves them back as it reads.  No
+// word is ever shared by two writers.
 #include "tl_device.cuh"
 
 #include <cstdint>
 
 namespace tl {
 
-enum : uint8_t { SH_EMPTY = 0, SH_HL = 1, SH_HR = 2, SH_VB = 3, SH_VT = 4 };
-
-TL_DEV bool in_diamond(int x, int y, int k) { return abs(2 * x + 1) + abs(2 * y + 1) <= 2 * k; }
-
-// Row pitch of the cell buffers in bytes.
-TL_DEV int cell_pitch(int n) { return (2 * n + 3) & ~3; }
-
-// Word of this thread: block row blockIdx.y is diamond row y = blockIdx.y - K,
-// whose cells are x in [-w, w) with w = K - |y + 1/2| + 1/2; its words run
-// from the one holding x = -w to the one holding x = w - 1.  Threads past
-// them return false.
-TL_DEV bool row_word(int n, int K, int& wi, int& y)
+constexpr int kShufThreads = 512, kShufWarps = kShufThreads / 32;
+// per warp: the blocks to fill of 32 words (at most 1024), and their draws
+struct ShufScratch {
+    uint16_t list[1024];
+    uint32_t coin[32];
+};
+struct ShufParams {
+    int n, Kw;                  // order, words per plane row (multiple of 4)
+    int h;                      // halo rows per side = steps per exchange
+    int K0, K1;                 // the launch runs steps K0 .. K1
+    const int* stripe_lo;       // [C + 1] vertex rows, n - K1 .. n + K1 + 1
+    DevRng rng;
+    unsigned long long* xbuf;   // [C][2][2][4 h Kw] tagged words, cleared before step 1
+    uint32_t* rows0;            // packed rows (chain layout), row 0: as step K0 - 1 left them, then as step K1 does
+    int* status;
+};
+TL_DEV void sh_ld2(const unsigned long long* p, unsigned long long* a, unsigned long long* b)
 {
-    y = (int)blockIdx.y - K;
-    const int w = K - (y >= 0 ? y : -y - 1);
-    const int wlo = (n - w) >> 2, whi = (n + w + 3) >> 2;
-    wi = wlo + (int)(blockIdx.x * blockDim.x + threadIdx.x);
-    return wi < whi;
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(*a), "=l"(*b) : "l"(p) : "memory");
 }
-
-// Word wi of buffer row r; 0 (four empty cells) outside the buffer.
-TL_DEV uint32_t word_at(const uint8_t* A, int n, int S, int r, int wi)
+TL_DEV void sh_st2(unsigned long long* p, unsigned long long a, unsigned long long b)
 {
-    if (r < 0 || r >= 2 * n || wi < 0 || wi >= S / 4) return 0u;
-    return reinterpret_cast<const uint32_t*>(A + (size_t)r * S)[wi];
+    asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(a), "l"(b) : "memory");
 }
-
-TL_DEV uint8_t byte_of(uint32_t w, int i) { return (uint8_t)(w >> (8 * i)); }
-
-// Cells 4 wi - 1 .. 4 wi + 4 of buffer rows r - 1, r, r + 1: cw[1 + dy][1 + i + dx]
-// is the cell (dx, dy) away from cell i of word wi.
-TL_DEV void load_window(const uint8_t* A, int n, int S, int r, int wi, uint8_t (&cw)[3][6])
+TL_DEV uint64_t sh_globaltimer()
 {
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        const uint32_t a = word_at(A, n, S, r - 1 + d, wi - 1), b = word_at(A, n, S, r - 1 + d, wi),
-                       c = word_at(A, n, S, r - 1 + d, wi + 1);
-        cw[d][0] = byte_of(a, 3);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) cw[d][1 + i] = byte_of(b, i);
-        cw[d][5] = byte_of(c, 0);
+    uint64_t t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+constexpr uint64_t kShufWaitLimitNs = 2000000000ull;   // 2 s: far beyond any healthy exchange
+
+// The draws of step K: bit 31 of word 0 of Philox4x32-10 with counter
+// (c0, K, 0xFFFE0000, stream), clear for a horizontal pair.  Only c0 differs
+// between the blocks of a step: the second product of round 1 is a constant
+// and the first of round 2 the same for the whole step, and the last two
+// rounds need one word each.  17 products per draw instead of 20.
+struct ShufDraw {
+    uint32_t a1, m2lo, m2hi;   // of the step
+    uint32_t stream, k0, k1;
+    TL_DEV ShufDraw(uint32_t K, const DevRng& rng)
+    {
+        constexpr uint64_t m = (uint64_t)0xFFFE0000u * 0xCD9E8D57u;
+        a1 = (uint32_t)m;
+        const uint32_t a0 = (uint32_t)(m >> 32) ^ K ^ rng.k0;
+        m2lo = a0 * 0xD2511F53u;
+        m2hi = __umulhi(a0, 0xD2511F53u);
+        stream = rng.stream;
+        k0 = rng.k0;
+        k1 = rng.k1;
     }
-}
-
-__global__ void shuffle_move_kernel(const uint8_t* __restrict__ A, uint8_t* __restrict__ B, int n, int k)
-{
-    const int K = k + 1, S = cell_pitch(n);
-    int wi, y;
-    if (!row_word(n, K, wi, y)) return;
-    const int r = y + n;
-#ifdef TL_DEBUG
-    // the word written: row r of 2n cell rows, bytes 4 wi .. 4 wi + 3 of a pitch-S row
-    if (!(TL_IN(r, 2 * n, 501) && TL_IN(4 * wi + 3, S, 502))) return;
-#endif
-    uint8_t cw[3][6];
-    load_window(A, n, S, r, wi, cw);
-    uint32_t outw = 0;
+    TL_DEV bool horizontal(uint32_t c0) const
+    {
+        uint32_t q0 = k0, q1 = k1;
+        const uint32_t a2 = __umulhi(c0, 0xD2511F53u) ^ stream ^ q1, a3 = c0 * 0xD2511F53u;
+        q0 += 0x9E3779B9u;
+        q1 += 0xBB67AE85u;
+        uint32_t x0 = __umulhi(a2, 0xCD9E8D57u) ^ a1 ^ q0, x1 = a2 * 0xCD9E8D57u, x2 = m2hi ^ a3 ^ q1, x3 = m2lo;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int x = 4 * wi + i - n;
-        if (!in_diamond(x, y, K)) continue;
-        uint8_t out = SH_EMPTY;
-        // from below, going north; destroyed if the cell above its left half
-        // holds the left half of a south-going one
-        uint8_t c = cw[0][1 + i];
-        if (c == SH_HL || c == SH_HR) {
-            const int ax = c == SH_HL ? x : x - 1;
-            if (((ax + y - 1 + k) & 1) == 0 && cw[1][1 + i + (ax - x)] != SH_HL) out = c;
+        for (int r = 2; r < 10; ++r) {
+            q0 += 0x9E3779B9u;
+            q1 += 0xBB67AE85u;
+            const uint32_t lo0 = x0 * 0xD2511F53u, hi0 = __umulhi(x0, 0xD2511F53u);
+            const uint32_t lo1 = x2 * 0xCD9E8D57u, hi1 = __umulhi(x2, 0xCD9E8D57u);
+            x0 = hi1 ^ x1 ^ q0;
+            x1 = lo1;
+            x2 = hi0 ^ x3 ^ q1;
+            x3 = lo0;
         }
-        c = cw[2][1 + i];   // from above, going south
-        if (c == SH_HL || c == SH_HR) {
-            const int ax = c == SH_HL ? x : x - 1;
-            if (((ax + y + 1 + k) & 1) == 1 && cw[1][1 + i + (ax - x)] != SH_HL) out = c;
-        }
-        c = cw[1][i];   // from the left, going east; destroyed by a west-going one right of it
-        if (c == SH_VB || c == SH_VT) {
-            const int ay = c == SH_VB ? y : y - 1;
-            if (((x - 1 + ay + k) & 1) == 0 && cw[1 + (ay - y)][1 + i] != SH_VB) out = c;
-        }
-        c = cw[1][2 + i];   // from the right, going west
-        if (c == SH_VB || c == SH_VT) {
-            const int ay = c == SH_VB ? y : y - 1;
-            if (((x + 1 + ay + k) & 1) == 1 && cw[1 + (ay - y)][1 + i] != SH_VB) out = c;
-        }
-        outw |= (uint32_t)out << (8 * i);
+        return (int)x0 >= 0;
     }
-    reinterpret_cast<uint32_t*>(B + (size_t)r * S)[wi] = outw;
+};
+
+// Columns that step K can touch in rows at distance >= d from the middle row:
+// words [lo, hi] of a plane row.
+TL_DEV void sh_words(int n, int K, int d, int& lo, int& hi)
+{
+    const int w = K - 1 - d;
+    lo = ((n - w - 1) >> 1) >> 5;
+    hi = ((n + w) >> 1) >> 5;
 }
 
-TL_DEV uint8_t cell_at(const uint8_t* A, int n, int S, int x, int y)
+// One warp's words of step K: lane's word k of row Y (`live` if it has one),
+// read from `src` and written to `dst`, both pointing at row Y (pitch RW
+// words; row Y - 1 holds the S edges).  The blocks to fill are sparse (a
+// quarter of the blocks in the disordered region, none in the frozen
+// corners) and uneven (8 +- 2.4 a word), and a draw costs a warp 68 cycles of
+// its scheduler's multiplier, so the warp lists them and its lanes share the
+// draws evenly, two in flight each.  Measured at order 2048: 7.3 ms a sample;
+// 9.5 with every lane drawing for its own word, 8.6 with the lanes drawing
+// for their own words until fewer than 20 have a block left.
+TL_DEV void sh_step_words(const uint32_t* src, uint32_t* dst, int Kw, int n, int K, int Y, int k, bool live,
+                          const ShufDraw& draw, ShufScratch& sc)
 {
-    if (x < -n || y < -n || x >= n || y >= n) return SH_EMPTY;
-    return A[(size_t)(y + n) * S + (x + n)];
-}
-
-// B (after the move, order K) -> C with every hole filled.
-// `rngp`: the Philox key and stream, read from device memory so that one
-// captured graph of the whole sample serves every seed.
-__global__ void shuffle_fill_kernel(const uint8_t* __restrict__ B, uint8_t* __restrict__ C, int n, int K,
-                                    const DevRng* __restrict__ rngp, uint32_t tbar, int* __restrict__ status)
-{
-    const int S = cell_pitch(n);
-    int wi, y;
-    if (!row_word(n, K, wi, y)) return;
-    const int r = y + n;
-#ifdef TL_DEBUG
-    if (!(TL_IN(r, 2 * n, 503) && TL_IN(4 * wi + 3, S, 504))) return;
-#endif
-    const uint32_t bw = word_at(B, n, S, r, wi);
-    uint32_t outw = bw;
-    bool any = false;
+    const int lane = threadIdx.x & 31;
+    const int RW = 4 * Kw;
+    const int p = (Y + K + 1) & 1;
+    uint32_t A = 0, B = 0, N = 0, S = 0, fill = 0;
+    if (live) {
+        const uint32_t* V = src + (2 + p) * Kw + k;
+        A = src[k];
+        const uint32_t ho = src[Kw + k];
+        const bool in = p ? k + 1 < Kw : k > 0;
+        const uint32_t adj = in ? src[Kw + k + (p ? 1 : -1)] : 0u;
+        B = p ? (ho >> 1) | (adj << 31) : (ho << 1) | (adj >> 31);
+        N = V[0];
+        S = V[-RW];
+        const int w = K - 1 - (Y > n ? Y - n : n - Y);
+        fill = ~(A | B | N | S) & range_mask(k, (n - w - p) >> 1, (n + w - p) >> 1);
+    }
+    uint32_t hor = 0;
+    if (__any_sync(0xFFFFFFFFu, fill != 0u)) {
+        // counter word 0 of bit 0 of this lane's word: (Y - 1) << 16 | (X - 1)
+        const uint32_t base = ((uint32_t)(Y - 1) << 16) + (uint32_t)(64 * k + p - 1);
+        const int cnt = __popc(fill);
+        int off = cnt;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) any |= byte_of(bw, i) == SH_EMPTY && in_diamond(4 * wi + i - n, y, K);
-    if (any) {
-        const DevRng rng = *rngp;
-        uint8_t cw[3][6];
-        load_window(B, n, S, r, wi, cw);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int x = 4 * wi + i - n;
-            if (cw[1][1 + i] != SH_EMPTY || !in_diamond(x, y, K)) continue;
-            // The block holding this cell has its lower-left corner at (x, y)
-            // or (x - 1, y - 1) if x + y + K is odd, else at (x - 1, y) or
-            // (x, y - 1).  When only one of the two has its other three cells
-            // empty, that is the block; otherwise the parity of the run of
-            // empty cells below this one in its column decides.
-            auto hole = [&](int dx, int dy) {
-                return in_diamond(x + dx, y + dy, K) && cw[1 + dy][1 + i + dx] == SH_EMPTY;
-            };
-            const bool odd = ((x + y + K) & 1) == 1;
-            const bool h1 = odd ? hole(1, 0) && hole(0, 1) && hole(1, 1) : hole(-1, 0) && hole(-1, 1) && hole(0, 1);
-            const bool h2 = odd ? hole(-1, 0) && hole(0, -1) && hole(-1, -1) : hole(0, -1) && hole(1, -1) && hole(1, 0);
-            int bx, by;
-            if (h1 != h2) {
-                bx = odd ? (h1 ? x : x - 1) : (h1 ? x - 1 : x);
-                by = h1 ? y : y - 1;
-            } else {
-                int below = 0;
-                for (int yy = y - 1; yy >= -K && in_diamond(x, yy, K) && cell_at(B, n, S, x, yy) == SH_EMPTY; --yy)
-                    ++below;
-                by = (below & 1) ? y - 1 : y;
-                bx = ((x + by + K) & 1) ? x : x - 1;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xFFFFFFFFu, off, o);
+            if (lane >= o) off += v;
+        }
+        const int total = __shfl_sync(0xFFFFFFFFu, off, 31);
+        off -= cnt;
+        sc.coin[lane] = 0u;
+        for (uint32_t m = fill; m; m &= m - 1) sc.list[off++] = (uint16_t)((lane << 5) | (__ffs(m) - 1));
+        __syncwarp();
+        for (int i0 = 0; i0 < total; i0 += 64) {
+            // two draws a lane in flight
+            const int ia = i0 + lane, ib = ia + 32;
+            const uint32_t ea = ia < total ? sc.list[ia] : 0u, eb = ib < total ? sc.list[ib] : 0u;
+            const uint32_t ca = __shfl_sync(0xFFFFFFFFu, base, ea >> 5) + 2u * (ea & 31u);
+            if (i0 + 32 < total) {
+                const uint32_t cb = __shfl_sync(0xFFFFFFFFu, base, eb >> 5) + 2u * (eb & 31u);
+                const bool ha = draw.horizontal(ca), hb = draw.horizontal(cb);
+                if (ha) atomicOr(&sc.coin[ea >> 5], 1u << (ea & 31u));
+                if (hb && ib < total) atomicOr(&sc.coin[eb >> 5], 1u << (eb & 31u));
+            } else if (draw.horizontal(ca) && ia < total) {
+                atomicOr(&sc.coin[ea >> 5], 1u << (ea & 31u));
             }
-            if (x == bx && y == by && (x + 1 >= n || y + 1 >= n || !hole(1, 0) || !hole(0, 1) || !hole(1, 1)))
-                atomicExch(status, 1);   // not a 2x2 hole: cannot happen for a valid tiling
-            const uint4 o = philox10(((uint32_t)(by + n) << 16) | (uint32_t)(bx + n), (uint32_t)K, 0xFFFE0000u,
-                                     rng.stream, rng.k0, rng.k1);
-            const uint8_t v = o.x < tbar ? (x > bx ? SH_HR : SH_HL) : (y > by ? SH_VT : SH_VB);
-            outw = (outw & ~(0xFFu << (8 * i))) | ((uint32_t)v << (8 * i));
         }
+        __syncwarp();
+        hor = sc.coin[lane];
+        __syncwarp();
     }
-    reinterpret_cast<uint32_t*>(C + (size_t)r * S)[wi] = outw;
+    if (live) {
+        const uint32_t ver = fill & ~hor;
+        uint32_t* V = dst + (2 + p) * Kw + k;
+        dst[k] = (B & ~A) | ver;
+        dst[Kw + k] = (A & ~B) | ver;
+        V[0] = (S & ~N) | hor;
+        V[-RW] = (N & ~S) | hor;
+    }
 }
 
-// Canonical domino state of the order-n diamond (box (2n+1)^2, zeroed):
-// a horizontal domino crosses the vertical edge between its cells, a
-// vertical one the horizontal edge.
-__global__ void shuffle_canon_kernel(const uint8_t* __restrict__ A, int n, uint8_t* __restrict__ canon)
+// The odd plane of row Y after step K, moved back if the row's class had p = 0.
+TL_DEV uint32_t sh_plain_odd(const uint32_t* row, int Kw, int Y, int K, int k)
 {
-    const int S = 2 * n, W = 2 * n + 1, P = cell_pitch(n);
-    const int64_t total = (int64_t)S * S;
+    const uint32_t o = row[Kw + k];
+    if ((Y + K + 1) & 1) return o;
+    return (o >> 1) | ((k + 1 < Kw ? row[Kw + k + 1] : 0u) << 31);
+}
+
+// Steps K0 .. K1 in one cooperative launch: every CTA keeps a stripe of rows
+// and h rows on each side in shared memory (two copies, alternating by step),
+// runs h steps while the exact region shrinks by one row per step and side,
+// then swaps boundary rows with its neighbours (64-bit words: cycle tag,
+// data).  Stripes the diamond has not reached yet do nothing, and a seam
+// starts its exchanges a few rows before the diamond arrives.
+//
+// Bound: the draws (about K^2 / 6 Philox calls in step K) in the middle
+// stripes, and below order 500 the latency of a step (a dependent read, list,
+// draw and write per word, one barrier).
+__global__ void __launch_bounds__(kShufThreads, 1) shuffle_kernel(const ShufParams P)
+{
+    extern __shared__ uint4 smem4[];
+    __shared__ ShufScratch s_scr[kShufWarps];
+    const int n = P.n, Kw = P.Kw, RW = 4 * Kw, h = P.h;
+    const int c = blockIdx.x, C = gridDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int lo = P.stripe_lo[c], hi = P.stripe_lo[c + 1];
+    const bool bot = c == 0, top = c == C - 1;
+    const int slo = bot ? lo : lo - h, shi = top ? hi : hi + h;
+    const int nloc = shi - slo;
+    uint32_t* const buf0 = reinterpret_cast<uint32_t*>(smem4);
+    const int bwords = nloc * RW;
+    {
+        // rows of the diamond so far into the first copy; the second is
+        // written before it is read, except where the diamond has not been
+        const uint4* g = reinterpret_cast<const uint4*>(P.rows0 + (int64_t)slo * RW);
+        for (int i = tid; i < bwords / 4; i += kShufThreads) {
+            smem4[i] = P.K0 > 1 ? __ldcg(g + i) : make_uint4(0u, 0u, 0u, 0u);
+            smem4[bwords / 4 + i] = make_uint4(0u, 0u, 0u, 0u);
+        }
+    }
+    __syncthreads();
+    int cur = 0;
+    const size_t side_words = (size_t)h * RW;
+    for (int Kc = P.K0;; Kc += h) {
+        const int hc = P.K1 - Kc + 1 < h ? P.K1 - Kc + 1 : h;
+        for (int i = 1; i <= hc; ++i) {
+            const int K = Kc + i - 1;
+            // rows whose inputs are exact and that the order-K diamond reaches
+            const int ya = bot ? slo + 1 : slo + i, yb = top ? shi : shi - (i - 1);
+            const int r0 = ya > n - K + 1 ? ya : n - K + 1, r1 = yb < n + K ? yb : n + K;
+            if (r1 <= r0) continue;
+            const int dmin = r0 > n ? r0 - n : (r1 <= n ? n - (r1 - 1) : 0);
+            int klo, khi;
+            sh_words(n, K, dmin, klo, khi);
+            const uint32_t nw = (uint32_t)(khi - klo + 1), total = (uint32_t)(r1 - r0) * nw;
+            // t / nw: exact, since t < 2^20 keeps the rounding below half of 1 / nw
+            const float inv = __frcp_rn((float)nw);
+            const uint32_t* src = buf0 + cur * bwords;
+            uint32_t* dst = buf0 + (cur ^ 1) * bwords;
+            const ShufDraw draw((uint32_t)K, P.rng);
+            // the same number of words for every warp and turn: fewer than 32
+            // spread a small step's draws over more warps
+            const uint32_t turns = (total + kShufThreads - 1) / kShufThreads;
+            uint32_t per = turns <= 1u ? (total + kShufWarps - 1) / kShufWarps
+                                       : (uint32_t)__float2int_ru(__fdividef((float)total, (float)(turns * kShufWarps)));
+            per = per < 4u ? 4u : (per > 32u ? 32u : per);
+            for (uint32_t t0 = (uint32_t)warp * per; t0 < total; t0 += per * kShufWarps) {
+                const uint32_t t = t0 + (uint32_t)lane;
+                const uint32_t rr = (uint32_t)(((float)t + 0.5f) * inv);
+                const int Y = r0 + (int)rr, k = klo + (int)(t - rr * nw);
+                bool live = t < total && (uint32_t)lane < per;
+#ifdef TL_DEBUG
+                // rows Y - 1 and Y are local, word k lies in a plane row
+                if (live && !(TL_IN(Y - 1 - slo, nloc, 501) && TL_IN(Y - slo, nloc, 501) && TL_IN(k, Kw, 502)))
+                    live = false;
+#endif
+                sh_step_words(src + (Y - slo) * RW, dst + (Y - slo) * RW, Kw, n, K, Y, k, live, draw,
+                              s_scr[warp]);
+            }
+            cur ^= 1;
+            __syncthreads();
+        }
+        const int K = Kc + hc - 1;
+        if (K >= P.K1) break;
+        // ---- exchange with the stripes below and above, where the diamond is
+        // within reach of the seam (both sides decide alike) ----
+        const int reach = K + 2 * h + 2;
+        const bool xb = !bot && lo - n <= reach && n - lo <= reach, xt = !top && hi - n <= reach && n - hi <= reach;
+        if (!xb && !xt) continue;
+        // the order of the rows names the exchange (never 0, increasing over
+        // the launches of a sample); the copy alternates within a launch
+        const unsigned long long tag = (unsigned long long)(uint32_t)K << 32;
+        const int par = ((Kc - P.K0) / h) & 1;
+        // words that can be non-zero after step K, in pairs
+        const int e0 = (n - K) >> 1, e1 = ((n + K) >> 1) + 1;
+        const int xk0 = ((e0 > 0 ? e0 - 1 : 0) >> 5) & ~1;
+        const int xk1 = ((e1 >> 5) < Kw ? (e1 >> 5) : Kw - 1) | 1;
+        const int npw = (xk1 - xk0 + 1) >> 1, units = 4 * h * npw;
+        uint32_t* const st = buf0 + cur * bwords;
+        unsigned long long* const mine = P.xbuf + ((size_t)c * 2 + par) * 2 * side_words;
+        for (int u = tid; u < 2 * units; u += kShufThreads) {
+            const int s = u >= units, v = u - (s ? units : 0);
+            if (!(s ? xt : xb)) continue;
+            const int rp = v / npw, wd = rp * Kw + xk0 + 2 * (v - rp * npw);   // (row, plane) block, word pair
+#ifdef TL_DEBUG
+            if (!TL_IN(wd + 1, (int64_t)side_words, 503)) continue;
+#endif
+            const uint32_t* a = st + ((s ? hi - h : lo) - slo) * RW + wd;
+            sh_st2(mine + (size_t)s * side_words + wd, tag | a[0], tag | a[1]);
+        }
+        int ok = 1;
+        const uint64_t t_wait = sh_globaltimer();
+        for (int u = tid; u < 2 * units && ok; u += kShufThreads) {
+            const int s = u >= units, v = u - (s ? units : 0);
+            if (!(s ? xt : xb)) continue;
+            const int rp = v / npw, wd = rp * Kw + xk0 + 2 * (v - rp * npw);
+#ifdef TL_DEBUG
+            if (!TL_IN(wd + 1, (int64_t)side_words, 504)) continue;
+#endif
+            // the neighbour below publishes its upper rows as side 1, the one above its lower rows as side 0
+            const unsigned long long* from =
+                P.xbuf + (((size_t)(s ? c + 1 : c - 1) * 2 + par) * 2 + (s ? 0 : 1)) * side_words + wd;
+            unsigned long long a, b;
+            for (;;) {
+                sh_ld2(from, &a, &b);
+                if ((a >> 32) == (tag >> 32) && (b >> 32) == (tag >> 32)) break;
+                if (*(volatile int*)P.status || sh_globaltimer() - t_wait > kShufWaitLimitNs) {
+                    atomicExch(P.status, 1);
+                    ok = 0;
+                    break;
+                }
+                __nanosleep(32);
+            }
+            uint32_t* d = st + ((s ? hi : lo - h) - slo) * RW + wd;
+            d[0] = (uint32_t)a;
+            d[1] = (uint32_t)b;
+        }
+        if (tid == 0 && *(volatile int*)P.status) ok = 0;
+        if (!__syncthreads_and(ok)) return;   // the host reports the timeout
+    }
+    const uint32_t* st = buf0 + cur * bwords;
+    for (int i = tid; i < (hi - lo) * RW; i += kShufThreads) {
+        const int rr = i / RW, rem = i - rr * RW, pl = rem / Kw, k = rem - pl * Kw;
+        const uint32_t* row = st + (lo + rr - slo) * RW;
+        P.rows0[(int64_t)lo * RW + i] = pl == 1 && P.K1 == n ? sh_plain_odd(row, Kw, lo + rr, n, k) : row[rem];
+    }
+}
+
+// One step with the rows in global memory (diamonds whose stripes do not fit
+// the SMs' shared memory): A is read, B written, both with a pad row below row
+// 0 and zero wherever the diamond has not been.
+__global__ void __launch_bounds__(kShufThreads) shuffle_step_kernel(const uint32_t* __restrict__ A,
+                                                                    uint32_t* __restrict__ B, int n, int Kw, int K,
+                                                                    DevRng rng)
+{
+    __shared__ ShufScratch s_scr[kShufWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t RW = 4 * (int64_t)Kw;
+    const int d = (int)blockIdx.y < K ? K - 1 - (int)blockIdx.y : (int)blockIdx.y - (K - 1);
+    const int Y = n - (K - 1) + (int)blockIdx.y;
+    int klo, khi;
+    sh_words(n, K, d, klo, khi);
+    const ShufDraw draw((uint32_t)K, rng);
+    for (int k0 = klo + (int)(blockIdx.x * kShufWarps + warp) * 32; k0 <= khi; k0 += (int)gridDim.x * kShufThreads) {
+        bool live = k0 + lane <= khi;
+#ifdef TL_DEBUG
+        if (live && !(TL_IN(Y, 2 * n + 1, 505) && TL_IN(k0 + lane, Kw, 506))) live = false;
+#endif
+        sh_step_words(A + (int64_t)Y * RW, B + (int64_t)Y * RW, Kw, n, K, Y, k0 + lane, live, draw, s_scr[warp]);
+    }
+}
+
+// The odd planes of B after the last step, moved back, into A (whose other
+// planes are copied).
+__global__ void shuffle_plain_kernel(const uint32_t* __restrict__ B, uint32_t* __restrict__ A, int n, int Kw)
+{
+    const int64_t RW = 4 * (int64_t)Kw, total = (2 * (int64_t)n + 1) * RW;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        const int cx = (int)(i % S), cy = (int)(i / S);   // cell (cx - n, cy - n)
-        const uint8_t v = A[(size_t)cy * P + cx];
-        if (v == SH_HL) canon[(size_t)W * W + (size_t)cy * W + cx + 1] = 1;    // Vt(x+1, y)
-        else if (v == SH_VB) canon[(size_t)(cy + 1) * W + cx] = 1;            // Hz(x, y+1)
+        const int Y = (int)(i / RW), rem = (int)(i - Y * RW), pl = rem / Kw, k = rem - pl * Kw;
+        A[i] = pl == 1 ? sh_plain_odd(B + Y * RW, Kw, Y, n, k) : B[i];
     }
 }
 
 static inline cudaStream_t SS_(void* s) { return reinterpret_cast<cudaStream_t>(s); }
 
-static int grid_for_cells(int64_t n)
+size_t shuffle_smem_bytes(int nloc, int Kw) { return (size_t)nloc * 4 * Kw * 4 * 2; }
+
+int shuffle_prepare_kernel(size_t smem_bytes, int* blocks_per_sm)
 {
-    const int64_t b = (n + 255) / 256;
-    return (int)(b < 4096 ? (b > 0 ? b : 1) : 4096);
+    *blocks_per_sm = 0;
+    cudaError_t e =
+        cudaFuncSetAttribute(shuffle_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, shuffle_kernel, kShufThreads, smem_bytes);
+    if (e != cudaSuccess) cudaGetLastError();
+    return (int)e;
 }
 
-// A, B, F: three zeroed buffers of 2n rows of (2n rounded up to 4) bytes;
-// rng: device copy of the key.  Enqueues 2n + 1 kernels (also under stream
-// capture).
-int launch_shuffle(int n, uint8_t* A, uint8_t* B, uint8_t* F, const DevRng* rng, int* status, uint8_t* canon,
-                   void* stream)
+size_t shuffle_static_smem() { return sizeof(ShufScratch) * kShufWarps; }
+
+int launch_shuffle(const ShufflePlan* seg, int nseg, int n, int Kw, size_t total_words, size_t xbuf_words,
+                   uint32_t* rows, const DevRng& rng, void* stream)
+{
+    cudaError_t e = cudaMemsetAsync(seg[0].xbuf, 0, xbuf_words * sizeof(unsigned long long), SS_(stream));
+    // rows the first launches do not cover
+    if (e == cudaSuccess) e = cudaMemsetAsync(rows, 0, total_words * 4, SS_(stream));
+    for (int i = 0; i < nseg && e == cudaSuccess; ++i) {
+        ShufParams P;
+        P.n = n;
+        P.Kw = Kw;
+        P.h = seg[i].halo;
+        P.K0 = i ? seg[i - 1].last + 1 : 1;
+        P.K1 = seg[i].last;
+        P.stripe_lo = seg[i].stripe_lo;
+        P.rng = rng;
+        P.xbuf = seg[i].xbuf;
+        P.rows0 = rows + 4 * (size_t)Kw;
+        P.status = seg[i].status;
+        void* args[] = {&P};
+        e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(&shuffle_kernel), dim3(seg[i].ctas),
+                                        dim3(kShufThreads), args, seg[i].smem_bytes, SS_(stream));
+    }
+    return (int)e;
+}
+
+int launch_shuffle_global(int n, int Kw, size_t total_words, uint32_t* A, uint32_t* B, const DevRng& rng, void* stream)
 {
     const cudaStream_t s = SS_(stream);
-    uint8_t *cur = A, *mid = B, *spare = F;
-    const uint32_t tbar = 0x80000000u;   // uniform: horizontal and vertical pairs equally likely
-    for (int k = 0; k < n; ++k) {
-        const int K = k + 1;
-        const int words = ((2 * K + 8) >> 2) + 1;   // words of the widest row, with both ragged ends
-        const dim3 grid((words + 127) / 128, 2 * K);   // x over a row's words, one block row per cell row
-        shuffle_move_kernel<<<grid, 128, 0, s>>>(cur, mid, n, k);
-        shuffle_fill_kernel<<<grid, 128, 0, s>>>(mid, spare, n, K, rng, tbar, status);
-        uint8_t* t = cur;
-        cur = spare;
-        spare = t;
+    cudaError_t e = cudaMemsetAsync(A, 0, total_words * 4, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(B, 0, total_words * 4, s);
+    if (e != cudaSuccess) return (int)e;
+    uint32_t *src = A + 4 * (size_t)Kw, *dst = B + 4 * (size_t)Kw;   // row 0, after the pad row
+    for (int K = 1; K <= n; ++K) {
+        const int words = ((2 * K) >> 6) + 2;   // of the widest row, with both ragged ends
+        const dim3 grid((words + kShufThreads - 1) / kShufThreads, 2 * K - 1);
+        shuffle_step_kernel<<<grid, kShufThreads, 0, s>>>(src, dst, n, Kw, K, rng);
+        uint32_t* t = src;
+        src = dst;
+        dst = t;
     }
-    shuffle_canon_kernel<<<grid_for_cells((int64_t)4 * n * n), 256, 0, s>>>(cur, n, canon);
+    // src holds the sample; the plain planes go to A
+    shuffle_plain_kernel<<<2048, 256, 0, s>>>(src, dst, n, Kw);
+    if (dst != A + 4 * (size_t)Kw) {
+        e = cudaMemcpyAsync(A, B, total_words * 4, cudaMemcpyDeviceToDevice, s);
+        if (e != cudaSuccess) return (int)e;
+    }
     return (int)cudaGetLastError();
 }
 
