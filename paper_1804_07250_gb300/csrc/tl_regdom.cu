@@ -459,6 +459,10 @@ __global__ void __launch_bounds__(NT, 1) regdom_kernel(const RegParams P)
         // zeros (cleared before every launch): a tag of cyc mod 4, plus one,
         // tells them apart
         const unsigned long long tag = (unsigned long long)((cyc & 3) + 1) << 61;
+        // a status word raised anywhere (a wait that gave up in another CTA,
+        // or raised by the host) ends every CTA at its next exchange: read
+        // here, used at the end, so that its latency hides behind the exchange
+        const int raised = tid == 0 ? *(volatile int*)P.status : 0;
         if (owned) {
             uint32_t w[32];
             {
@@ -516,18 +520,24 @@ __global__ void __launch_bounds__(NT, 1) regdom_kernel(const RegParams P)
                 for (int q = 0; q < kXUnits; ++q) rd_ld2(src + ((size_t)q * Kg + m) * 2, &f[2 * q], &f[2 * q + 1]);
             oA0 = philox10(grp0, sweep, 0u, P.rng.stream, P.rng.k0, P.rng.k1);
             oA1 = philox10(grp1, sweep, 0u, P.rng.stream, P.rng.k0, P.rng.k1);
-            const uint64_t t_wait = rd_globaltimer();
+            uint64_t t_wait = 0;
             unsigned need = (1u << kXUnits) - 1;
-            while (true) {
+            for (unsigned spin = 1;; ++spin) {
 #pragma unroll
                 for (int q = 0; q < kXUnits; ++q)
                     if ((need >> q & 1u) && (f[2 * q] & ~kXMask) == tag && (f[2 * q + 1] & ~kXMask) == tag)
                         need &= ~(1u << q);
                 if (!need) break;
-                if (*(volatile int*)P.status || rd_globaltimer() - t_wait > kRegWaitLimitNs) {
-                    atomicExch(P.status, 1);
-                    ok = 0;
-                    break;
+                // the limit and the status word are looked at every 16th
+                // round: their reads take as long as the poll's own
+                if ((spin & 15u) == 0u) {
+                    const uint64_t now = rd_globaltimer();
+                    if (!t_wait) t_wait = now;
+                    if (*(volatile int*)P.status || now - t_wait > kRegWaitLimitNs) {
+                        atomicExch(P.status, 1);
+                        ok = 0;
+                        break;
+                    }
                 }
                 __nanosleep(32);
 #pragma unroll
@@ -550,9 +560,7 @@ __global__ void __launch_bounds__(NT, 1) regdom_kernel(const RegParams P)
             RV[2 * tid + 1] = Vo1;
             RH[tid] = make_uint2(Ho0.w, Ho1.w);
         }
-        // a status word raised anywhere (a wait that gave up in another CTA,
-        // or raised by the host) ends every CTA at its next exchange
-        if (tid == 0 && *(volatile int*)P.status) ok = 0;
+        if (raised) ok = 0;
         if (!__syncthreads_and(ok)) return;   // the state is undefined; the host reports TL_ETIMEOUT
         if (act) {
             if (ib >= 0) {

@@ -276,6 +276,7 @@ __global__ void __launch_bounds__(kShufThreads, 1) shuffle_kernel(const ShufPara
         // the order of the rows names the exchange (never 0, increasing over
         // the launches of a sample); the copy alternates within a launch
         const unsigned long long tag = (unsigned long long)(uint32_t)K << 32;
+        const int raised = tid == 0 ? *(volatile int*)P.status : 0;   // used at the end of the exchange
         const int par = ((Kc - P.K0) / h) & 1;
         // words that can be non-zero after step K, in pairs
         const int e0 = (n - K) >> 1, e1 = ((n + K) >> 1) + 1;
@@ -295,7 +296,7 @@ __global__ void __launch_bounds__(kShufThreads, 1) shuffle_kernel(const ShufPara
             sh_st2(mine + (size_t)s * side_words + wd, tag | a[0], tag | a[1]);
         }
         int ok = 1;
-        const uint64_t t_wait = sh_globaltimer();
+        uint64_t t_wait = 0;
         for (int u = tid; u < 2 * units && ok; u += kShufThreads) {
             const int s = u >= units, v = u - (s ? units : 0);
             if (!(s ? xt : xb)) continue;
@@ -307,13 +308,19 @@ __global__ void __launch_bounds__(kShufThreads, 1) shuffle_kernel(const ShufPara
             const unsigned long long* from =
                 P.xbuf + (((size_t)(s ? c + 1 : c - 1) * 2 + par) * 2 + (s ? 0 : 1)) * side_words + wd;
             unsigned long long a, b;
-            for (;;) {
+            for (unsigned spin = 1;; ++spin) {
                 sh_ld2(from, &a, &b);
                 if ((a >> 32) == (tag >> 32) && (b >> 32) == (tag >> 32)) break;
-                if (*(volatile int*)P.status || sh_globaltimer() - t_wait > kShufWaitLimitNs) {
-                    atomicExch(P.status, 1);
-                    ok = 0;
-                    break;
+                // the limit and the status word are looked at every 16th
+                // round: their reads take as long as the poll's own
+                if ((spin & 15u) == 0u) {
+                    const uint64_t now = sh_globaltimer();
+                    if (!t_wait) t_wait = now;
+                    if (*(volatile int*)P.status || now - t_wait > kShufWaitLimitNs) {
+                        atomicExch(P.status, 1);
+                        ok = 0;
+                        break;
+                    }
                 }
                 __nanosleep(32);
             }
@@ -321,7 +328,7 @@ __global__ void __launch_bounds__(kShufThreads, 1) shuffle_kernel(const ShufPara
             d[0] = (uint32_t)a;
             d[1] = (uint32_t)b;
         }
-        if (tid == 0 && *(volatile int*)P.status) ok = 0;
+        if (raised) ok = 0;
         if (!__syncthreads_and(ok)) return;   // the host reports the timeout
     }
     const uint32_t* st = buf0 + cur * bwords;
