@@ -1230,6 +1230,7 @@ TL_API uint64_t tl_chain_sweep(const tl_chain* c) { return c ? c->sweep : 0; }
 TL_API uint64_t tl_chain_launches(const tl_chain* c) { return c ? c->launches : 0; }
 
 static bool want_resident(tl_chain* c);
+static void free_resident(tl_chain* c);
 
 TL_API int tl_chain_set_plan(tl_chain* c, const tl_plan* p)
 {
@@ -1242,14 +1243,7 @@ TL_API int tl_chain_set_plan(tl_chain* c, const tl_plan* p)
     c->spl = p->sweeps_per_launch;
     if (p->halo != c->halo_req || p->threads != c->threads_req || p->npre != c->npre_req || kernel_changed) {
         CUDA_TRY(cudaDeviceSynchronize());
-        cudaFree(c->stripe_d);
-        cudaFree(c->xbuf_d);
-        cudaFree(c->status_d);
-        cudaFree(c->hull_d);
-        c->stripe_d = nullptr;
-        c->xbuf_d = nullptr;
-        c->status_d = nullptr;
-        c->hull_d = nullptr;
+        free_resident(c);
         c->use_reg = false;
         c->res_ready = c->res_failed = false;
         c->halo_req = p->halo;
@@ -1345,31 +1339,11 @@ static int take_sample(tl_chain* c, void* stream)
     return TL_OK;
 }
 
-// Default halo depth (passes per exchange), threads per CTA and random
-// planes generated ahead for the resident kernel.
-// Dominoes at t = 2^31 take the single-plane update when it fits.
+// Dominoes at t = 2^31 take the single-plane updates when they fit.
 static bool fast_candidate(const tl_chain* c)
 {
     return c->g.lattice == LAT_DOMINO && c->th.kind == THR_SCALAR && c->th.scalar == 0x80000000u &&
            c->npre_req <= 1;
-}
-
-// Defaults measured on the Aztec diamond of order 2048, the hexagon 1024^3
-// and the domain-wall square 2048: the single-plane domino update runs
-// fastest with 1024 threads and 6 passes per exchange, the others with 512
-// threads and 8 (dominoes, six-vertex) or 6 (lozenges) passes.
-static int default_halo(const tl_chain* c)
-{
-    if (fast_candidate(c)) return 6;
-    return c->g.lattice == LAT_LOZENGE ? 6 : 8;
-}
-static int default_threads(const tl_chain* c) { return fast_candidate(c) ? 1024 : 512; }
-static int default_npre(const tl_chain* c)
-{
-    if (c->th.kind == THR_SCALAR) return c->th.kmax < 0 ? 1 : std::min(8, c->th.kmax + 1);
-    // six-vertex tables (DWBC 2048 at c = sqrt 2: 12 planes 7.70 us/sweep
-    // against 7.87 with 8 and 8.60 with 16); per-site thresholds: 8
-    return c->g.lattice == LAT_SIXV ? 12 : 8;
 }
 
 // Groups one pass of the single-plane domino update can hold: each of the
@@ -1577,137 +1551,237 @@ static int plan_regdom(tl_chain* c)
     return TL_OK;
 }
 
-// Stripe partition, shared-memory budget and buffers of the resident kernel.
+// Device buffers of a resident plan with stripe bounds `lo` (C + 1).
+static int alloc_resident(tl_chain* c, const std::vector<int>& lo, int h)
+{
+    const Geom& g = c->g;
+    const int C = (int)lo.size() - 1;
+    int rc;
+    if ((rc = dev_alloc(&c->stripe_d, (size_t)C + 1, "stripes")) ||
+        (rc = dev_alloc(&c->xbuf_d, (size_t)C * 4 * h * g.row_words, "exchange buffer")) ||
+        (rc = dev_alloc(&c->status_d, 1, "status")))
+        return rc;
+    CUDA_TRY(cudaMemcpy(c->stripe_d, lo.data(), sizeof(int) * (C + 1), cudaMemcpyHostToDevice));
+    CUDA_TRY(cudaMemset(c->xbuf_d, 0, sizeof(unsigned long long) * C * 4 * h * g.row_words));
+    CUDA_TRY(cudaMemset(c->status_d, 0, sizeof(int)));
+    c->res.ctas = C;
+    c->res.halo = h;
+    c->res.stripe_lo = c->stripe_d;
+    c->res.xbuf = c->xbuf_d;
+    c->res.status = c->status_d;
+    c->res_ready = true;
+    return TL_OK;
+}
+
+// Row bounds of C stripes of at least h rows each with equal shares of the
+// weights (prefix sums `pre`, one more than rows); bounds are rounded up to
+// multiples of `step` where that keeps h rows.
+static std::vector<int> even_stripes(const std::vector<double>& pre, int C, int h, int step)
+{
+    const int H = (int)pre.size() - 1;
+    std::vector<int> lo(C + 1, 0);
+    int y = 0;
+    for (int k = 1; k < C; ++k) {
+        const double target = pre[H] * k / C;
+        const int ymin = lo[k - 1] + h, ymax = H - h * (C - k);
+        while (y < H && pre[y] < target) ++y;
+        int v = std::min(std::max(y, ymin), ymax);
+        if (v % step && v + step - v % step <= ymax) v += step - v % step;
+        lo[k] = v;
+    }
+    lo[C] = H;
+    return lo;
+}
+
+// Dominoes at t = 2^31 on the shared-memory kernel with the single-plane
+// update: 1024 threads and 6 passes per exchange run fastest on the Aztec
+// diamond of order 2048.
+static int plan_fast(tl_chain* c)
+{
+    const Geom& g = c->g;
+    const tl_domain& d = c->dom_copy;
+    const int h = c->halo_req > 0 ? c->halo_req : 6;
+    const int threads = c->threads_req > 0 ? c->threads_req : 1024;
+    std::vector<int> pre(g.H + 1, 0);
+    std::vector<double> w(g.H + 1, 0.0);
+    for (int y = 0; y < g.H; ++y) {
+        const int act = std::max(0, d.grange[y].y - d.grange[y].x);
+        pre[y + 1] = pre[y] + act;
+        w[y + 1] = w[y] + 0.1 + act;
+    }
+    auto items_in = [&](int a, int b) {
+        a = std::max(a, 0);
+        b = std::min(b, g.H);
+        return b <= a ? 0 : pre[b] - pre[a];
+    };
+    const int C = std::min(c->ctx->sms, g.H / h);
+    if (C < 2) {
+        c->res_why = "domain too small for stripes";
+        return TL_EUNSUPPORTED;
+    }
+    const std::vector<int> lo = even_stripes(w, C, h, 1);
+    int max_nloc = 0, cap_items = 0, cap_cycle = 0, max_pass = 0;
+    for (int k = 0; k < C; ++k) {
+        int slo, shi;
+        stripe_local(lo[k], lo[k + 1], k, C, h, g.H, &slo, &shi);
+        max_nloc = std::max(max_nloc, shi - slo);
+        cap_items = std::max(cap_items, items_in(slo, shi));
+        int cyc = 0;
+        for (int i = 1; i <= h; ++i) {
+            const int n = items_in(k == 0 ? 0 : slo + i, k == C - 1 ? g.H + 1 : shi - (i - 1));
+            cyc += n;
+            max_pass = std::max(max_pass, n);
+        }
+        cap_cycle = std::max(cap_cycle, cyc);
+    }
+    const size_t smem = (size_t)max_nloc * g.row_words * 4 + (size_t)cap_cycle * 16 + (size_t)cap_items * 12 +
+                        (size_t)(max_nloc + 1) * 4 + 24;
+    int bps = 0;
+    if (max_pass > fast_capacity(threads) || (long)smem > (long)c->ctx->smem_optin ||
+        resident_prepare(threads, smem, &bps) != 0 || bps < 1 || C > bps * c->ctx->sms) {
+        c->res_why = "a pass does not fit the single-plane update";
+        return TL_EUNSUPPORTED;
+    }
+    c->res = ResidentPlan{};
+    c->res.threads = threads;
+    c->res.slots = 1;
+    c->res.npre = 1;
+    c->res.cap_items = cap_items;
+    c->res.cap_cycle = cap_cycle;
+    c->res.fast = true;
+    c->res.smem_bytes = smem;
+    return alloc_resident(c, lo, h);
+}
+
+// The word kernel: stripes, passes per exchange, threads and words per thread.
+//
+// A pass is modelled as a fixed chain (update and barrier), a cost per
+// 128-site group of the CTA (owned, and half of the halo rows on average: they
+// fall out one by one), the exchange spread over the `halo` passes of a cycle
+// (none with one stripe), and what the builds of fewer registers cost:
+//   T = 1000 + 24 groups + 3500 / halo + 350 (over 512 threads) + 1500 (more
+//   than one word a thread) cycles,
+// fitted to the passes measured with halos of 2 to 12 on the hexagons 1024^3
+// and 301 x 467 x 214, the domain-wall squares 333 and 2048 and the Aztec
+// diamond 1333; the minimum is flat.
+static int plan_words(tl_chain* c)
+{
+    const Geom& g = c->g;
+    const tl_domain& d = c->dom_copy;
+    const bool sixv = g.lattice == LAT_SIXV;
+    // groups of every row; six-vertex items are pairs of face rows
+    const int step = sixv ? 2 : 1, U = (g.H + step - 1) / step;
+    std::vector<int> pre(U + 1, 0);
+    std::vector<double> w(g.H + 1, 0.0);
+    int maxact = 0;
+    for (int r = 0; r < U; ++r) {
+        int2 gr = d.grange[step * r];
+        if (sixv && 2 * r + 1 < g.H) {
+            const int2 b = d.grange[2 * r + 1];
+            if (gr.y <= gr.x) gr = b;
+            else if (b.y > b.x) gr = make_int2(std::min(gr.x, b.x), std::max(gr.y, b.y));
+        }
+        const int act = std::max(0, gr.y - gr.x);
+        pre[r + 1] = pre[r] + act;
+        maxact = std::max(maxact, act);
+        for (int y = step * r; y < std::min(g.H, step * r + step); ++y) w[y + 1] = w[y] + 0.1 + act;
+    }
+    auto items_in = [&](int slo, int shi) {
+        const int a = std::max(slo, 0) / step, b = (std::min(shi, g.H) + step - 1) / step;
+        return b <= a ? 0 : pre[b] - pre[a];
+    };
+    if (c->kernel == 2 && std::min(c->ctx->sms, g.H / (c->halo_req > 0 ? c->halo_req : g.lattice == LAT_LOZENGE ? 6 : 8)) < 2) {
+        c->res_why = "domain too small for stripes";
+        return TL_EUNSUPPORTED;
+    }
+    struct Cand {
+        double t;
+        int h, C;
+    };
+    auto model = [](double own, double halo, int h) {
+        const double lanes = 4 * (own + 2 * halo);
+        return 1000 + 24 * (own + halo) + (h ? 3500.0 / h : 0) + (lanes > 512 ? 350 : 0) + (lanes > 1024 ? 1500 : 0);
+    };
+    std::vector<Cand> cand;
+    // whole sweeps per exchange (the pass loop is then unrolled)
+    const int hs[3][4] = {{4, 6, 8, 12}, {3, 6, 9, 12}, {4, 8, 12, 16}};
+    for (int hi = 0; hi < 4; ++hi) {
+        const int h = c->halo_req > 0 ? c->halo_req : hs[g.lattice][hi];
+        const int cmax = std::min(c->ctx->sms, g.H / h);
+        for (int C = 2; C <= cmax; C = C < 16 ? C + 1 : (C < cmax && C + C / 8 > cmax ? cmax : C + C / 8))
+            cand.push_back(Cand{model((double)pre[U] / C, (double)h * maxact / step, h), h, C});
+        if (c->halo_req > 0) break;
+    }
+    cand.push_back(Cand{model(pre[U], 0, 0), c->halo_req > 0 ? c->halo_req : 60, 1});
+    std::stable_sort(cand.begin(), cand.end(), [](const Cand& a, const Cand& b) { return a.t < b.t; });
+    c->res_why = "stripe does not fit in shared memory";
+    for (const Cand& cd : cand) {
+        const int h = cd.h, C = cd.C;
+        const std::vector<int> lo = even_stripes(w, C, h, step);
+        int max_nloc = 0, items = 0;
+        for (int k = 0; k < C; ++k) {
+            int slo, shi;
+            stripe_local(lo[k], lo[k + 1], k, C, h, g.H, &slo, &shi);
+            max_nloc = std::max(max_nloc, shi - slo);
+            items = std::max(items, items_in(slo, shi));
+        }
+        const int lanes = std::max(32, 4 * items);
+        const size_t smem = words_smem_bytes(g, max_nloc);
+        if (smem > (size_t)c->ctx->smem_optin || lanes > 4096) continue;
+        // `threads` asks for at most that many; results never depend on it
+        const int cap = c->threads_req == 512 && lanes <= 2048 ? 512 : 1024;
+        int slots = 1;
+        while (slots * cap < lanes) slots *= 2;
+        const int threads = ((lanes + slots - 1) / slots + 31) / 32 * 32;
+        int bps = 0;
+        if (words_prepare(g, c->th, threads, slots, smem, &bps) != 0 || bps < 1 || C > bps * c->ctx->sms) {
+            c->res_why = "resident kernel does not fit on an SM";
+            continue;
+        }
+        c->res = ResidentPlan{};
+        c->res.threads = threads;
+        c->res.slots = slots;
+        // six-vertex words carry 8 or 4 planes by their build
+        c->res.npre = sixv ? (slots <= 2 ? 8 : 4)
+                           : c->npre_req > 0 ? c->npre_req
+                                             : (c->th.kind == THR_SCALAR ? std::max(1, std::min(8, c->th.kmax + 1)) : 8);
+        c->res.smem_bytes = smem;
+        return alloc_resident(c, lo, h);
+    }
+    return TL_EUNSUPPORTED;
+}
+
+static void free_resident(tl_chain* c)
+{
+    cudaFree(c->stripe_d);
+    cudaFree(c->hull_d);
+    cudaFree(c->xbuf_d);
+    cudaFree(c->status_d);
+    c->stripe_d = nullptr;
+    c->hull_d = nullptr;
+    c->xbuf_d = nullptr;
+    c->status_d = nullptr;
+}
+
+// Plan of the chain's resident kernel: registers for dominoes at t = 2^31
+// where they fit, else shared memory.
 static int plan_resident(tl_chain* c)
 {
     if (c->kernel != 2 && fast_candidate(c) && c->g.Kg <= 4096) {
         const int rc = plan_regdom(c);
         if (rc == TL_OK) return TL_OK;
         if (c->kernel == 3) return rc;
-        cudaFree(c->stripe_d);
-        cudaFree(c->hull_d);
-        cudaFree(c->xbuf_d);
-        cudaFree(c->status_d);
-        c->stripe_d = nullptr;
-        c->hull_d = nullptr;
-        c->xbuf_d = nullptr;
-        c->status_d = nullptr;
+        free_resident(c);
     }
     if (c->kernel == 3) {
         c->res_why = "the register-resident kernel covers dominoes at t = 2^31 only";
         return TL_EUNSUPPORTED;
     }
-    const Geom& g = c->g;
-    const tl_domain& d = c->dom_copy;
-    const int h = c->halo_req > 0 ? c->halo_req : default_halo(c);
-    const int threads = c->threads_req > 0 ? c->threads_req : default_threads(c);
-    const int npre = c->npre_req > 0 ? c->npre_req : default_npre(c);
-    const bool sixv = g.lattice == LAT_SIXV;
-    std::vector<int> act(g.H, 0);
-    std::vector<double> w(g.H, 0.0);
-    double total = 0;
-    for (int y = 0; y < g.H; ++y) {
-        const int2 r = d.grange[y];
-        act[y] = std::max(0, r.y - r.x);
-        w[y] = 0.1 + act[y];
-        total += w[y];
+    if (fast_candidate(c)) {
+        if (plan_fast(c) == TL_OK) return TL_OK;
+        free_resident(c);
     }
-    // items of rows [a, b) (optionally one parity)
-    std::vector<int> pre(g.H + 1, 0), pre_par[2] = {std::vector<int>(g.H + 1, 0), std::vector<int>(g.H + 1, 0)};
-    for (int y = 0; y < g.H; ++y) {
-        pre[y + 1] = pre[y] + act[y];
-        for (int p = 0; p < 2; ++p) pre_par[p][y + 1] = pre_par[p][y] + ((y & 1) == p ? act[y] : 0);
-    }
-    auto items_in = [&](int a, int b, int par) {
-        a = std::max(a, 0);
-        b = std::min(b, g.H);
-        if (b <= a) return 0;
-        return par < 0 ? pre[b] - pre[a] : pre_par[par][b] - pre_par[par][a];
-    };
-    int C = std::min(c->ctx->sms, g.H / h);
-    if (C < 2) {
-        c->res_why = "domain too small for stripes";
-        return TL_EUNSUPPORTED;
-    }
-    const size_t row_bytes = (size_t)g.row_words * 4;
-    for (;;) {
-        std::vector<int> lo(C + 1, 0);
-        int y = 0;
-        double acc = 0;
-        for (int k = 1; k < C; ++k) {
-            const double target = total * k / C;
-            const int ymin = lo[k - 1] + h;
-            const int ymax = g.H - h * (C - k);
-            while (y < g.H && (acc < target || y < ymin)) acc += w[y++];
-            y = std::min(std::max(y, ymin), ymax);
-            acc = 0;
-            for (int t = 0; t < y; ++t) acc += w[t];
-            lo[k] = y;
-        }
-        lo[C] = g.H;
-        int max_nloc = 0, cap_items = 0, cap_cycle = 0, max_pass = 0;
-        for (int k = 0; k < C; ++k) {
-            int slo, shi;
-            stripe_local(lo[k], lo[k + 1], k, C, h, g.H, &slo, &shi);
-            max_nloc = std::max(max_nloc, shi - slo);
-            cap_items = std::max(cap_items, items_in(slo, shi, -1));
-            int cyc = 0;
-            for (int i = 1; i <= h; ++i) {
-                const int vlo = k == 0 ? -1 : slo + (i - 1);
-                const int vhi = k == C - 1 ? g.H + 1 : shi - (i - 1);
-                int n;
-                if (sixv) {
-                    const int a = std::max(vlo, 1), last = std::min(vhi - 2, g.N - 1);
-                    n = std::max(items_in(a, last + 1, 0), items_in(a, last + 1, 1));
-                } else {
-                    n = items_in(vlo + 1, vhi, -1);
-                }
-                cyc += n;
-                max_pass = std::max(max_pass, n);
-            }
-            cap_cycle = std::max(cap_cycle, cyc);
-        }
-        const int ntab = sixv ? 2 : 1;
-        const bool fast = g.lattice == LAT_DOMINO && c->th.kind == THR_SCALAR && c->th.scalar == 0x80000000u &&
-                          max_pass <= fast_capacity(threads) && c->npre_req <= 1;
-        size_t smem = (size_t)max_nloc * row_bytes + (size_t)npre * cap_cycle * 16 + (size_t)cap_items * 4 +
-                      (size_t)ntab * (max_nloc + 1) * 4 + 16;
-        if (fast) smem += (size_t)cap_items * 8 + 8;
-        if ((long)smem > (long)c->ctx->smem_optin) {
-            c->res_why = "stripe does not fit in shared memory";
-            return TL_EUNSUPPORTED;
-        }
-        int bps = 0;
-        if (resident_prepare(g, c->th.kind, threads, fast, smem, &bps) != 0 || bps < 1) {
-            c->res_why = "resident kernel does not fit on an SM";
-            return TL_EUNSUPPORTED;
-        }
-        if (C > bps * c->ctx->sms) {
-            C = bps * c->ctx->sms;
-            continue;
-        }
-        int rc;
-        if ((rc = dev_alloc(&c->stripe_d, (size_t)C + 1, "stripes")) ||
-            (rc = dev_alloc(&c->xbuf_d, (size_t)C * 4 * h * g.row_words, "exchange buffer")) ||
-            (rc = dev_alloc(&c->status_d, 1, "status")))
-            return rc;
-        CUDA_TRY(cudaMemcpy(c->stripe_d, lo.data(), sizeof(int) * (C + 1), cudaMemcpyHostToDevice));
-        CUDA_TRY(cudaMemset(c->xbuf_d, 0, sizeof(unsigned long long) * C * 4 * h * g.row_words));
-        CUDA_TRY(cudaMemset(c->status_d, 0, sizeof(int)));
-        c->res.ctas = C;
-        c->res.threads = threads;
-        c->res.halo = h;
-        c->res.npre = npre;
-        c->res.cap_items = cap_items;
-        c->res.cap_cycle = cap_cycle;
-        c->res.fast = fast;
-        c->res.smem_bytes = smem;
-        c->res.stripe_lo = c->stripe_d;
-        c->res.xbuf = c->xbuf_d;
-        c->res.status = c->status_d;
-        c->res_ready = true;
-        return TL_OK;
-    }
+    return plan_words(c);
 }
 
 static bool want_resident(tl_chain* c)
@@ -1765,10 +1839,15 @@ static int run_resident(tl_chain* c, uint64_t k, unsigned long long* ring, void*
                                 ring ? ring + done : nullptr, dens ? c->cplanes : nullptr, c->burn,
                                 dens ? c->stride : 0, c->random_order ? c->colours : nullptr,
                                 c->count_flips ? c->flips_d : nullptr, stream)
-                : launch_resident(c->g, c->rows, c->res, (uint32_t)c->sweep, (uint32_t)n, c->rng, c->th, c->grange,
+            : c->res.fast
+                ? launch_resident(c->g, c->rows, c->res, (uint32_t)c->sweep, (uint32_t)n, c->rng, c->grange,
                                   ++c->epoch, ring ? ring + done : nullptr, dens ? c->cplanes : nullptr, c->burn,
                                   dens ? c->stride : 0, c->random_order ? c->colours : nullptr,
-                                  c->count_flips ? c->flips_d : nullptr, stream);
+                                  c->count_flips ? c->flips_d : nullptr, stream)
+                : launch_words(c->g, c->rows, c->res, (uint32_t)c->sweep, (uint32_t)n, c->rng, c->th, c->grange,
+                               ++c->epoch, ring ? ring + done : nullptr, dens ? c->cplanes : nullptr, c->burn,
+                               dens ? c->stride : 0, c->random_order ? c->colours : nullptr,
+                               c->count_flips ? c->flips_d : nullptr, stream);
         if (e) return fail(TL_ECUDA, "resident kernel: %s", cudaGetErrorString((cudaError_t)e));
         if (dens) c->samples += samples_upto(c, c->sweep + n) - samples_upto(c, c->sweep);
         c->sweep += n;
@@ -1847,6 +1926,7 @@ TL_API int tl_debug_checks(int clear, uint64_t* failures, int* first_id, int64_t
 #ifdef TL_DEBUG
     CUDA_TRY(cudaDeviceSynchronize());
     int (*const fetch[])(unsigned long long*, bool) = {dbg_fetch_kernels, dbg_fetch_regdom, dbg_fetch_resident,
+                                                       dbg_fetch_words_domino, dbg_fetch_words_lozenge, dbg_fetch_words_sixv,
                                                        dbg_fetch_batch, dbg_fetch_shuffle};
     uint64_t n = 0;
     int id = 0;

@@ -115,38 +115,47 @@ int noalloc_prepare(int device);
 int launch_height_noalloc(const Geom& g, const uint32_t* rows, const int* seg, int nseg, int hw, int hh,
                           int32_t* out, int device, void* stream);
 
-// Resident multi-sweep kernel.  One cooperative launch runs `nsweeps`
+// Resident multi-sweep kernels.  One cooperative launch runs `nsweeps`
 // sweeps from absolute sweep `sweep0`.  CTA c owns the rows
 // [stripe_lo[c], stripe_lo[c+1]) and keeps them, plus `halo` rows on each
 // side, in shared memory for the whole launch.  Every `halo` passes the
 // CTAs publish their boundary rows and read their neighbours' (double
-// buffered, ordered by per-CTA progress flags); in between, the halo rows
-// are recomputed redundantly, the valid region shrinking by one row per pass.
+// buffered, tagged words); in between, the halo rows are recomputed
+// redundantly, the valid region shrinking by one row per pass.
 struct ResidentPlan {
     int ctas;                      // cooperative grid size
-    int threads;                   // threads per CTA (512 or 1024)
+    int threads;                   // threads per CTA
+    int slots;                     // words per thread (the word kernel)
     int halo;                      // passes per exchange cycle (= halo rows per side)
     int npre;                      // random planes generated ahead per group
-    int cap_items;                 // item-table capacity per CTA
-    int cap_cycle;                 // groups touched per cycle, per CTA (upper bound)
-    bool fast;                     // dominoes at t = 2^31: branch-free single-plane update
+    int cap_items;                 // `fast`: item-table capacity per CTA
+    int cap_cycle;                 // `fast`: groups touched per cycle, per CTA (upper bound)
+    bool fast;                     // dominoes at t = 2^31: branch-free single-plane update (tl_resident.cu)
     size_t smem_bytes;             // dynamic shared memory per CTA
     const int* stripe_lo;          // device [ctas + 1]
     unsigned long long* xbuf;      // device [ctas][2][2][halo][row_words] tagged words
     int* status;                   // device error word: 0 ok, 1 a bounded wait gave up
 };
 
-// Shared-memory attribute and occupancy for the resident kernel of this
-// lattice / threshold kind: blocks that fit on one SM (0 if none).
-int resident_prepare(const Geom& g, int thr_kind, int threads, bool fast, size_t smem_bytes, int* blocks_per_sm);
+// Shared-memory attribute and occupancy: blocks that fit on one SM (0 if none).
+int resident_prepare(int threads, size_t smem_bytes, int* blocks_per_sm);
 
 // ring: per-sweep hashes (nullptr = off; must be zeroed).  counts: density
 // counters sampled after every sweep s with s + 1 >= burn and
 // (s + 1 - burn) % stride == 0 (nullptr or stride 0 = off).
 int launch_resident(const Geom& g, uint32_t* rows, const ResidentPlan& plan, uint32_t sweep0,
-                    uint32_t nsweeps, const DevRng& rng, const ThrView& th, const int2* grange,
+                    uint32_t nsweeps, const DevRng& rng, const int2* grange,
                     unsigned int epoch, unsigned long long* ring, uint32_t* counts, uint64_t burn,
                     uint32_t stride, const uint8_t* colours, unsigned long long* flips, void* stream);
+
+// The word kernel (tl_words.cu): every lattice and threshold kind; a thread
+// owns up to plan.slots 32-site words of the stripe and its halos.
+size_t words_smem_bytes(const Geom& g, int local_rows);
+int words_prepare(const Geom& g, const ThrView& th, int threads, int slots, size_t smem_bytes, int* blocks_per_sm);
+int launch_words(const Geom& g, uint32_t* rows, const ResidentPlan& plan, uint32_t sweep0, uint32_t nsweeps,
+                 const DevRng& rng, const ThrView& th, const int2* grange, unsigned int epoch, unsigned long long* ring,
+                 uint32_t* counts, uint64_t burn, uint32_t stride, const uint8_t* colours, unsigned long long* flips,
+                 void* stream);
 // Colours of the pass slots of nsweeps sweeps under the random pass order.
 int launch_slot_colours(uint8_t* out, uint32_t sweep0, uint32_t nsweeps, int passes, const DevRng& rng, void* stream);
 
@@ -207,6 +216,9 @@ int launch_validate(const Geom& g, const uint8_t* canon, const uint8_t* aux, uns
 int dbg_fetch_kernels(unsigned long long* out, bool clear);
 int dbg_fetch_regdom(unsigned long long* out, bool clear);
 int dbg_fetch_resident(unsigned long long* out, bool clear);
+int dbg_fetch_words_domino(unsigned long long* out, bool clear);
+int dbg_fetch_words_lozenge(unsigned long long* out, bool clear);
+int dbg_fetch_words_sixv(unsigned long long* out, bool clear);
 int dbg_fetch_batch(unsigned long long* out, bool clear);
 int dbg_fetch_shuffle(unsigned long long* out, bool clear);
 int dbg_selftest();

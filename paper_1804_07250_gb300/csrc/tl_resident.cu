@@ -1,24 +1,18 @@
-// Shared-memory resident multi-sweep kernel (cooperative launch).
+// Shared-memory resident multi-sweep kernel for dominoes at t = 2^31 whose
+// stripes do not fit the register-resident kernel, or when a plan asks for it
+// (cooperative launch).
 //
-// The paper launches Rotate and Update once per half-step and moves the
-// whole tiling through device memory every time (Sec. 2.2).  Here one launch
-// runs many sweeps: each CTA keeps a horizontal stripe of the packed state
-// plus `halo` rows above and below it in shared memory.  A pass updates every
-// row whose inputs are still exact; because a site only reads edges within
-// one row of it, the exact region shrinks by one row at each interior stripe
-// edge per pass, so after `halo` passes the CTA still holds its own rows
-// exactly.  It then publishes its top and bottom `halo` rows and refreshes its
-// halos from its two neighbours.  State crosses the memory system once per
-// `halo` passes and only at stripe seams; otherwise it stays on chip.
+// Each CTA keeps a horizontal stripe of the packed state plus `halo` rows
+// above and below it in shared memory for a whole launch.  A pass updates
+// every row whose inputs are still exact; because a site only reads edges
+// within one row of it, the exact region shrinks by one row at each interior
+// stripe edge per pass, so after `halo` passes the CTA still holds its own
+// rows exactly.  It then publishes its top and bottom `halo` rows and
+// refreshes its halos from its two neighbours.
 //
-// Within a cycle of `halo` passes the work is split in two phases:
-//  1. random planes: the first `npre` Philox planes of every group the cycle
-//     will touch are generated up front into shared memory -- independent
-//     work that keeps the integer pipes busy;
-//  2. passes: each active 128-site group (from a per-CTA item table that
-//     lists only groups holding domain sites) reads its planes from shared
-//     memory, so a pass is a short chain of shared-memory loads and bitwise
-//     logic; planes beyond `npre` are generated on the spot when needed.
+// Half the warps update the current pass, from an item table of the active
+// 128-site groups, while the other half generate the random plane of the
+// next: at t = 2^31 one plane decides every site.
 //
 // Exchange: every boundary word travels with a 32-bit tag (launch epoch,
 // cycle) in one 64-bit store; the reader polls the 64-bit words until the
@@ -35,13 +29,12 @@ struct ResParams {
     uint32_t* rows0;            // global row 0 (after the pad row)
     Geom g;
     const int* stripe_lo;
-    int halo, npre;
+    int halo;
     const uint8_t* colours;     // random pass order: colour of every slot of the launch, else nullptr
     int cap_items;              // item-table capacity per CTA
     int cap_cycle;              // random-plane buffer capacity (groups per cycle)
     uint32_t sweep0, nsweeps;
     DevRng rng;
-    ThrView th;
     const int2* grange;
     unsigned long long* xbuf;   // tagged exchange words
     int* status;
@@ -94,47 +87,24 @@ TL_DEV void copy_rows_from_global(uint32_t* dst, const uint32_t* src, int64_t wo
     for (int64_t i = tid; i < words / 4; i += nt) d[i] = __ldcg(s + i);
 }
 
-// Item range of pass i (1-based) of a cycle: table `tab` entries [s, e).
+// Item range [s, e) of pass i (1-based) of a cycle.
 struct PassRange {
-    int tab, s, e;
+    int s, e;
 };
 
-template <int LAT>
-TL_DEV PassRange pass_range(const Geom& g, int i, uint32_t pass, int slo, int shi, bool bot, bool top,
-                            const int* off, int nloc)
+TL_DEV PassRange pass_range(const Geom& g, int i, int slo, int shi, bool bot, bool top, const int* off)
 {
     const int vlo = bot ? -1 : slo + (i - 1);
     const int vhi = top ? g.H + 1 : shi - (i - 1);
-    PassRange r;
-    if (LAT == LAT_SIXV) {
-        // face rows Y in [max(vlo,1), min(vhi-2, N-1)] of the class parity
-        const int a = vlo > 1 ? vlo : 1;
-        const int last = (vhi - 2) < (g.N - 1) ? (vhi - 2) : (g.N - 1);
-        r.tab = sixv_py(pass);
-        if (last < a) {
-            r.s = r.e = 0;
-            return r;
-        }
-        const int* o = off + r.tab * (nloc + 1);
-        r.s = o[a - slo];
-        r.e = o[last + 1 - slo];
-    } else {
-        const int a = (vlo + 1) > 0 ? (vlo + 1) : 0;
-        const int b = vhi < g.H ? vhi : g.H;
-        r.tab = 0;
-        if (b <= a) {
-            r.s = r.e = 0;
-            return r;
-        }
-        r.s = off[a - slo];
-        r.e = off[b - slo];
-    }
-    return r;
+    const int a = (vlo + 1) > 0 ? (vlo + 1) : 0;
+    const int b = vhi < g.H ? vhi : g.H;
+    if (b <= a) return PassRange{0, 0};
+    return PassRange{off[a - slo], off[b - slo]};
 }
 
-// FAST: dominoes at t = 2^31 with the branch-free, atomic-free group update;
-// every updater thread handles at most two groups per pass.
-template <int LAT, int TK, int NT, bool FAST>
+// Branch-free, atomic-free group update; every updater thread handles at most
+// two groups per pass.
+template <int NT>
 __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResParams P)
 {
     extern __shared__ uint4 smem4[];
@@ -143,8 +113,6 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResParams P)
     __shared__ int4 s_ptab[64];
     __shared__ uint32_t s_psweep[64];
     __shared__ uint32_t s_next_sweep, s_next_pass;
-    __shared__ __align__(16) uint32_t s_ttab[LAT == LAT_SIXV ? 32 * 16 : 4];   // expanded six-vertex table
-    __shared__ __align__(16) uint32_t s_ctab[LAT == LAT_SIXV ? 32 * 8 : 4];    // expanded count table
     const Geom& g = P.g;
     const int64_t RW = g.row_words;
     const int c = blockIdx.x, C = gridDim.x;
@@ -155,75 +123,57 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResParams P)
     const int slo = bot ? -1 : lo - h;
     const int shi = top ? g.H + 1 : hi + h;
     const int nloc = shi - slo;
-    constexpr int NTAB = (LAT == LAT_SIXV) ? 2 : 1;
 
     // shared memory carve-up: rows | random planes | item table | offsets
     uint32_t* sm = reinterpret_cast<uint32_t*>(smem4);
     uint32_t* srow0 = sm - (int64_t)slo * RW;   // srow0 + y * RW is global row y
     uint4* rbuf = reinterpret_cast<uint4*>(sm + (int64_t)nloc * RW);
-    uint32_t* items = reinterpret_cast<uint32_t*>(rbuf + (size_t)P.npre * P.cap_cycle);
+    uint32_t* items = reinterpret_cast<uint32_t*>(rbuf + P.cap_cycle);
     int* off = reinterpret_cast<int*>(items + P.cap_items);
-    // FAST only: 8-byte aligned after the offsets
-    uint2* fitems = reinterpret_cast<uint2*>((reinterpret_cast<uintptr_t>(off + NTAB * (nloc + 1)) + 7) & ~(uintptr_t)7);
+    // 8-byte aligned after the offsets
+    uint2* fitems = reinterpret_cast<uint2*>((reinterpret_cast<uintptr_t>(off + nloc + 1) + 7) & ~(uintptr_t)7);
 
     copy_rows_from_global(sm, P.rows0 + (int64_t)slo * RW, (int64_t)nloc * RW, tid, NT);
-    if (LAT == LAT_SIXV) {
-        for (int i = tid; i < 32 * 16; i += NT) s_ttab[i] = ((P.th.tmask[i >> 4] >> (i & 15)) & 1u) ? 0xFFFFFFFFu : 0u;
-        for (int i = tid; i < 32 * 8; i += NT) {
-            const int n = i & 7;
-            s_ctab[i] = (n < 5 && ((P.th.t5[n] >> (31 - (i >> 3))) & 1u)) ? 0xFFFFFFFFu : 0u;
-        }
-    }
-    const uint32_t* ctab = (LAT == LAT_SIXV && P.th.cpol >= 0) ? s_ctab : nullptr;
 
-    // item tables: active groups of each local row (six-vertex: one table per
-    // face-row parity), prefix offsets per table
-    for (int t = 0; t < NTAB; ++t)
-        for (int r = tid; r < nloc; r += NT) {
-            const int y = slo + r;
-            int cnt = 0;
-            if (y >= 0 && y < g.H && (NTAB == 1 || (y & 1) == t)) {
-                const int2 gr = P.grange[y];
-                cnt = gr.y > gr.x ? gr.y - gr.x : 0;
-            }
-            off[t * (nloc + 1) + r + 1] = cnt;
+    // item table: active groups of each local row, prefix offsets
+    for (int r = tid; r < nloc; r += NT) {
+        const int y = slo + r;
+        int cnt = 0;
+        if (y >= 0 && y < g.H) {
+            const int2 gr = P.grange[y];
+            cnt = gr.y > gr.x ? gr.y - gr.x : 0;
         }
+        off[r + 1] = cnt;
+    }
     __syncthreads();
     if (tid == 0) {
-        // absolute offsets: the tables are stored one after the other
-        int run = 0;
-        for (int t = 0; t < NTAB; ++t) {
-            int* o = off + t * (nloc + 1);
-            o[0] = run;
-            for (int r = 0; r < nloc; ++r) o[r + 1] += o[r];
-            run = o[nloc];
-        }
+        off[0] = 0;
+        for (int r = 0; r < nloc; ++r) off[r + 1] += off[r];
     }
     __syncthreads();
-    for (int t = 0; t < NTAB; ++t)
-        for (int r = tid; r < nloc; r += NT) {
-            const int y = slo + r;
-            if (y < 0 || y >= g.H || (NTAB == 2 && (y & 1) != t)) continue;
-            const int2 gr = P.grange[y];
-            int o = off[t * (nloc + 1) + r];
-            for (int m = gr.x; m < gr.y; ++m) {
+    for (int r = tid; r < nloc; r += NT) {
+        const int y = slo + r;
+        if (y < 0 || y >= g.H) continue;
+        const int2 gr = P.grange[y];
+        int o = off[r];
+        for (int m = gr.x; m < gr.y; ++m) {
 #ifdef TL_DEBUG
-                if (!TL_IN(o, P.cap_items, 201)) break;
+            if (!TL_IN(o, P.cap_items, 201)) break;
 #endif
-                if (FAST) {
-                    // word offset of (row y, plane 0, word 4m) and whether m+1 follows in this row
-                    fitems[o] = make_uint2((uint32_t)((int64_t)r * RW + 4 * m),
-                                           (uint32_t)y | ((uint32_t)m << 16) | (m + 1 < gr.y ? 0x80000000u : 0u));
-                }
-                items[o++] = ((uint32_t)r << 8) | (uint32_t)m;
-            }
+            // word offset of (row y, plane 0, word 4m) and whether m+1 follows in this row
+            fitems[o] = make_uint2((uint32_t)((int64_t)r * RW + 4 * m),
+                                   (uint32_t)y | ((uint32_t)m << 16) | (m + 1 < gr.y ? 0x80000000u : 0u));
+            items[o++] = ((uint32_t)r << 8) | (uint32_t)m;
         }
+    }
     __syncthreads();
 
     const int passes = g.passes;
     const uint64_t total = (uint64_t)P.nsweeps * passes;
     const size_t side_words = (size_t)h * RW;
+#ifdef TL_DEBUG
     const int cap = P.cap_cycle;
+#endif
     // warp roles: the first half updates the current pass, the second half
     // generates the random planes of the next pass
     constexpr int HALF = NT / 2;
@@ -248,7 +198,7 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResParams P)
         int base = 0;
         for (int i = 1; i <= hc_; ++i) {
             const uint32_t colour = P.colours ? P.colours[(size_t)(sweep - P.sweep0) * passes + pass] : pass;
-            const PassRange pr = pass_range<LAT>(g, i, colour, slo, shi, bot, top, off, nloc);
+            const PassRange pr = pass_range(g, i, slo, shi, bot, top, off);
             s_ptab[i - 1] = make_int4(pr.s, pr.e - pr.s, base, (int)(pass | (colour << 8)));
             s_psweep[i - 1] = sweep;
             base += pr.e - pr.s;
@@ -260,10 +210,7 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResParams P)
         s_next_sweep = sweep;
         s_next_pass = pass;
     };
-    // random planes of one pass (generator warps): per group, four planes
-    // at a time -- independent Philox chains the scheduler interleaves
-    // (computing all four even when fewer are kept measured faster than
-    // guarding them, and than spreading single planes over threads)
+    // random plane of one pass (generator warps)
     auto gen = [&](int i) {
         const int4 e = s_ptab[i];
         const uint32_t sweep = s_psweep[i], pass = (uint32_t)e.w & 255u;   // slot
@@ -273,17 +220,8 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResParams P)
 #endif
             const uint32_t item = items[e.x + it];
             const int y = slo + (int)(item >> 8), m = (int)(item & 255u);
-            const uint32_t grp = (uint32_t)(((LAT == LAT_SIXV) ? (y >> 1) : y) * g.Kg + m);
-            for (int k0 = 0; k0 < P.npre; k0 += 4) {
-                uint4 o[4];
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    o[q] = philox10(grp, sweep, ((uint32_t)(k0 + q) << 16) | pass, P.rng.stream, P.rng.k0,
-                                    P.rng.k1);
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    if (k0 + q < P.npre) rbuf[(size_t)(k0 + q) * cap + e.z + it] = o[q];
-            }
+            rbuf[e.z + it] =
+                philox10((uint32_t)(y * g.Kg + m), sweep, pass, P.rng.stream, P.rng.k0, P.rng.k1);
         }
     };
     // the first cycle's table and random planes; later cycles get theirs from
@@ -297,8 +235,8 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResParams P)
         const uint32_t next_sweep = s_next_sweep, next_pass = s_next_pass;
         for (int i = 0; i < hc; ++i) {
             const int4 e = s_ptab[i];
-            const uint32_t sweep = s_psweep[i], slot = (uint32_t)e.w & 255u, pass = (uint32_t)e.w >> 8;
-            if (FAST && upd_role) {
+            const uint32_t slot = (uint32_t)e.w & 255u, pass = (uint32_t)e.w >> 8, sweep = s_psweep[i];
+            if (upd_role) {
                 // read and decide every group of the pass, then store: groups
                 // read their neighbours' boundary words
                 constexpr int MAXI = NT >= 1024 ? 1 : 2;
@@ -332,24 +270,6 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResParams P)
 #pragma unroll
                 for (int q = 0; q < MAXI; ++q)
                     if (has[q]) domino_fast_store(r[q]);
-            } else if (!FAST && upd_role) {
-                for (int it = rtid; it < e.y; it += HALF) {
-#ifdef TL_DEBUG
-                    if (!TL_IN(e.x + it, P.cap_items, 207) || !TL_IN(e.z + it, cap, 203)) continue;
-                    // dominoes and lozenges read rows y - 1 and y, a six-vertex
-                    // face row the vertex rows y and y + 1
-                    if (!TL_IN((int)(items[e.x + it] >> 8) - (LAT == LAT_SIXV ? 0 : 1), nloc - 1, 208)) continue;
-#endif
-                    const uint32_t item = items[e.x + it];
-                    const int y = slo + (int)(item >> 8), m = (int)(item & 255u);
-                    const uint32_t grp = (uint32_t)(((LAT == LAT_SIXV) ? (y >> 1) : y) * g.Kg + m);
-                    const RndPre rnd{rbuf + e.z + it, P.npre, cap, RndPhilox{grp, sweep, slot, P.rng}};
-                    // a six-vertex face row y touches vertex rows y and y + 1
-                    // and is this stripe's if its lower row is
-                    group_update<LAT, TK>(srow0 + (int64_t)y * RW, RW, g, y, m, pass, rnd, P.th,
-                                          LAT == LAT_SIXV ? s_ttab : nullptr, ctab,
-                                          (P.flips && y >= lo && y < hi) ? &nflip : nullptr);
-                }
             } else if (i + 1 < hc) {
                 gen(i + 1);
             }
@@ -483,29 +403,16 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResParams P)
     if (P.flips && nflip) atomicAdd(P.flips, (unsigned long long)nflip);
 }
 
-template <int LAT, int TK>
-static const void* kernel_ptr(int threads)
+static const void* pick(int threads)
 {
-    return threads > 512 ? reinterpret_cast<const void*>(&resident_kernel<LAT, TK, 1024, false>)
-                         : reinterpret_cast<const void*>(&resident_kernel<LAT, TK, 512, false>);
+    return threads > 512 ? reinterpret_cast<const void*>(&resident_kernel<1024>)
+                         : reinterpret_cast<const void*>(&resident_kernel<512>);
 }
 
-static const void* pick(int lattice, int tk, int threads, bool fast = false)
-{
-    if (fast)
-        return threads > 512 ? reinterpret_cast<const void*>(&resident_kernel<LAT_DOMINO, THR_SCALAR, 1024, true>)
-                             : reinterpret_cast<const void*>(&resident_kernel<LAT_DOMINO, THR_SCALAR, 512, true>);
-    if (lattice == LAT_DOMINO)
-        return tk == THR_SITE ? kernel_ptr<LAT_DOMINO, THR_SITE>(threads) : kernel_ptr<LAT_DOMINO, THR_SCALAR>(threads);
-    if (lattice == LAT_LOZENGE)
-        return tk == THR_SITE ? kernel_ptr<LAT_LOZENGE, THR_SITE>(threads) : kernel_ptr<LAT_LOZENGE, THR_SCALAR>(threads);
-    return kernel_ptr<LAT_SIXV, THR_TABLE>(threads);
-}
-
-int resident_prepare(const Geom& g, int thr_kind, int threads, bool fast, size_t smem_bytes, int* blocks_per_sm)
+int resident_prepare(int threads, size_t smem_bytes, int* blocks_per_sm)
 {
     *blocks_per_sm = 0;
-    const void* k = pick(g.lattice, thr_kind, threads, fast);
+    const void* k = pick(threads);
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -517,7 +424,7 @@ int resident_prepare(const Geom& g, int thr_kind, int threads, bool fast, size_t
 }
 
 int launch_resident(const Geom& g, uint32_t* rows, const ResidentPlan& plan, uint32_t sweep0,
-                    uint32_t nsweeps, const DevRng& rng, const ThrView& th, const int2* grange,
+                    uint32_t nsweeps, const DevRng& rng, const int2* grange,
                     unsigned int epoch, unsigned long long* ring, uint32_t* counts, uint64_t burn,
                     uint32_t stride, const uint8_t* colours, unsigned long long* flips, void* stream)
 {
@@ -527,14 +434,12 @@ int launch_resident(const Geom& g, uint32_t* rows, const ResidentPlan& plan, uin
     P.g = g;
     P.stripe_lo = plan.stripe_lo;
     P.halo = plan.halo;
-    P.npre = plan.npre;
     P.colours = colours;
     P.cap_items = plan.cap_items;
     P.cap_cycle = plan.cap_cycle;
     P.sweep0 = sweep0;
     P.nsweeps = nsweeps;
     P.rng = rng;
-    P.th = th;
     P.grange = grange;
     P.xbuf = plan.xbuf;
     P.status = plan.status;
@@ -544,7 +449,7 @@ int launch_resident(const Geom& g, uint32_t* rows, const ResidentPlan& plan, uin
     P.stride = stride;
     P.epoch = epoch;
     void* args[] = {&P};
-    const void* k = pick(g.lattice, th.kind, plan.threads, plan.fast);
+    const void* k = pick(plan.threads);
     return (int)cudaLaunchCooperativeKernel(k, dim3(plan.ctas), dim3(plan.threads), args, plan.smem_bytes,
                                             reinterpret_cast<cudaStream_t>(stream));
 }
