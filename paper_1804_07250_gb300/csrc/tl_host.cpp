@@ -202,12 +202,11 @@ struct Canon {
     }
 };
 
-// Groups of a row that hold sites of the domain, plus one group to the left
-// (it owns the word whose top bit is the W edge of the first site).
+// Groups of a row that hold sites of the domain.
 static void set_group_range(tl_domain* d, int row, int jmin, int jmax)
 {
     if (jmin > jmax) d->grange[row] = make_int2(0, 0);
-    else d->grange[row] = make_int2(std::max(0, (jmin >> 7) - 1), (jmax >> 7) + 1);
+    else d->grange[row] = make_int2(jmin >> 7, (jmax >> 7) + 1);
 }
 
 // Height segments over a grid of hw x hh points, given membership tests
@@ -1605,7 +1604,9 @@ static int plan_fast(tl_chain* c)
     std::vector<int> pre(g.H + 1, 0);
     std::vector<double> w(g.H + 1, 0.0);
     for (int y = 0; y < g.H; ++y) {
-        const int act = std::max(0, d.grange[y].y - d.grange[y].x);
+        // and the group left of them, which writes the word they share
+        const int2 gr = d.grange[y];
+        const int act = gr.y > gr.x ? gr.y - std::max(0, gr.x - 1) : 0;
         pre[y + 1] = pre[y] + act;
         w[y + 1] = w[y] + 0.1 + act;
     }

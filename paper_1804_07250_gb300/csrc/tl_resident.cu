@@ -135,12 +135,18 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResParams P)
 
     copy_rows_from_global(sm, P.rows0 + (int64_t)slo * RW, (int64_t)nloc * RW, tid, NT);
 
-    // item table: active groups of each local row, prefix offsets
+    // item table: active groups of each local row and the one left of them
+    // (it writes the word they share), prefix offsets
+    auto row_groups = [&](int y) {
+        int2 gr = P.grange[y];
+        if (gr.y > gr.x && gr.x > 0) --gr.x;
+        return gr;
+    };
     for (int r = tid; r < nloc; r += NT) {
         const int y = slo + r;
         int cnt = 0;
         if (y >= 0 && y < g.H) {
-            const int2 gr = P.grange[y];
+            const int2 gr = row_groups(y);
             cnt = gr.y > gr.x ? gr.y - gr.x : 0;
         }
         off[r + 1] = cnt;
@@ -154,7 +160,7 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResParams P)
     for (int r = tid; r < nloc; r += NT) {
         const int y = slo + r;
         if (y < 0 || y >= g.H) continue;
-        const int2 gr = P.grange[y];
+        const int2 gr = row_groups(y);
         int o = off[r];
         for (int m = gr.x; m < gr.y; ++m) {
 #ifdef TL_DEBUG
