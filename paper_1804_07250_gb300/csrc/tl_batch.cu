@@ -10,7 +10,7 @@
 // writes the other; consecutive launches alternate.  Sweep indices come from
 // a per-chain device counter, so a block of launches captured in a CUDA graph
 // can be replayed: the graph ends with a kernel that advances the counters.
-#include "tl_device.cuh"
+#include "tl_words.cuh"
 
 #include <cstdint>
 
@@ -70,72 +70,137 @@ TL_DEV void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" :
 TL_DEV void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 TL_DEV void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
-template <int LAT, int TK>
-TL_DEV void tile_passes(const BatchChain& ch, uint32_t* srow0, int slo, int shi, bool bot, bool top, uint32_t sweep0,
-                        int R)
+struct TileView {
+    uint32_t* sm;              // row slo
+    const uint32_t* items;     // (row - slo) << 8 | group; six-vertex: of the even row of the pair
+    const int* off;            // first item of every row (pair) from r0 on
+    const uint32_t* ttab;      // six-vertex table, expanded; or
+    const uint32_t* ctab;      // its count form, expanded (nullptr: general)
+    uint4* pk;                 // [2][32] plane keys of a pass, by its parity
+    int r0;
+    int slo, shi;
+    bool bot, top;
+};
+
+// Random planes of one group: 16 of Philox's 20 products, the rest in the
+// group's key and in the pass's table of plane keys.
+struct RndKeyed {
+    GroupKey key;
+    const uint4* pk;
+    DevRng rng;
+    TL_DEV uint4 operator()(int k) const
+    {
+        const uint4 v = pk[k];
+        const PlaneKey p{v.x, v.y, v.z};
+        return philox_keyed(key, p, rng);
+    }
+};
+// Two planes compared as one subtraction (borrow out: less; no difference:
+// undecided).
+TL_DEV void hb_pair(uint32_t& lt, uint32_t& und, uint32_t u0, uint32_t t0, uint32_t u1, uint32_t t1)
 {
+    const uint32_t l = (~u0 & t0) | (~(u0 ^ t0) & ~u1 & t1);
+    lt |= und & l;
+    und &= ~(u0 ^ t0) & ~(u1 ^ t1);
+}
+template <class TB>
+TL_DEV uint4 heat_bath(uint4 f, int kmax, const RndKeyed& rnd, const TB& tb)
+{
+    uint4 und = f;
+    uint4 lt = make_uint4(0u, 0u, 0u, 0u);
+    int k = 0;
+    for (; k + 1 <= kmax; k += 2) {
+        if (!any4(und)) return lt;
+        const uint4 o0 = rnd(k), o1 = rnd(k + 1);
+        const uint4 t0 = tb(k), t1 = tb(k + 1);
+        hb_pair(lt.x, und.x, o0.x, t0.x, o1.x, t1.x);
+        hb_pair(lt.y, und.y, o0.y, t0.y, o1.y, t1.y);
+        hb_pair(lt.z, und.z, o0.z, t0.z, o1.z, t1.z);
+        hb_pair(lt.w, und.w, o0.w, t0.w, o1.w, t1.w);
+    }
+    if (k <= kmax && any4(und)) hb_compare(lt, und, rnd(k), tb(k));
+    return lt;
+}
+
+template <int LAT, int TK, int NT>
+TL_DEV void tile_passes(const BatchChain& ch, const TileView& t, uint32_t sweep0, int R)
+{
+    constexpr bool SIX = LAT == LAT_SIXV;
     const Geom& g = ch.g;
     const int64_t RW = g.row_words;
-    const int passes = g.passes;
+    const int Kg = g.Kg, passes = g.passes;
+    const DevRng rng = ch.rng;
     int i = 0;
     for (int r = 0; r < R; ++r) {
         const uint32_t sweep = sweep0 + (uint32_t)r;
         for (int p = 0; p < passes; ++p, ++i) {
-            const int vlo = bot ? -1 : slo + i;
-            const int vhi = top ? g.H + 1 : shi - i;
-            int a, nrows, step;
-            if (LAT == LAT_SIXV) {
+            const uint32_t pass = (uint32_t)p;
+            const int vlo = t.bot ? -1 : t.slo + i;
+            const int vhi = t.top ? g.H + 1 : t.shi - i;
+            // exact rows [a, b) (six-vertex: face rows), and their items
+            int a, b;
+            if (SIX) {
                 a = vlo > 1 ? vlo : 1;
-                const int last = (vhi - 2) < (g.N - 1) ? (vhi - 2) : (g.N - 1);
-                if ((a & 1) != sixv_py((uint32_t)p)) ++a;
-                step = 2;
-                nrows = last >= a ? (last - a) / 2 + 1 : 0;
+                b = ((vhi - 2) < (g.N - 1) ? (vhi - 2) : (g.N - 1)) + 1;
             } else {
                 a = (vlo + 1) > 0 ? (vlo + 1) : 0;
-                const int b = vhi < g.H ? vhi : g.H;
-                step = 1;
-                nrows = b > a ? b - a : 0;
+                b = vhi < g.H ? vhi : g.H;
             }
-            const int items = nrows * g.Kg;
-            for (int it = threadIdx.x; it < items; it += blockDim.x) {
-                const int ri = it / g.Kg, m = it - ri * g.Kg;
-                const int y = a + ri * step;
-                const int2 gr = ch.grange[y];
-                if (m < gr.x || m >= gr.y) continue;
-                const uint32_t grp = (uint32_t)(((LAT == LAT_SIXV) ? (y >> 1) : y) * g.Kg + m);
-                const RndPhilox rnd{grp, sweep, (uint32_t)p, ch.rng};
-                group_update<LAT, TK>(srow0 + (int64_t)y * RW, RW, g, y, m, (uint32_t)p, rnd, ch.th);
+            const int v = SIX ? sixv_py(pass) : 0;
+            int s = 0, e = 0;
+            if (b > a) {
+                s = t.off[(SIX ? a >> 1 : a) - t.r0];
+                e = t.off[(SIX ? ((b - 1) >> 1) + 1 : b) - t.r0];
+            }
+            // the next pass's plane keys
+            if (threadIdx.x < 32) {
+                const bool wrap = p + 1 == passes;
+                PlaneKey k;
+                k.set(threadIdx.x, wrap ? 0u : pass + 1u, wrap ? sweep + 1u : sweep, rng);
+                t.pk[((i + 1) & 1) * 32 + threadIdx.x] = make_uint4(k.l1, k.l0, k.h0, 0u);
+            }
+            for (int x = s + (int)threadIdx.x; x < e; x += NT) {
+                const uint32_t en = t.items[x];
+                const int y = t.slo + (int)(en >> 8) + v, m = (int)(en & 255u);
+                if (SIX && (y < a || y >= b)) continue;
+                RndKeyed rnd;
+                rnd.key.set((uint32_t)((SIX ? y >> 1 : y) * Kg + m), rng);
+                rnd.pk = t.pk + (i & 1) * 32;
+                rnd.rng = rng;
+                group_update<LAT, TK>(t.sm + (int64_t)(y - t.slo) * RW, RW, g, y, m, pass, rnd, ch.th, t.ttab, t.ctab);
             }
             __syncthreads();
         }
     }
 }
 
-// NT threads per tile: a thread takes every NT-th 128-face group of a pass
-// (the faces per thread the autotuner picks).  256 threads: three CTAs per
-// SM (at most 85 registers a thread): the passes of a tile are separated by
-// barriers, and a third resident tile hides them better than the registers
-// spilled to L1 cost (two CTAs at 124 registers measured 9% slower, four at
-// 64 registers no faster).  128 threads: six CTAs per SM at the same
-// registers, twice the faces per thread, as many tiles as shared memory
-// holds.
+// NT threads per tile: the plan's 256 or 128, or 512 where a launch has too few
+// tiles to fill the SMs that way.  Registers without spills (128 a
+// thread) beat more threads: 128 weighted diamonds of order 16 to 512, read
+// out after 500 sweeps, take 6.9 ms at 512 threads an SM, 7.4 at 768 (80
+// registers), 7.7 at 1,024; a lane per 32 sites instead of per 128 (a quad
+// sharing the Philox outputs) 9.6: its update costs as much per word as this
+// one per group.
 template <int NT>
-__global__ void __launch_bounds__(NT, NT == 128 ? 6 : 3) batch_kernel(const BatchChain* __restrict__ chains,
-                                                                    const BatchTile* __restrict__ tiles, int ntiles,
-                                                                    int R, uint32_t sweep_off, int src,
-                                                                    unsigned int* cursor, int* __restrict__ status)
+__global__ void __launch_bounds__(NT, 512 / NT) batch_kernel(const BatchChain* __restrict__ chains,
+                                                              const BatchTile* __restrict__ tiles, int ntiles, int R,
+                                                              uint32_t sweep_off, int src, unsigned int* cursor,
+                                                              int* __restrict__ status)
 {
     extern __shared__ uint4 smem4[];
     __shared__ int s_tile;
     __shared__ __align__(8) unsigned long long s_bar;
+    __shared__ uint4 s_pk[2 * 32];
+    __shared__ __align__(16) uint32_t s_ttab[32 * 16];   // expanded six-vertex table
+    const int tid = threadIdx.x;
     uint32_t* sm = reinterpret_cast<uint32_t*>(smem4);
-    if (threadIdx.x == 0) mbar_init(&s_bar, 1);
+    if (tid == 0) mbar_init(&s_bar, 1);
     __syncthreads();
     uint32_t parity = 0;
     for (;;) {
         // a raised status word (a wait that gave up elsewhere, or raised by
         // the host) stops the block before it issues another copy
-        if (threadIdx.x == 0) s_tile = *(volatile int*)status ? ntiles : (int)atomicAdd(cursor, 1u);
+        if (tid == 0) s_tile = *(volatile int*)status ? ntiles : (int)atomicAdd(cursor, 1u);
         __syncthreads();
         const int t = s_tile;
         __syncthreads();
@@ -146,23 +211,59 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 6 : 3) batch_kernel(const Batc
         const int64_t RW = g.row_words;
         const int halo = g.passes * R;
         const bool bot = tile.lo == 0, top = tile.hi == g.H;
-        const int slo = bot ? -1 : (tile.lo - halo > -1 ? tile.lo - halo : -1);
-        const int shi = top ? g.H + 1 : (tile.hi + halo < g.H + 1 ? tile.hi + halo : g.H + 1);
+        TileView tv;
+        tv.slo = bot ? -1 : (tile.lo - halo > -1 ? tile.lo - halo : -1);
+        tv.shi = top ? g.H + 1 : (tile.hi + halo < g.H + 1 ? tile.hi + halo : g.H + 1);
         // a halo clamped at a pad row is exact from then on
-        const bool bot_x = slo == -1, top_x = shi == g.H + 1;
+        tv.bot = tv.slo == -1;
+        tv.top = tv.shi == g.H + 1;
+        const int nloc = tv.shi - tv.slo;
         const uint32_t* srcp = ch.rows[src] + RW;   // global row 0
         uint32_t* dstp = ch.rows[src ^ 1] + RW;
+        // rows (pairs of face rows) with items, and their prefix counts
+        const bool six = g.lattice == LAT_SIXV;
+        const int r1 = tv.shi < g.H ? tv.shi : g.H;
+        tv.r0 = tv.slo > 0 ? tv.slo : 0;
+        if (six) tv.r0 >>= 1;
+        const int nr = (six ? (r1 + 1) >> 1 : r1) - tv.r0;
+        int* const off = reinterpret_cast<int*>(sm + (int64_t)nloc * RW);
+        uint32_t* const items = reinterpret_cast<uint32_t*>(off + nr + 1);
 #ifdef TL_DEBUG
         {
-            // the tile and its halo rows fit the block's shared memory
+            // the tile, its halo rows and its item table fit the block's shared memory
             uint32_t dyn;
             asm volatile("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn));
-            if (!TL_IN((int64_t)(shi - slo) * RW * 4 - 1, (int64_t)dyn, 301)) continue;
+            const int64_t need = (int64_t)nloc * RW * 4 + 4 * (nr + 1) + 4 * (int64_t)(ch.gpre[tv.r0 + nr] - ch.gpre[tv.r0]);
+            if (!TL_IN(need - 1, (int64_t)dyn, 301)) continue;
         }
 #endif
         // the tile and its halo rows are contiguous: one bulk copy into shared
         // memory (rows are whole 16-byte units, buffers 256-byte aligned)
-        if (threadIdx.x == 0) bulk_load(sm, srcp + (int64_t)slo * RW, (uint32_t)((int64_t)(shi - slo) * RW * 4), &s_bar);
+        if (tid == 0) bulk_load(sm, srcp + (int64_t)tv.slo * RW, (uint32_t)((int64_t)nloc * RW * 4), &s_bar);
+        const int first = ch.gpre[tv.r0];
+        for (int r = tid; r <= nr; r += NT) off[r] = ch.gpre[tv.r0 + r] - first;
+        for (int r = tid; r < nr; r += NT) {
+            const int x0 = ch.gpre[tv.r0 + r] - first, n = ch.gpre[tv.r0 + r + 1] - first - x0;
+            const int m0 = ch.gfirst[tv.r0 + r], y = (six ? 2 : 1) * (tv.r0 + r);
+            for (int j = 0; j < n; ++j) items[x0 + j] = (uint32_t)(y - tv.slo) << 8 | (uint32_t)(m0 + j);
+        }
+        if (six) {
+            // threshold bits by corner index, or (count form) by corner count
+            if (ch.th.cpol < 0)
+                for (int x = tid; x < 32 * 16; x += NT)
+                    s_ttab[x] = ((ch.th.tmask[x >> 4] >> (x & 15)) & 1u) ? 0xFFFFFFFFu : 0u;
+            else
+                for (int x = tid; x < 32 * 8; x += NT) {
+                    const int n = x & 7;
+                    s_ttab[x] = (n < 5 && ((ch.th.t5[n] >> (31 - (x >> 3))) & 1u)) ? 0xFFFFFFFFu : 0u;
+                }
+        }
+        const uint32_t sweep0 = *ch.sweep_base + sweep_off;
+        if (tid < 32) {
+            PlaneKey k;
+            k.set((uint32_t)tid, 0u, sweep0, ch.rng);
+            s_pk[tid] = make_uint4(k.l1, k.l0, k.h0, 0u);
+        }
         const int arrived = __syncthreads_and(mbar_wait_bounded(&s_bar, parity) ? 1 : 0);
         parity ^= 1u;
         if (!arrived) {
@@ -170,37 +271,41 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 6 : 3) batch_kernel(const Batc
             // one more bounded wait so that nothing is left writing this
             // block's shared memory, and stop (every thread of the block
             // takes this branch together)
-            if (threadIdx.x == 0) {
+            if (tid == 0) {
                 atomicExch(status, 1);
                 mbar_wait_bounded(&s_bar, parity ^ 1u);
             }
             __syncthreads();
             return;
         }
-        const uint32_t sweep0 = *ch.sweep_base + sweep_off;
-        uint32_t* srow0 = sm - (int64_t)slo * RW;
+        tv.sm = sm;
+        tv.items = items;
+        tv.off = off;
+        tv.ttab = s_ttab;
+        tv.ctab = six && ch.th.cpol >= 0 ? s_ttab : nullptr;
+        tv.pk = s_pk;
         if (g.lattice == LAT_DOMINO) {
-            if (ch.th.kind == THR_SITE) tile_passes<LAT_DOMINO, THR_SITE>(ch, srow0, slo, shi, bot_x, top_x, sweep0, R);
-            else tile_passes<LAT_DOMINO, THR_SCALAR>(ch, srow0, slo, shi, bot_x, top_x, sweep0, R);
+            if (ch.th.kind == THR_SITE) tile_passes<LAT_DOMINO, THR_SITE, NT>(ch, tv, sweep0, R);
+            else tile_passes<LAT_DOMINO, THR_SCALAR, NT>(ch, tv, sweep0, R);
         } else if (g.lattice == LAT_LOZENGE) {
-            if (ch.th.kind == THR_SITE) tile_passes<LAT_LOZENGE, THR_SITE>(ch, srow0, slo, shi, bot_x, top_x, sweep0, R);
-            else tile_passes<LAT_LOZENGE, THR_SCALAR>(ch, srow0, slo, shi, bot_x, top_x, sweep0, R);
+            if (ch.th.kind == THR_SITE) tile_passes<LAT_LOZENGE, THR_SITE, NT>(ch, tv, sweep0, R);
+            else tile_passes<LAT_LOZENGE, THR_SCALAR, NT>(ch, tv, sweep0, R);
         } else {
-            tile_passes<LAT_SIXV, THR_TABLE>(ch, srow0, slo, shi, bot_x, top_x, sweep0, R);
+            tile_passes<LAT_SIXV, THR_TABLE, NT>(ch, tv, sweep0, R);
         }
         // the tile's own rows back in one bulk copy; shared memory is reused
         // by the next tile once the copy has read it
         fence_proxy_async();
         __syncthreads();
-        if (threadIdx.x == 0) {
-            bulk_store(dstp + (int64_t)tile.lo * RW, srow0 + (int64_t)tile.lo * RW,
+        if (tid == 0) {
+            bulk_store(dstp + (int64_t)tile.lo * RW, sm + (int64_t)(tile.lo - tv.slo) * RW,
                        (uint32_t)((int64_t)(tile.hi - tile.lo) * RW * 4));
             bulk_wait_read();
         }
         // the pad rows of the destination stay zero: they are never written
         __syncthreads();
     }
-    if (threadIdx.x == 0) bulk_wait_all();
+    if (tid == 0) bulk_wait_all();
 }
 
 __global__ void batch_advance_kernel(const BatchChain* __restrict__ chains, int nchains, uint32_t k,
@@ -213,19 +318,24 @@ __global__ void batch_advance_kernel(const BatchChain* __restrict__ chains, int 
 
 static const void* batch_pick(int threads)
 {
-    return threads == 128 ? reinterpret_cast<const void*>(&batch_kernel<128>)
-                          : reinterpret_cast<const void*>(&batch_kernel<256>);
+    return threads == 128   ? reinterpret_cast<const void*>(&batch_kernel<128>)
+           : threads == 256 ? reinterpret_cast<const void*>(&batch_kernel<256>)
+                            : reinterpret_cast<const void*>(&batch_kernel<512>);
 }
 
 int batch_prepare(size_t smem_bytes, int threads, int* blocks_per_sm)
 {
     const void* k = batch_pick(threads);
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        return (int)e;
-    }
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, threads == 128 ? 128 : 256, smem_bytes);
+    // the largest limit, whatever this plan needs: a plan must not lower
+    // another batch's
+    int dev = 0, optin = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    cudaFuncAttributes fa{};
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, threads, smem_bytes);
     if (e != cudaSuccess) cudaGetLastError();
     return (int)e;
 }
@@ -233,12 +343,9 @@ int batch_prepare(size_t smem_bytes, int threads, int* blocks_per_sm)
 int launch_batch(const BatchChain* chains, const BatchTile* tiles, int ntiles, int R, uint32_t sweep_off, int src,
                  unsigned int* cursor, int grid, int threads, size_t smem_bytes, int* status, void* stream)
 {
-    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    if (threads == 128)
-        batch_kernel<128><<<grid, 128, smem_bytes, st>>>(chains, tiles, ntiles, R, sweep_off, src, cursor, status);
-    else
-        batch_kernel<256><<<grid, 256, smem_bytes, st>>>(chains, tiles, ntiles, R, sweep_off, src, cursor, status);
-    return (int)cudaGetLastError();
+    void* args[] = {&chains, &tiles, &ntiles, &R, &sweep_off, &src, &cursor, &status};
+    return (int)cudaLaunchKernel(batch_pick(threads), dim3(grid), dim3(threads), args, smem_bytes,
+                                 reinterpret_cast<cudaStream_t>(stream));
 }
 
 int launch_batch_advance(const BatchChain* chains, int nchains, uint32_t k, unsigned int* cursors, int ncursors,

@@ -1086,6 +1086,24 @@ static int upload_state(tl_chain* c, const uint8_t* canon, bool device_src, void
     return TL_OK;
 }
 
+// Active groups [x, y) of every row; six-vertex: of every pair of face rows.
+static std::vector<int2> unit_groups(const tl_domain& d)
+{
+    const Geom& g = d.g;
+    if (g.lattice != LAT_SIXV) return d.grange;
+    std::vector<int2> u;
+    for (int y = 0; y < g.H; y += 2) {
+        int2 a = d.grange[y];
+        if (y + 1 < g.H) {
+            const int2 b = d.grange[y + 1];
+            if (a.y <= a.x) a = b;
+            else if (b.y > b.x) a = make_int2(std::min(a.x, b.x), std::max(a.y, b.y));
+        }
+        u.push_back(a);
+    }
+    return u;
+}
+
 TL_API int tl_chain_create(tl_ctx* ctx, const tl_domain* d, const uint8_t* canon_init, uint64_t seed,
                            uint32_t stream_id, const tl_thresholds* th, tl_chain** out)
 {
@@ -1117,14 +1135,27 @@ TL_API int tl_chain_create(tl_ctx* ctx, const tl_domain* d, const uint8_t* canon
     const size_t ncanon = (size_t)g.ntype * g.W * g.H;
     if ((rc = dev_alloc(&c->rows, (size_t)g.total_words, "state")) ||
         (rc = dev_alloc(&c->rows0, (size_t)g.total_words, "start state")) ||
-        (rc = dev_alloc(&c->grange, (size_t)g.H, "group ranges")) ||
+        (rc = dev_alloc(&c->grange, (size_t)g.H + ((size_t)g.H + 2), "group ranges")) ||
         (rc = dev_alloc(&c->canon, ncanon, "staging")) || (rc = dev_alloc(&c->hash, 1, "hash")) ||
         (rc = dev_alloc(&c->hseg, (size_t)6 * std::max(d->nseg, 1), "height plan")) ||
         (rc = dev_alloc(&c->hbase, (size_t)std::max(d->nseg, 1), "height plan"))) {
         chain_free(c);
         return rc;
     }
-    cudaError_t e = cudaMemcpy(c->grange, d->grange.data(), sizeof(int2) * g.H, cudaMemcpyHostToDevice);
+    // group ranges, then (for batches) the prefix counts and first groups of
+    // the rows, for the six-vertex model of the pairs of face rows
+    std::vector<int2> gr(d->grange);
+    gr.resize((size_t)g.H + ((size_t)g.H + 2), make_int2(0, 0));
+    {
+        const std::vector<int2> u = unit_groups(*d);
+        int* const pre = reinterpret_cast<int*>(gr.data() + g.H);
+        int* const first = pre + g.H + 2;
+        for (size_t r = 0; r < u.size(); ++r) {
+            pre[r + 1] = pre[r] + std::max(0, u[r].y - u[r].x);
+            first[r] = u[r].x;
+        }
+    }
+    cudaError_t e = cudaMemcpy(c->grange, gr.data(), sizeof(int2) * gr.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess && d->nseg)
         e = cudaMemcpy(c->hseg, d->hseg.data(), sizeof(int) * 6 * d->nseg, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
@@ -1675,13 +1706,9 @@ static int plan_words(tl_chain* c)
     std::vector<int> pre(U + 1, 0);
     std::vector<double> w(g.H + 1, 0.0);
     int maxact = 0;
+    const std::vector<int2> unit = unit_groups(d);
     for (int r = 0; r < U; ++r) {
-        int2 gr = d.grange[step * r];
-        if (sixv && 2 * r + 1 < g.H) {
-            const int2 b = d.grange[2 * r + 1];
-            if (gr.y <= gr.x) gr = b;
-            else if (b.y > b.x) gr = make_int2(std::min(gr.x, b.x), std::max(gr.y, b.y));
-        }
+        const int2 gr = unit[r];
         const int act = std::max(0, gr.y - gr.x);
         pre[r + 1] = pre[r] + act;
         maxact = std::max(maxact, act);
@@ -2685,6 +2712,7 @@ struct tl_batch {
     int* d_status = nullptr;              // raised by a bounded wait that gave up
     int tile_rows = 64, R = 2, block = 100, grid = 0;
     int threads = 256;                    // threads per tile (faces per thread)
+    int run_threads = 256;                // threads per tile of the launches: more where tiles are few
     size_t smem = 0;
     int ntiles = 0;
     int src = 0;                          // buffer holding the current state
@@ -2737,29 +2765,44 @@ static int batch_plan(tl_batch* b, int tile_rows, int R, int threads)
     std::vector<double> work;
     std::vector<int> first;
     size_t smem = 0;
+    // a batch with fewer tiles than SMs takes lower tiles (down to 32 rows)
+    // and more threads per tile: a serving mix of 12 jobs in 62 tiles of 128
+    // rows left 90 SMs idle
+    int rows = tile_rows;
+    auto count = [&](int r) {
+        size_t n = 0;
+        for (const tl_chain* c : b->chains) n += (size_t)((c->g.H + r - 1) / r);
+        return n;
+    };
+    while (rows >= 64 && count(rows) < (size_t)b->ctx->sms) rows = (rows + 3) / 4 * 2;
     for (size_t i = 0; i < b->chains.size(); ++i) {
         const tl_chain* c = b->chains[i];
         const Geom& g = c->g;
-        const int halo = g.passes * R;
+        const int halo = g.passes * R, step = g.lattice == LAT_SIXV ? 2 : 1;
+        const std::vector<int2> unit = unit_groups(c->dom_copy);
+        std::vector<int> pre(unit.size() + 1, 0);
+        for (size_t r = 0; r < unit.size(); ++r) pre[r + 1] = pre[r] + std::max(0, unit[r].y - unit[r].x);
         first.push_back((int)tiles.size());
-        for (int lo = 0; lo < g.H; lo += tile_rows) {
-            const int hi = std::min(g.H, lo + tile_rows);
+        for (int lo = 0; lo < g.H; lo += rows) {
+            const int hi = std::min(g.H, lo + rows);
             tiles.push_back(BatchTile{(int)i, lo, hi});
             const int slo = std::max(lo - halo, -1), shi = std::min(hi + halo, g.H + 1);
-            smem = std::max(smem, (size_t)(shi - slo) * (size_t)g.row_words * 4);
-            double wk = 0;
-            for (int y = std::max(slo, 0); y < std::min(shi, g.H); ++y) {
-                const int2 r = c->dom_copy.grange[y];
-                wk += 0.1 + std::max(0, r.y - r.x);
-            }
-            work.push_back(wk * R);
+            const int ra = std::max(slo, 0) / step, rb = (std::min(shi, g.H) + step - 1) / step;
+            const int items = pre[rb] - pre[ra];
+            // rows, then the item table
+            smem = std::max(smem, (size_t)(shi - slo) * (size_t)g.row_words * 4 + 4 * (size_t)(rb - ra + 1 + items));
+            work.push_back((0.1 * (rb - ra) + items) * R);
         }
     }
     first.push_back((int)tiles.size());
     if ((long)smem > (long)b->ctx->smem_optin) return fail(TL_EUNSUPPORTED, "batch plan: a tile needs %zu B of shared memory", smem);
     int bps = 0;
-    if (batch_prepare(smem, threads, &bps) != 0 || bps < 1)
-        return fail(TL_EUNSUPPORTED, "batch plan: tile kernel does not fit");
+    int run_threads = tiles.size() <= (size_t)b->ctx->sms ? 512 : tiles.size() <= 2 * (size_t)b->ctx->sms ? 256 : threads;
+    if (batch_prepare(smem, run_threads, &bps) != 0 || bps < 1) {
+        run_threads = threads;
+        if (batch_prepare(smem, threads, &bps) != 0 || bps < 1)
+            return fail(TL_EUNSUPPORTED, "batch plan: tile kernel does not fit");
+    }
     std::vector<int> order(tiles.size());
     for (size_t i = 0; i < order.size(); ++i) order[i] = (int)i;
     std::stable_sort(order.begin(), order.end(), [&](int a, int c) { return work[a] > work[c]; });
@@ -2777,6 +2820,7 @@ static int batch_plan(tl_batch* b, int tile_rows, int R, int threads)
     b->tile_rows = tile_rows;
     b->R = R;
     b->threads = threads;
+    b->run_threads = run_threads;
     b->smem = smem;
     b->grid = std::min(bps * b->ctx->sms, b->ntiles);
     return TL_OK;
@@ -2812,7 +2856,8 @@ static int batch_rebuild(tl_batch* b)
         bc.g = c->g;
         bc.rows[0] = c->rows;
         bc.rows[1] = b->alt[i];
-        bc.grange = c->grange;
+        bc.gpre = reinterpret_cast<const int*>(c->grange + c->g.H);
+        bc.gfirst = bc.gpre + c->g.H + 2;
         bc.th = c->th;
         bc.rng = c->rng;
         bc.sweep_base = b->d_sweep + i;
@@ -2919,7 +2964,7 @@ static int batch_launch(tl_batch* b, int r, uint32_t off, int slot, void* stream
     unsigned int* cur = b->d_cursor + (slot % b->ncursor);
     if (!per_chain) {
         CUDA_TRY(cudaMemsetAsync(cur, 0, 4, SS(stream)));
-        const int e = launch_batch(b->d_chains, b->d_tiles_lpt, b->ntiles, r, off, b->src, cur, b->grid, b->threads,
+        const int e = launch_batch(b->d_chains, b->d_tiles_lpt, b->ntiles, r, off, b->src, cur, b->grid, b->run_threads,
                                    b->smem, b->d_status, stream);
         if (e) return fail(TL_ECUDA, "batch kernel: %s", cudaGetErrorString((cudaError_t)e));
         b->launches += 1;
@@ -2929,7 +2974,7 @@ static int batch_launch(tl_batch* b, int r, uint32_t off, int slot, void* stream
             unsigned int* ci = b->d_cursor + ((slot * (int)b->chains.size() + (int)i) % b->ncursor);
             CUDA_TRY(cudaMemsetAsync(ci, 0, 4, SS(stream)));
             const int e = launch_batch(b->d_chains, b->d_tiles_chain + t0, nt, r, off, b->src, ci,
-                                       std::min(nt, b->grid), b->threads, b->smem, b->d_status, stream);
+                                       std::min(nt, b->grid), b->run_threads, b->smem, b->d_status, stream);
             if (e) return fail(TL_ECUDA, "batch kernel: %s", cudaGetErrorString((cudaError_t)e));
             b->launches += 1;
         }

@@ -184,7 +184,8 @@ int launch_regdom(const Geom& g, uint32_t* rows, const RegPlan& plan, uint32_t s
 struct BatchChain {
     Geom g;
     uint32_t* rows[2];          // two packed state buffers (ping-pong), each with pad rows
-    const int2* grange;
+    const int* gpre;            // active groups of the rows before each row (six-vertex: pair of face rows)
+    const int* gfirst;          // first active group of each row (pair)
     ThrView th;
     DevRng rng;
     uint32_t* sweep_base;       // device counter: absolute sweep of the next launch block
@@ -192,7 +193,7 @@ struct BatchChain {
 struct BatchTile {
     int chain, lo, hi;          // owned rows [lo, hi) of chain `chain`
 };
-// threads per tile: 256 or 128
+// threads per tile: 128, 256 or 512
 int batch_prepare(size_t smem_bytes, int threads, int* blocks_per_sm);
 // status: device int raised if a bounded wait for a tile's bulk copy gave up.
 int launch_batch(const BatchChain* chains, const BatchTile* tiles, int ntiles, int R, uint32_t sweep_off, int src,
