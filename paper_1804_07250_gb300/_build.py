@@ -22,7 +22,7 @@ LIB_DEBUG = os.path.join(HERE, "libtiling_debug.so")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SOURCES = ["tl_kernels.cu", "tl_resident.cu", "tl_words.cu", "tl_words_domino.cu", "tl_words_lozenge.cu",
-           "tl_words_sixv.cu", "tl_regdom.cu", "tl_batch.cu", "tl_shuffle.cu", "tl_host.cpp", "tl_thurston.cpp"]
+           "tl_words_sixv.cu", "tl_regdom.cu", "tl_small.cu", "tl_batch.cu", "tl_shuffle.cu", "tl_host.cpp", "tl_thurston.cpp"]
 
 
 def nvcc() -> str:

@@ -998,6 +998,7 @@ struct tl_chain {
     // register-resident domino kernel (dominoes at t = 2^31)
     bool use_reg = false;
     RegPlan reg{};
+    int small_threads = 0;             // > 0: plain runs take the one-block kernel
     int2* hull_d = nullptr;
     // device validation of written states: the domain's cover or boundary
     // edges, and the first failure found
@@ -1578,6 +1579,20 @@ static int plan_regdom(tl_chain* c)
     c->res.status = c->status_d;
     c->use_reg = true;
     c->res_ready = true;
+    // domains of at most 1,024 words of sites: plain runs take the one-block
+    // kernel (automatic plans only); hashed, sampled, counted and randomly
+    // ordered runs stay here
+    c->small_threads = 0;
+    if (c->kernel == 0 && c->halo_req == 0) {
+        long groups[2] = {0, 0};
+        for (int y = 0; y < H; ++y) {
+            const int2 r = d.grange[y];
+            groups[y & 1] += r.y > r.x ? r.y - std::max(0, r.x - 1) : 0;
+        }
+        const int st = small_threads(groups[0], groups[1]);
+        bool fits = false;
+        if (st <= 1024 && small_prepare(small_smem_bytes(g), st, &fits) == 0 && fits) c->small_threads = st;
+    }
     return TL_OK;
 }
 
@@ -1826,6 +1841,12 @@ static bool want_resident(tl_chain* c)
 // (the largest halo a plan takes).
 constexpr size_t kMaxLaunchSlots = (size_t)60000 * 64;
 
+// Whether a plain run of the (planned) chain takes the one-block kernel.
+static bool small_run(const tl_chain* c)
+{
+    return c->use_reg && c->small_threads > 0 && !c->density_on && !c->random_order && !c->count_flips;
+}
+
 // Resident launches over [c->sweep, c->sweep + k), at most spl sweeps each.
 static int run_resident(tl_chain* c, uint64_t k, unsigned long long* ring, void* stream)
 {
@@ -1854,7 +1875,8 @@ static int run_resident(tl_chain* c, uint64_t k, unsigned long long* ring, void*
             if (ec) return fail(TL_ECUDA, "colour kernel: %s", cudaGetErrorString((cudaError_t)ec));
             c->launches += 1;
         }
-        if (c->use_reg && (uint64_t)n * c->g.passes > (uint64_t)c->reg.halo) {
+        const bool small = small_run(c) && !ring;
+        if (c->use_reg && !small && (uint64_t)n * c->g.passes > (uint64_t)c->reg.halo) {
             // the register kernel's exchange tags count cycles within one
             // launch: its buffers start every launch cleared
             CUDA_TRY(cudaMemsetAsync(c->xbuf_d, 0,
@@ -1862,7 +1884,10 @@ static int run_resident(tl_chain* c, uint64_t k, unsigned long long* ring, void*
                                      SS(stream)));
         }
         const int e =
-            c->use_reg
+            small
+                ? launch_small(c->g, c->rows, nullptr, c->small_threads, (uint32_t)c->sweep, (uint32_t)n, c->rng,
+                               c->grange, stream)
+            : c->use_reg
                 ? launch_regdom(c->g, c->rows, c->reg, (uint32_t)c->sweep, (uint32_t)n, c->rng, ++c->epoch,
                                 ring ? ring + done : nullptr, dens ? c->cplanes : nullptr, c->burn,
                                 dens ? c->stride : 0, c->random_order ? c->colours : nullptr,
@@ -1953,7 +1978,7 @@ TL_API int tl_debug_checks(int clear, uint64_t* failures, int* first_id, int64_t
 {
 #ifdef TL_DEBUG
     CUDA_TRY(cudaDeviceSynchronize());
-    int (*const fetch[])(unsigned long long*, bool) = {dbg_fetch_kernels, dbg_fetch_regdom, dbg_fetch_resident,
+    int (*const fetch[])(unsigned long long*, bool) = {dbg_fetch_kernels, dbg_fetch_regdom, dbg_fetch_small, dbg_fetch_resident,
                                                        dbg_fetch_words_domino, dbg_fetch_words_lozenge, dbg_fetch_words_sixv,
                                                        dbg_fetch_batch, dbg_fetch_shuffle};
     uint64_t n = 0;
@@ -2528,12 +2553,45 @@ TL_API int tl_cftp(tl_ctx* ctx, const tl_domain* d, uint64_t seed, uint32_t stre
     std::vector<uint8_t> a, b;
     uint64_t T = t0;
     bool done = false;
+    // the two chains share every random number and run at the same time: in
+    // one launch of the one-block kernel where they take it, else on two streams
+    // where their stripes fit the SMs together
+    const bool res = rc == TL_OK && want_resident(top) && want_resident(bot);
+    const bool pair = res && small_run(top) && small_run(bot);
+    cudaStream_t side = nullptr;
+    cudaEvent_t ready = nullptr;
+    if (res && !pair && top->res.ctas + bot->res.ctas <= ctx->sms &&
+        (cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking) != cudaSuccess ||
+         cudaEventCreateWithFlags(&ready, cudaEventDisableTiming) != cudaSuccess))
+        rc = fail(TL_ECUDA, "tl_cftp: side stream");
     while (rc == TL_OK && !done) {
         for (tl_chain* c : {top, bot}) {
             if (rc == TL_OK) rc = tl_chain_reset(c, stream);
             if (rc == TL_OK) rc = tl_chain_seek(c, 0x100000000ull - T);
-            if (rc == TL_OK) rc = tl_run_sweeps(c, T, stream);
-            if (rc == TL_OK) rc = tl_chain_sync(c, stream);
+        }
+        if (pair) {
+            const int e = rc == TL_OK ? launch_small(top->g, top->rows, bot->rows, top->small_threads,
+                                                     (uint32_t)top->sweep, (uint32_t)T, top->rng, top->grange, stream)
+                                      : 0;
+            if (e) rc = fail(TL_ECUDA, "tl_cftp: %s", cudaGetErrorString((cudaError_t)e));
+            for (tl_chain* c : {top, bot}) {
+                c->sweep += T;
+                c->launches += 1;
+            }
+        } else if (side) {
+            cudaError_t e = cudaEventRecord(ready, SS(stream));   // the resets
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(side, ready, 0);
+            if (rc == TL_OK && e != cudaSuccess) rc = fail(TL_ECUDA, "tl_cftp: %s", cudaGetErrorString(e));
+            if (rc == TL_OK) rc = tl_run_sweeps(top, T, stream);
+            if (rc == TL_OK) rc = tl_run_sweeps(bot, T, side);
+            const int rs = tl_chain_sync(bot, side);
+            if (rc == TL_OK) rc = rs;
+            if (rc == TL_OK) rc = tl_chain_sync(top, stream);
+        } else {
+            for (tl_chain* c : {top, bot}) {
+                if (rc == TL_OK) rc = tl_run_sweeps(c, T, stream);
+                if (rc == TL_OK) rc = tl_chain_sync(c, stream);
+            }
         }
         uint64_t ht = 0, hb = 0;
         if (rc == TL_OK) rc = tl_state_hash(top, &ht, stream);
@@ -2565,6 +2623,9 @@ TL_API int tl_cftp(tl_ctx* ctx, const tl_domain* d, uint64_t seed, uint32_t stre
         }
         if (t_used) *t_used = T;
     }
+    if (side) cudaStreamSynchronize(side);
+    if (ready) cudaEventDestroy(ready);
+    if (side) cudaStreamDestroy(side);
     tl_chain_destroy(top);
     tl_chain_destroy(bot);
     return rc;

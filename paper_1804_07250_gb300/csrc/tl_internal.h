@@ -180,6 +180,14 @@ int launch_regdom(const Geom& g, uint32_t* rows, const RegPlan& plan, uint32_t s
                   const DevRng& rng, unsigned int epoch, unsigned long long* ring, uint32_t* counts, uint64_t burn,
                   uint32_t stride, const uint8_t* colours, unsigned long long* flips, void* stream);
 
+// One-block kernel for small domino domains at t = 2^31 (tl_small.cu), on one
+// chain or on two of the same domain and randomness at once (rows_b).
+size_t small_smem_bytes(const Geom& g);
+int small_threads(long even, long odd);
+int small_prepare(size_t smem_bytes, int threads, bool* fits);
+int launch_small(const Geom& g, uint32_t* rows_a, uint32_t* rows_b, int threads, uint32_t sweep0, uint32_t nsweeps,
+                 const DevRng& rng, const int2* grange, void* stream);
+
 // ---- batched chains (tl_batch.cu) ----
 struct BatchChain {
     Geom g;
@@ -216,6 +224,7 @@ int launch_validate(const Geom& g, const uint8_t* canon, const uint8_t* aux, uns
 // on an out-of-range index (id 999) without the access it guards.
 int dbg_fetch_kernels(unsigned long long* out, bool clear);
 int dbg_fetch_regdom(unsigned long long* out, bool clear);
+int dbg_fetch_small(unsigned long long* out, bool clear);
 int dbg_fetch_resident(unsigned long long* out, bool clear);
 int dbg_fetch_words_domino(unsigned long long* out, bool clear);
 int dbg_fetch_words_lozenge(unsigned long long* out, bool clear);
