@@ -2742,12 +2742,12 @@ TL_API int tl_read_domino_nsew(tl_chain* c, double* out, size_t cap, void* strea
     if (cap < n) return fail(TL_EINVAL, "tl_read_domino_nsew: cap %zu < %zu", cap, n);
     CUDA_TRY(cudaSetDevice(c->ctx->device));
     TL_TRY(zero_counts_if_needed(c, stream));
-    const int ed = launch_density_decode(c->g, c->cplanes, c->samples, c->counts, stream);
-    if (ed) return fail(TL_ECUDA, "density decode: %s", cudaGetErrorString((cudaError_t)ed));
-    c->launches += 1;
-    return to_output(c, out, n, stream, [&](double* o) {
-        return launch_nsew(c->g, c->counts, c->samples, c->kappa, o, stream);
+    int launches = 1;
+    const int rc = to_output(c, out, n, stream, [&](double* o) {
+        return launch_nsew(c->g, c->cplanes, c->counts, c->samples, c->kappa, c->ctx->smem_optin, o, &launches, stream);
     });
+    if (rc == TL_OK) c->launches += (uint64_t)(launches - 1);
+    return rc;
 }
 
 // ---------------------------------------------------------------------------

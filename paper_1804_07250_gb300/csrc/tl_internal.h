@@ -76,8 +76,9 @@ int launch_density_accumulate(const Geom& g, const uint32_t* rows, uint32_t* cpl
 int launch_density_decode(const Geom& g, const uint32_t* cplanes, uint64_t samples, uint32_t* counts, void* stream);
 int launch_density_read(const uint32_t* counts, uint64_t n, uint64_t samples, double* out,
                         void* stream);
-int launch_nsew(const Geom& g, const uint32_t* counts, uint64_t samples, int kappa, double* out,
-                void* stream);
+// counts: canonical counters, used where a row does not fit shared memory.
+int launch_nsew(const Geom& g, const uint32_t* cplanes, uint32_t* counts, uint64_t samples, int kappa, int smem_optin,
+                double* out, int* launches, void* stream);
 // Domino shuffling of the Aztec diamond of order n (tl_shuffle.cu) into
 // packed rows of the diamond's chain layout (Kw words per plane row).
 // Resident form: cooperative launches of consecutive steps, in each of which
