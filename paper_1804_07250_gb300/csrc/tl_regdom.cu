@@ -27,7 +27,7 @@
 // and a 3-bit cycle tag, double buffered by cycle parity (the buffers are
 // cleared before every launch); every wait is bounded (2 s) and raises a
 // status word instead of hanging.
-#include "tl_device.cuh"
+#include "tl_words.cuh"
 
 #include <cstdint>
 #include <type_traits>
@@ -327,10 +327,18 @@ __global__ void __launch_bounds__(NT, 1) regdom_kernel(const RegParams P)
     // passes, so cycles (and launches) start at slot 0 and the shared-memory
     // buffer of a pass is its slot.
     uint4 oA0 = {}, oA1 = {}, oB0 = {}, oB1 = {};
-    if (act) {
-        oA0 = philox10(grp0, sweep, 0u, P.rng.stream, P.rng.k0, P.rng.k1);
-        oA1 = philox10(grp1, sweep, 0u, P.rng.stream, P.rng.k0, P.rng.k1);
-    }
+    // 16 of Philox's 20 products a call: those of the first two rounds are in
+    // the groups' keys, or the same for the whole pass
+    GroupKey key0, key1;
+    key0.set(grp0, P.rng);
+    key1.set(grp1, P.rng);
+    auto draw2 = [&](uint32_t sw, uint32_t slot, uint4& a, uint4& b) {
+        PlaneKey pk;
+        pk.set(0u, slot, sw, P.rng);
+        a = philox_keyed(key0, pk, P.rng);
+        b = philox_keyed(key1, pk, P.rng);
+    };
+    if (act) draw2(sweep, 0u, oA0, oA1);
     // One pass: colour parity PAR1 (the parity of row y0, y0 even), slot SL.
     auto pass = [&](auto par1c, auto slc, int ip, const uint4& oc0, const uint4& oc1, uint4& on0, uint4& on1) {
         constexpr bool par1 = decltype(par1c)::value;
@@ -343,8 +351,7 @@ __global__ void __launch_bounds__(NT, 1) regdom_kernel(const RegParams P)
         if (live) {
             uint4 f0, f1;
             uint32_t b0, b1;
-            on0 = philox10(grp0, nsweep, nslot, P.rng.stream, P.rng.k0, P.rng.k1);
-            on1 = philox10(grp1, nsweep, nslot, P.rng.stream, P.rng.k0, P.rng.k1);
+            draw2(nsweep, nslot, on0, on1);
             if (!par1) {
                 f0 = row_par0(He0, Ho0, pv0, Ve0, Se, oc0, b0);
                 f1 = row_par1(He1, Ho1, Vo1, Vo0, oc1, b1);
@@ -518,8 +525,7 @@ __global__ void __launch_bounds__(NT, 1) regdom_kernel(const RegParams P)
 #endif
 #pragma unroll
                 for (int q = 0; q < kXUnits; ++q) rd_ld2(src + ((size_t)q * Kg + m) * 2, &f[2 * q], &f[2 * q + 1]);
-            oA0 = philox10(grp0, sweep, 0u, P.rng.stream, P.rng.k0, P.rng.k1);
-            oA1 = philox10(grp1, sweep, 0u, P.rng.stream, P.rng.k0, P.rng.k1);
+            draw2(sweep, 0u, oA0, oA1);
             uint64_t t_wait = 0;
             unsigned need = (1u << kXUnits) - 1;
             for (unsigned spin = 1;; ++spin) {
