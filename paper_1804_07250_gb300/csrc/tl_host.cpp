@@ -2647,7 +2647,7 @@ TL_API int tl_read_height(tl_chain* c, int32_t* out, size_t cap, void* stream)
     }
     const int e = launch_height(c->g, c->rows, c->hseg, d.nseg, d.hw, d.hh, dst, c->hbase, stream);
     if (e) return fail(TL_ECUDA, "height kernels: %s", cudaGetErrorString((cudaError_t)e));
-    c->launches += d.nseg ? 4 : 1;
+    c->launches += (uint64_t)height_launches(d.nseg, d.hw, d.hh);
     if (!dev) {
         CUDA_TRY(cudaMemcpyAsync(out, dst, n * sizeof(int32_t), cudaMemcpyDeviceToHost, SS(stream)));
         CUDA_TRY(cudaStreamSynchronize(SS(stream)));
@@ -2671,7 +2671,7 @@ TL_API int tl_read_height_noalloc(tl_chain* c, int32_t* out, size_t cap, void* s
                                "need a staging allocation)");
     const int e = launch_height_noalloc(c->g, c->rows, c->hseg, d.nseg, d.hw, d.hh, out, c->ctx->device, stream);
     if (e) return fail(TL_ECUDA, "tl_read_height_noalloc: %s", cudaGetErrorString((cudaError_t)e));
-    c->launches += d.nseg ? 4 : 1;
+    c->launches += (uint64_t)height_launches(d.nseg, d.hw, d.hh);
     return TL_OK;
 }
 

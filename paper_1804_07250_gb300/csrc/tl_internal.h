@@ -104,6 +104,7 @@ int launch_shuffle_global(int n, int Kw, size_t total_words, uint32_t* A, uint32
 // seg: [nseg][6] height segments (y, lo, hi, parent, xs, dir); base_scratch: nseg ints.
 int launch_height(const Geom& g, const uint32_t* rows, const int* seg, int nseg, int hw, int hh,
                   int32_t* out, int* base_scratch, void* stream);
+int height_launches(int nseg, int hw, int hh);   // kernels it launches
 int launch_threshold_planes(const Geom& g, const uint32_t* t_site_dev, uint32_t* planes,
                             void* stream);
 // Device-generated log-normal weights -> per-site thresholds [H][W].

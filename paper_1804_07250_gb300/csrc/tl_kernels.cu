@@ -428,8 +428,37 @@ __global__ void hash_kernel(const uint32_t* __restrict__ rows0, Geom g, unsigned
     if ((threadIdx.x & 31) == 0 && acc) atomicAdd(out, (unsigned long long)acc);
 }
 
+// The same in one block, writing the result itself (small states: one launch
+// instead of a clear and a launch).
+constexpr int64_t kSmallHashWords = 8192;
+__global__ void __launch_bounds__(1024) hash_small_kernel(const uint32_t* __restrict__ rows0, Geom g,
+                                                          unsigned long long* out)
+{
+    __shared__ unsigned long long part[32];
+    const int n = g.H * (int)g.row_words, RW = (int)g.row_words;
+    uint64_t acc = 0;
+    for (int i = threadIdx.x; i < n; i += 1024) {
+        const uint32_t w = rows0[i];
+        if (!w) continue;
+        const int y = i / RW, rem = i - y * RW, pl = rem / g.K;
+        acc += word_hash(w, g, y, pl, rem - pl * g.K);
+    }
+    for (int off = 16; off; off >>= 1) acc += __shfl_down_sync(0xFFFFFFFFu, acc, off);
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        unsigned long long t = 0;
+        for (int w = 0; w < 32; ++w) t += part[w];
+        *out = t;
+    }
+}
+
 int launch_hash(const Geom& g, const uint32_t* rows, unsigned long long* out, void* stream)
 {
+    if ((int64_t)g.H * g.row_words <= kSmallHashWords) {
+        hash_small_kernel<<<1, 1024, 0, S(stream)>>>(rows + g.row_words, g, out);
+        return (int)cudaGetLastError();
+    }
     cudaError_t e = cudaMemsetAsync(out, 0, sizeof(unsigned long long), S(stream));
     if (e != cudaSuccess) return (int)e;
     const int64_t n = (int64_t)g.H * g.row_words;
@@ -662,6 +691,26 @@ __global__ void height_fill_kernel(int32_t* __restrict__ out, int64_t n)
         out[i] = INT32_MIN;
 }
 
+// Heights of vertices [a, b) of row y (a warp, 32 at a time), from `run` at a;
+// the row's segment ends at hi.
+template <int LAT>
+TL_DEV void scan_steps(const uint32_t* rows0, const Geom& g, int y, int a, int b, int hi, int run, int32_t* o)
+{
+    const int lane = threadIdx.x & 31;
+    for (int x0 = a; x0 < b; x0 += 32) {
+        const int x = x0 + lane;
+        const int st = x < hi && x < b ? hstep<LAT>(rows0, g, x, y) : 0;
+        int inc = st;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int v = __shfl_up_sync(0xFFFFFFFFu, inc, d);
+            if (lane >= d) inc += v;
+        }
+        if (x < b) o[x] = run + inc - st;
+        run += __shfl_sync(0xFFFFFFFFu, inc, 31);
+    }
+}
+
 // Heights along each segment relative to its left end: each of the block's
 // warps takes an eighth of it, sums its steps, and then scans them 32 at a
 // time from the sum of the warps before it.
@@ -689,29 +738,16 @@ __global__ void __launch_bounds__(256) height_seg_kernel(const uint32_t* __restr
     __syncthreads();
     int run = 0;   // height of the warp's first vertex relative to lo
     for (int w = 0; w < warp; ++w) run += part[w];
-    for (int x0 = a; x0 < b; x0 += 32) {
-        const int x = x0 + lane;
-        const int st = x < hi && x < b ? hstep<LAT>(rows0, g, x, y) : 0;
-        int inc = st;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const int v = __shfl_up_sync(0xFFFFFFFFu, inc, d);
-            if (lane >= d) inc += v;
-        }
-        if (x < b) o[x] = run + inc - st;
-        run += __shfl_sync(0xFFFFFFFFu, inc, 31);
-    }
+    scan_steps<LAT>(rows0, g, y, a, b, hi, run, o);
 }
 
 // Offsets of the segments, 1,024 at a time: the differences to the parents,
 // then every segment follows its parents within the batch, doubling its reach
 // each round (parents come first, so those of earlier batches are done).
 template <int LAT>
-__global__ void __launch_bounds__(1024) height_link_kernel(const uint32_t* __restrict__ rows0, Geom g,
-                                                           const int* __restrict__ seg, int nseg, int hw,
-                                                           const int32_t* __restrict__ rel, int* __restrict__ base)
+TL_DEV void link_segments(const uint32_t* rows0, const Geom& g, const int* seg, int nseg, int hw, const int32_t* rel,
+                          int* base, int* val, int* up)
 {
-    __shared__ int val[1024], up[1024];
     const int t = threadIdx.x;
     for (int c0 = 0; c0 < nseg; c0 += 1024) {
         const int s = c0 + t;
@@ -742,6 +778,39 @@ __global__ void __launch_bounds__(1024) height_link_kernel(const uint32_t* __res
     }
 }
 
+template <int LAT>
+__global__ void __launch_bounds__(1024) height_link_kernel(const uint32_t* __restrict__ rows0, Geom g,
+                                                           const int* __restrict__ seg, int nseg, int hw,
+                                                           const int32_t* __restrict__ rel, int* __restrict__ base)
+{
+    __shared__ int val[1024], up[1024];
+    link_segments<LAT>(rows0, g, seg, nseg, hw, rel, base, val, up);
+}
+
+// All of it in one block, for grids so small that four launches take longer.
+constexpr int64_t kSmallHeights = 32768;
+template <int LAT>
+__global__ void __launch_bounds__(1024) height_small_kernel(const uint32_t* __restrict__ rows0, Geom g,
+                                                            const int* __restrict__ seg, int nseg, int hw, int n,
+                                                            int32_t* out, int* base)
+{
+    __shared__ int val[1024], up[1024];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int i = threadIdx.x; i < n; i += 1024) out[i] = INT32_MIN;
+    __syncthreads();
+    for (int s = warp; s < nseg; s += 32) {
+        const int y = seg[6 * s], lo = seg[6 * s + 1], hi = seg[6 * s + 2];
+        scan_steps<LAT>(rows0, g, y, lo, hi + 1, hi, 0, out + (size_t)y * hw);
+    }
+    __syncthreads();
+    link_segments<LAT>(rows0, g, seg, nseg, hw, out, base, val, up);
+    __syncthreads();
+    for (int s = warp; s < nseg; s += 32) {
+        const int y = seg[6 * s], lo = seg[6 * s + 1], hi = seg[6 * s + 2], b = base[s];
+        for (int x = lo + lane; x <= hi; x += 32) out[(size_t)y * hw + x] += b;
+    }
+}
+
 __global__ void __launch_bounds__(256) height_add_kernel(int32_t* __restrict__ out, const int* __restrict__ seg,
                                                          const int* __restrict__ base, int hw)
 {
@@ -752,22 +821,31 @@ __global__ void __launch_bounds__(256) height_add_kernel(int32_t* __restrict__ o
     for (int x = lo + threadIdx.x; x <= hi; x += 256) o[x] += b;
 }
 
+int height_launches(int nseg, int hw, int hh)
+{
+    return nseg <= 0 || ((int64_t)hw * hh <= kSmallHeights && nseg <= 1024) ? 1 : 4;
+}
+
 int launch_height(const Geom& g, const uint32_t* rows, const int* seg, int nseg, int hw, int hh, int32_t* out,
                   int* base_scratch, void* stream)
 {
     const uint32_t* rows0 = rows + g.row_words;
-    height_fill_kernel<<<grid_for((int64_t)hw * hh, 256), 256, 0, S(stream)>>>(out, (int64_t)hw * hh);
-    if (nseg > 0) {
-        auto run = [&](auto lat) {
-            constexpr int LAT = decltype(lat)::value;
-            height_seg_kernel<LAT><<<nseg, 256, 0, S(stream)>>>(rows0, g, seg, hw, out);
-            height_link_kernel<LAT><<<1, 1024, 0, S(stream)>>>(rows0, g, seg, nseg, hw, out, base_scratch);
-        };
-        if (g.lattice == LAT_DOMINO) run(std::integral_constant<int, LAT_DOMINO>{});
-        else if (g.lattice == LAT_LOZENGE) run(std::integral_constant<int, LAT_LOZENGE>{});
-        else run(std::integral_constant<int, LAT_SIXV>{});
+    const int64_t n = (int64_t)hw * hh;
+    auto run = [&](auto lat) {
+        constexpr int LAT = decltype(lat)::value;
+        if (nseg > 0 && height_launches(nseg, hw, hh) == 1) {
+            height_small_kernel<LAT><<<1, 1024, 0, S(stream)>>>(rows0, g, seg, nseg, hw, (int)n, out, base_scratch);
+            return;
+        }
+        height_fill_kernel<<<grid_for(n, 256), 256, 0, S(stream)>>>(out, n);
+        if (nseg <= 0) return;
+        height_seg_kernel<LAT><<<nseg, 256, 0, S(stream)>>>(rows0, g, seg, hw, out);
+        height_link_kernel<LAT><<<1, 1024, 0, S(stream)>>>(rows0, g, seg, nseg, hw, out, base_scratch);
         height_add_kernel<<<nseg, 256, 0, S(stream)>>>(out, seg, base_scratch, hw);
-    }
+    };
+    if (g.lattice == LAT_DOMINO) run(std::integral_constant<int, LAT_DOMINO>{});
+    else if (g.lattice == LAT_LOZENGE) run(std::integral_constant<int, LAT_LOZENGE>{});
+    else run(std::integral_constant<int, LAT_SIXV>{});
     return (int)cudaGetLastError();
 }
 
