@@ -1388,29 +1388,30 @@ static void stripe_local(int lo, int hi, int k, int C, int h, int H, int* slo, i
     *shi = k == C - 1 ? H + 1 : hi + h;
 }
 
-// Register-resident domino kernel: the groups each row pair holds, a stripe
-// partition of the pairs that balances the work of a cycle (owned pairs every
-// pass, halo pairs while they can still reach the stripe), and buffers.
-static int plan_regdom(tl_chain* c)
+// Groups that the register-resident domino kernel holds of each row pair.
+struct RegHull {
+    std::vector<int2> hull;
+    std::vector<long> w, pre;   // their number, prefix sums
+};
+
+static RegHull reg_hull(const tl_chain* c)
 {
     const Geom& g = c->g;
     const tl_domain& d = c->dom_copy;
-    const int h = c->halo_req > 0 ? c->halo_req : 8;
-    if (h & 1) {
-        c->res_why = "the register-resident kernel needs an even halo";
-        return TL_EUNSUPPORTED;
-    }
+    RegHull rh;
     const int H = g.H, W = g.W;
     const int npairs = (H + 1) / 2;
-    const int hp = h / 2;
     // extents of the domain's faces per face row
     std::vector<int> fmin(std::max(H - 1, 0), 1 << 30), fmax(std::max(H - 1, 0), -1);
-    for (int fy = 0; fy + 1 < H; ++fy)
-        for (int fx = 0; fx + 1 < W; ++fx)
-            if (d.cover[(size_t)fy * (W - 1) + fx]) {
-                fmin[fy] = std::min(fmin[fy], fx);
-                fmax[fy] = std::max(fmax[fy], fx);
-            }
+    for (int fy = 0; fy + 1 < H; ++fy) {
+        const uint8_t* cv = d.cover.data() + (size_t)fy * (W - 1);
+        int a = 0, b = W - 2;
+        while (a < W - 1 && !cv[a]) ++a;
+        if (a == W - 1) continue;
+        while (!cv[b]) --b;
+        fmin[fy] = a;
+        fmax[fy] = b;
+    }
     auto join = [](int2 a, int2 b) {
         if (a.y <= a.x) return b;
         if (b.y <= b.x) return a;
@@ -1436,11 +1437,46 @@ static int plan_regdom(tl_chain* c)
         w[q] = hull[q].y - hull[q].x;
         pre[q + 1] = pre[q] + w[q];
     }
-    const int max_threads = 512;
+    rh.hull = std::move(hull);
+    rh.w = std::move(w);
+    rh.pre = std::move(pre);
+    return rh;
+}
+
+// Register-resident domino kernel with `h` passes per exchange: a stripe
+// partition of the row pairs that balances the work of a cycle (owned pairs
+// every pass, halo pairs while they can still reach the stripe), and buffers.
+//
+// `max_threads`: threads a stripe may take (512, or fewer to find out whether a
+// deeper halo keeps the stripes that small).
+static int plan_regdom(tl_chain* c, const RegHull& rh, int h, int max_threads)
+{
+    const Geom& g = c->g;
+    const tl_domain& d = c->dom_copy;
+    if (h & 1) {
+        c->res_why = "the register-resident kernel needs an even halo";
+        return TL_EUNSUPPORTED;
+    }
+    const int H = g.H;
+    const int npairs = (H + 1) / 2;
+    const int hp = h / 2;
+    const std::vector<int2>& hull = rh.hull;
+    const std::vector<long>&w = rh.w, &pre = rh.pre;
     auto items = [&](int a, int b) {
         const int lo = a > 0 ? std::max(0, a - hp) : a, hi = b < npairs ? std::min(npairs, b + hp) : b;
         return pre[hi] - pre[lo];
     };
+    if (max_threads < 512) {
+        // a quick answer where the stripes cannot be that small: the fewest
+        // stripes that hold the groups, halos included
+        int stripes = 0;
+        for (int a = 0; a < npairs; ++stripes) {
+            int b = std::min(npairs, a + hp);
+            if (items(a, b) > max_threads || stripes >= c->ctx->sms) return TL_EUNSUPPORTED;
+            while (b < npairs && items(a, b + 1) <= max_threads) ++b;
+            a = b;
+        }
+    }
     // Work of one exchange cycle, in warp-passes: threads take the held
     // groups of the stripe's local pairs in order, 32 to a warp, and a warp
     // runs in the passes where any of its pairs is still useful (owned pairs
@@ -1811,7 +1847,23 @@ static void free_resident(tl_chain* c)
 static int plan_resident(tl_chain* c)
 {
     if (c->kernel != 2 && fast_candidate(c) && c->g.Kg <= 4096) {
-        const int rc = plan_regdom(c);
+        // Passes per exchange: 8, or the deepest halo with which no stripe
+        // needs more than four warps.  Up to one warp per scheduler a pass
+        // costs the latency of one warp's chain, so halo rows are free and
+        // every exchange (about 3,500 cycles) counts; beyond, halo rows cost
+        // more than the exchanges they save.  us a sweep at 8 -> the chosen
+        // halo: Aztec 140 0.96 -> 0.73 (24), 300 1.01 -> 0.76 (24), 450 1.02
+        // -> 0.79 (20), 700 1.05 -> 0.91 (12), 1000 1.04 -> 0.96 (10); at 1400
+        // and 2048 8 stays (1.15 and 1.41; 1.23 and 1.80 with 10).
+        int rc = TL_EUNSUPPORTED;
+        const RegHull rh = reg_hull(c);
+        if (c->halo_req <= 0)
+            for (int h : {24, 20, 16, 12, 10}) {
+                rc = plan_regdom(c, rh, h, 128);
+                if (rc == TL_OK) return TL_OK;
+                free_resident(c);
+            }
+        rc = plan_regdom(c, rh, c->halo_req > 0 ? c->halo_req : 8, 512);
         if (rc == TL_OK) return TL_OK;
         if (c->kernel == 3) return rc;
         free_resident(c);
