@@ -86,7 +86,7 @@ int launch_nsew(const Geom& g, const uint32_t* cplanes, uint32_t* counts, uint64
 // rows on each side.
 struct ShufflePlan {
     int last;                      // last step of the launch
-    int ctas;
+    int ctas, threads;             // 512 or 768 threads
     int halo;                      // = steps per exchange
     size_t smem_bytes;             // dynamic shared memory per CTA
     const int* stripe_lo;          // device [ctas + 1]
@@ -94,8 +94,8 @@ struct ShufflePlan {
     int* status;                   // device error word: 0 ok, 1 a bounded wait gave up
 };
 size_t shuffle_smem_bytes(int local_rows, int Kw);
-size_t shuffle_static_smem();
-int shuffle_prepare_kernel(size_t smem_bytes, int* blocks_per_sm);
+size_t shuffle_static_smem(int threads);
+int shuffle_prepare_kernel(int threads, size_t smem_bytes, int* blocks_per_sm);
 int launch_shuffle(const ShufflePlan* seg, int nseg, int n, int Kw, size_t total_words, size_t xbuf_words,
                    uint32_t* rows, const DevRng& rng, void* stream);
 // One launch per step over two global buffers of total_words words each; the

@@ -25,7 +25,7 @@
 // them there (word j of Ho then holds the odd edges left of its sites), and
 // the next step of the row, at p = 1, moves them back as it reads.  No
 // word is ever shared by two writers.
-#include "tl_device.cuh"
+#include "tl_words.cuh"
 
 #include <cstdint>
 
@@ -119,7 +119,7 @@ TL_DEV void sh_words(int n, int K, int d, int& lo, int& hi)
 // quarter of the blocks in the disordered region, none in the frozen
 // corners) and uneven (8 +- 2.4 a word), and a draw costs a warp 68 cycles of
 // its scheduler's multiplier, so the warp lists them and its lanes share the
-// draws evenly, two in flight each.  Measured at order 2048: 7.3 ms a sample;
+// draws evenly, two in flight each.  Measured at order 2048 (512 threads): 7.3 ms a sample;
 // 9.5 with every lane drawing for its own word, 8.6 with the lanes drawing
 // for their own words until fewer than 20 have a block left.
 TL_DEV void sh_step_words(const uint32_t* src, uint32_t* dst, int Kw, int n, int K, int Y, int k, bool live,
@@ -139,7 +139,7 @@ TL_DEV void sh_step_words(const uint32_t* src, uint32_t* dst, int Kw, int n, int
         N = V[0];
         S = V[-RW];
         const int w = K - 1 - (Y > n ? Y - n : n - Y);
-        fill = ~(A | B | N | S) & range_mask(k, (n - w - p) >> 1, (n + w - p) >> 1);
+        fill = ~(A | B | N | S) & span_mask(((n - w - p) >> 1) - 32 * k, ((n + w - p) >> 1) - 32 * k);
     }
     uint32_t hor = 0;
     if (__any_sync(0xFFFFFFFFu, fill != 0u)) {
@@ -155,7 +155,13 @@ TL_DEV void sh_step_words(const uint32_t* src, uint32_t* dst, int Kw, int n, int
         const int total = __shfl_sync(0xFFFFFFFFu, off, 31);
         off -= cnt;
         sc.coin[lane] = 0u;
-        for (uint32_t m = fill; m; m &= m - 1) sc.list[off++] = (uint16_t)((lane << 5) | (__ffs(m) - 1));
+        // from the top: one trip to the special-function unit a block (lowest
+        // first takes two, and the list as long as the draws)
+        for (uint32_t m = fill; m;) {
+            const int j = 31 - __clz((int)m);
+            sc.list[off++] = (uint16_t)((lane << 5) | j);
+            m ^= 1u << j;
+        }
         __syncwarp();
         for (int i0 = 0; i0 < total; i0 += 64) {
             // two draws a lane in flight
@@ -203,10 +209,11 @@ TL_DEV uint32_t sh_plain_odd(const uint32_t* row, int Kw, int Y, int K, int k)
 // Bound: the draws (about K^2 / 6 Philox calls in step K) in the middle
 // stripes, and below order 500 the latency of a step (a dependent read, list,
 // draw and write per word, one barrier).
-__global__ void __launch_bounds__(kShufThreads, 1) shuffle_kernel(const ShufParams P)
+template <int NT>
+__global__ void __launch_bounds__(NT, 1) shuffle_kernel(const ShufParams P)
 {
     extern __shared__ uint4 smem4[];
-    __shared__ ShufScratch s_scr[kShufWarps];
+    __shared__ ShufScratch s_scr[NT / 32];
     const int n = P.n, Kw = P.Kw, RW = 4 * Kw, h = P.h;
     const int c = blockIdx.x, C = gridDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int lo = P.stripe_lo[c], hi = P.stripe_lo[c + 1];
@@ -219,7 +226,7 @@ __global__ void __launch_bounds__(kShufThreads, 1) shuffle_kernel(const ShufPara
         // rows of the diamond so far into the first copy; the second is
         // written before it is read, except where the diamond has not been
         const uint4* g = reinterpret_cast<const uint4*>(P.rows0 + (int64_t)slo * RW);
-        for (int i = tid; i < bwords / 4; i += kShufThreads) {
+        for (int i = tid; i < bwords / 4; i += NT) {
             smem4[i] = P.K0 > 1 ? __ldcg(g + i) : make_uint4(0u, 0u, 0u, 0u);
             smem4[bwords / 4 + i] = make_uint4(0u, 0u, 0u, 0u);
         }
@@ -229,28 +236,38 @@ __global__ void __launch_bounds__(kShufThreads, 1) shuffle_kernel(const ShufPara
     const size_t side_words = (size_t)h * RW;
     for (int Kc = P.K0;; Kc += h) {
         const int hc = P.K1 - Kc + 1 < h ? P.K1 - Kc + 1 : h;
+        // for all steps of the cycle: the words of the widest row that its last
+        // step reaches, and the same number of words for every warp and turn
+        // (fewer than 32 spread a small step's draws over more warps)
+        uint32_t nw = 1, per = 4;
+        int klo = 0;
+        {
+            const int K = Kc + hc - 1, ya = slo + 1, yb = shi;
+            const int r0 = ya > n - K + 1 ? ya : n - K + 1, r1 = yb < n + K ? yb : n + K;
+            if (r1 > r0) {
+                const int dmin = r0 > n ? r0 - n : (r1 <= n ? n - (r1 - 1) : 0);
+                int khi;
+                sh_words(n, K, dmin, klo, khi);
+                nw = (uint32_t)(khi - klo + 1);
+                const uint32_t total = (uint32_t)(r1 - r0) * nw;
+                const uint32_t turns = (total + NT - 1) / NT;
+                per = (uint32_t)__float2int_ru(__fdividef((float)total, (float)(turns * (NT / 32))));
+                per = per < 4u ? 4u : (per > 32u ? 32u : per);
+            }
+        }
+        // t / nw: exact, since t < 2^20 keeps the rounding below half of 1 / nw
+        const float inv = __frcp_rn((float)nw);
         for (int i = 1; i <= hc; ++i) {
             const int K = Kc + i - 1;
             // rows whose inputs are exact and that the order-K diamond reaches
             const int ya = bot ? slo + 1 : slo + i, yb = top ? shi : shi - (i - 1);
             const int r0 = ya > n - K + 1 ? ya : n - K + 1, r1 = yb < n + K ? yb : n + K;
             if (r1 <= r0) continue;
-            const int dmin = r0 > n ? r0 - n : (r1 <= n ? n - (r1 - 1) : 0);
-            int klo, khi;
-            sh_words(n, K, dmin, klo, khi);
-            const uint32_t nw = (uint32_t)(khi - klo + 1), total = (uint32_t)(r1 - r0) * nw;
-            // t / nw: exact, since t < 2^20 keeps the rounding below half of 1 / nw
-            const float inv = __frcp_rn((float)nw);
+            const uint32_t total = (uint32_t)(r1 - r0) * nw;
             const uint32_t* src = buf0 + cur * bwords;
             uint32_t* dst = buf0 + (cur ^ 1) * bwords;
             const ShufDraw draw((uint32_t)K, P.rng);
-            // the same number of words for every warp and turn: fewer than 32
-            // spread a small step's draws over more warps
-            const uint32_t turns = (total + kShufThreads - 1) / kShufThreads;
-            uint32_t per = turns <= 1u ? (total + kShufWarps - 1) / kShufWarps
-                                       : (uint32_t)__float2int_ru(__fdividef((float)total, (float)(turns * kShufWarps)));
-            per = per < 4u ? 4u : (per > 32u ? 32u : per);
-            for (uint32_t t0 = (uint32_t)warp * per; t0 < total; t0 += per * kShufWarps) {
+            for (uint32_t t0 = (uint32_t)warp * per; t0 < total; t0 += per * (NT / 32)) {
                 const uint32_t t = t0 + (uint32_t)lane;
                 const uint32_t rr = (uint32_t)(((float)t + 0.5f) * inv);
                 const int Y = r0 + (int)rr, k = klo + (int)(t - rr * nw);
@@ -285,7 +302,7 @@ __global__ void __launch_bounds__(kShufThreads, 1) shuffle_kernel(const ShufPara
         const int npw = (xk1 - xk0 + 1) >> 1, units = 4 * h * npw;
         uint32_t* const st = buf0 + cur * bwords;
         unsigned long long* const mine = P.xbuf + ((size_t)c * 2 + par) * 2 * side_words;
-        for (int u = tid; u < 2 * units; u += kShufThreads) {
+        for (int u = tid; u < 2 * units; u += NT) {
             const int s = u >= units, v = u - (s ? units : 0);
             if (!(s ? xt : xb)) continue;
             const int rp = v / npw, wd = rp * Kw + xk0 + 2 * (v - rp * npw);   // (row, plane) block, word pair
@@ -297,7 +314,7 @@ __global__ void __launch_bounds__(kShufThreads, 1) shuffle_kernel(const ShufPara
         }
         int ok = 1;
         uint64_t t_wait = 0;
-        for (int u = tid; u < 2 * units && ok; u += kShufThreads) {
+        for (int u = tid; u < 2 * units && ok; u += NT) {
             const int s = u >= units, v = u - (s ? units : 0);
             if (!(s ? xt : xb)) continue;
             const int rp = v / npw, wd = rp * Kw + xk0 + 2 * (v - rp * npw);
@@ -332,7 +349,7 @@ __global__ void __launch_bounds__(kShufThreads, 1) shuffle_kernel(const ShufPara
         if (!__syncthreads_and(ok)) return;   // the host reports the timeout
     }
     const uint32_t* st = buf0 + cur * bwords;
-    for (int i = tid; i < (hi - lo) * RW; i += kShufThreads) {
+    for (int i = tid; i < (hi - lo) * RW; i += NT) {
         const int rr = i / RW, rem = i - rr * RW, pl = rem / Kw, k = rem - pl * Kw;
         const uint32_t* row = st + (lo + rr - slo) * RW;
         P.rows0[(int64_t)lo * RW + i] = pl == 1 && P.K1 == n ? sh_plain_odd(row, Kw, lo + rr, n, k) : row[rem];
@@ -378,18 +395,30 @@ static inline cudaStream_t SS_(void* s) { return reinterpret_cast<cudaStream_t>(
 
 size_t shuffle_smem_bytes(int nloc, int Kw) { return (size_t)nloc * 4 * Kw * 4 * 2; }
 
-int shuffle_prepare_kernel(size_t smem_bytes, int* blocks_per_sm)
+static const void* shuffle_pick(int threads)
+{
+    return threads > 512 ? reinterpret_cast<const void*>(&shuffle_kernel<768>)
+                         : reinterpret_cast<const void*>(&shuffle_kernel<512>);
+}
+
+int shuffle_prepare_kernel(int threads, size_t smem_bytes, int* blocks_per_sm)
 {
     *blocks_per_sm = 0;
-    cudaError_t e =
-        cudaFuncSetAttribute(shuffle_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
+    const void* k = shuffle_pick(threads);
+    // one limit for all orders: a context must not lower another's
+    int dev = 0, optin = 0;
+    cudaFuncAttributes fa{};
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k);
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, shuffle_kernel, kShufThreads, smem_bytes);
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, threads, smem_bytes);
     if (e != cudaSuccess) cudaGetLastError();
     return (int)e;
 }
 
-size_t shuffle_static_smem() { return sizeof(ShufScratch) * kShufWarps; }
+size_t shuffle_static_smem(int threads) { return sizeof(ShufScratch) * (size_t)(threads / 32); }
 
 int launch_shuffle(const ShufflePlan* seg, int nseg, int n, int Kw, size_t total_words, size_t xbuf_words,
                    uint32_t* rows, const DevRng& rng, void* stream)
@@ -410,8 +439,8 @@ int launch_shuffle(const ShufflePlan* seg, int nseg, int n, int Kw, size_t total
         P.rows0 = rows + 4 * (size_t)Kw;
         P.status = seg[i].status;
         void* args[] = {&P};
-        e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(&shuffle_kernel), dim3(seg[i].ctas),
-                                        dim3(kShufThreads), args, seg[i].smem_bytes, SS_(stream));
+        e = cudaLaunchCooperativeKernel(shuffle_pick(seg[i].threads), dim3(seg[i].ctas), dim3(seg[i].threads), args,
+                                        seg[i].smem_bytes, SS_(stream));
     }
     return (int)e;
 }
