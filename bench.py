@@ -56,11 +56,14 @@ WORKLOADS = {
                      oracle_sweeps=16, baseline_sweeps=60),
 }
 UNIFORM_T = 1 << 31
-KERNEL_SOURCES = ["paper_1804_07250_gb300/csrc/tl_resident.cu", "paper_1804_07250_gb300/csrc/tl_device.cuh"]
-REG_SOURCES = ["paper_1804_07250_gb300/csrc/tl_regdom.cu", "paper_1804_07250_gb300/csrc/tl_device.cuh"]
+KERNEL_SOURCES = ["paper_1804_07250_gb300/csrc/tl_words_kernel.cuh", "paper_1804_07250_gb300/csrc/tl_words.cuh",
+                  "paper_1804_07250_gb300/csrc/tl_device.cuh"]
+REG_SOURCES = ["paper_1804_07250_gb300/csrc/tl_regdom.cu", "paper_1804_07250_gb300/csrc/tl_words.cuh",
+               "paper_1804_07250_gb300/csrc/tl_device.cuh"]
 # plan kernel -> (ncu kernel name, sources whose hash keys the recorded traffic)
-RESIDENT_KERNELS = {2: ("resident_kernel", KERNEL_SOURCES), 3: ("regdom_kernel", REG_SOURCES)}
-BATCH_SOURCES = ["paper_1804_07250_gb300/csrc/tl_batch.cu", "paper_1804_07250_gb300/csrc/tl_device.cuh"]
+RESIDENT_KERNELS = {2: ("words_kernel", KERNEL_SOURCES), 3: ("regdom_kernel", REG_SOURCES)}
+BATCH_SOURCES = ["paper_1804_07250_gb300/csrc/tl_batch.cu", "paper_1804_07250_gb300/csrc/tl_words.cuh",
+                 "paper_1804_07250_gb300/csrc/tl_device.cuh"]
 
 
 def kernel_hash(sources=None):

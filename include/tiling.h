@@ -364,7 +364,9 @@ int tl_aztec_shuffle(tl_ctx* ctx, int n, uint64_t seed, uint32_t stream_id, uint
  * six-vertex model when a <= c and b <= c, Sec. 1.2.4), so once both chains
  * end in the same configuration every start would have, and that
  * configuration is an exact sample.  Coalescence is detected by equal state
- * hashes and confirmed by comparing the configurations.  The result goes to
+ * hashes and confirmed by comparing the configurations.  The two chains run
+ * at the same time (one launch, or a side stream ordered after `stream`).  The
+ * result goes to
  * `canon_out` (host or device, cap >= canon_bytes) and the T used to
  * *t_used.  Synchronous.  Errors: TL_EINVAL (t0 < 1, tmax < t0 or tmax >
  * 2^31), TL_EBUDGET (no coalescence within tmax sweeps), TL_ENOMEM,
@@ -453,18 +455,23 @@ int tl_read_domino_nsew(tl_chain* c, double* out, size_t cap, void* stream);
 /* Launch plan of a chain.  Every field 0 means "automatic".  Results never
  * depend on the plan: the random numbers are keyed by site and sweep.
  *  kernel:            1 one launch per pass over global memory; 2 the
- *                     shared-memory resident multi-sweep kernel (cooperative
- *                     launch; TL_EUNSUPPORTED if the domain does not fit it);
- *                     3 the register-resident multi-sweep kernel for
+ *                     shared-memory resident multi-sweep kernels (cooperative
+ *                     launch; a thread per 32 sites, for dominoes at t = 2^31
+ *                     a thread per 128; TL_EUNSUPPORTED if the domain does not
+ *                     fit); 3 the register-resident multi-sweep kernel for
  *                     dominoes at t = 2^31 (every 128-site group of a row
  *                     pair held in one thread's registers; the automatic
  *                     choice for such chains when it fits, TL_EUNSUPPORTED
- *                     otherwise).
+ *                     otherwise; with automatic plans, tl_run_sweeps on a
+ *                     domain of at most 1,024 words of sites takes a one-block
+ *                     kernel instead).
  *  sweeps_per_launch: cap on sweeps per resident launch.
  *  halo:              passes between boundary exchanges of the resident
  *                     kernels (1..64; even for kernel 3).
- *  threads:           threads per CTA of the resident kernel (512 or 1024).
- *  npre:              random bit planes generated ahead per group (1..16).
+ *  threads:           threads per CTA of the shared-memory kernels, at most
+ *                     (512 or 1024).
+ *  npre:              random bit planes generated ahead per group (1..16, in
+ *                     fours; six-vertex: 8 or 4 by the build).
  * tl_chain_get_plan also fills the resolved values and ctas / smem_bytes. */
 typedef struct {
     int kernel;
@@ -494,8 +501,9 @@ uint64_t tl_chain_launches(const tl_chain* c);
  * A batch references existing chains (it does not own them) and adds a
  * second device buffer per chain.  tl_batch_run advances every chain by k
  * sweeps: each launch runs R sweeps on every tile (a stripe of tile_rows
- * rows plus a halo of R * passes rows) of every chain, tiles taken largest
- * first from one work list; blocks of `graph_block` sweeps are replayed as a
+ * rows plus a halo of R * passes rows; fewer rows, down to 64, where the
+ * batch has fewer tiles than the GPU has SMs) of every chain, tiles taken
+ * largest first from one work list; blocks of `graph_block` sweeps are replayed as a
  * CUDA graph when `stream` is not the legacy stream.  Every chain ends in
  * exactly the state, sweep count and hash it would reach with
  * tl_run_sweeps alone (random numbers are keyed by site, sweep and the

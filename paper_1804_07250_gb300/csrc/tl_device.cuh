@@ -17,8 +17,9 @@ namespace tl {
 // index and bound of the first) and the access is skipped, so a wrong index
 // shows up as a reported failure (tl_debug_checks) instead of a fault.  In
 // the normal build the checks compile to nothing.  The ids name the check
-// sites: 1xx register kernel, 2xx shared-memory resident kernel, 3xx batch
-// kernel, 4xx per-pass and read-back kernels, 5xx domino shuffling.
+// sites: 1xx register kernel, 2xx shared-memory and word kernels, 3xx batch
+// kernel, 4xx per-pass and read-back kernels, 5xx domino shuffling, 6xx
+// one-block kernel.
 #ifdef TL_DEBUG
 static __device__ unsigned long long tl_dbg_word[4];
 __device__ __noinline__ static bool tl_dbg_fail(long long i, long long n, int id)
@@ -149,18 +150,6 @@ TL_DEV uint32_t slot_colour(const DevRng& rng, uint32_t sweep, uint32_t slot, in
     return (uint32_t)(((uint64_t)o.x * (uint64_t)P) >> 32);
 }
 
-// The first `npre` planes precomputed (shared memory, plane-major with
-// stride `stride` uint4s), the rest computed on the spot.
-struct RndPre {
-    const uint4* pre;
-    int npre, stride;
-    RndPhilox more;
-    TL_DEV uint4 operator()(int k) const { return k < npre ? pre[(size_t)k * stride] : more(k); }
-};
-
-// Same draw with the first `npre` planes read from shared memory: two loops,
-// so the on-the-spot Philox of later planes is never evaluated for the
-// planes that were generated ahead.
 TL_DEV void hb_compare(uint4& lt, uint4& und, uint4 o, uint4 t)
 {
     uint32_t d;
@@ -169,40 +158,6 @@ TL_DEV void hb_compare(uint4& lt, uint4& und, uint4 o, uint4 t)
     d = o.z ^ t.z; lt.z |= und.z & d & t.z; und.z &= ~d;
     d = o.w ^ t.w; lt.w |= und.w & d & t.w; und.w &= ~d;
 }
-template <class TB>
-TL_DEV uint4 heat_bath(uint4 f, int kmax, const RndPre& rnd, const TB& tb)
-{
-    uint4 und = f;
-    uint4 lt = make_uint4(0u, 0u, 0u, 0u);
-    const int kp = (kmax + 1) < rnd.npre ? (kmax + 1) : rnd.npre;
-    int k = 0;
-    // Planes are compared in small blocks whose loads and draws are issued
-    // together: comparing a plane after every site is decided changes
-    // nothing (the undecided mask is then zero), so only the latency of the
-    // chain changes, not the result.
-    for (; k + 4 <= kp; k += 4) {
-        if (!any4(und)) return lt;
-        const uint4 p0 = rnd.pre[(size_t)k * rnd.stride], p1 = rnd.pre[(size_t)(k + 1) * rnd.stride],
-                    p2 = rnd.pre[(size_t)(k + 2) * rnd.stride], p3 = rnd.pre[(size_t)(k + 3) * rnd.stride];
-        hb_compare(lt, und, p0, tb(k));
-        hb_compare(lt, und, p1, tb(k + 1));
-        hb_compare(lt, und, p2, tb(k + 2));
-        hb_compare(lt, und, p3, tb(k + 3));
-    }
-    for (; k < kp; ++k) {
-        if (!any4(und)) return lt;
-        hb_compare(lt, und, rnd.pre[(size_t)k * rnd.stride], tb(k));
-    }
-    for (; k + 1 <= kmax; k += 2) {
-        if (!any4(und)) return lt;
-        const uint4 o0 = rnd.more(k), o1 = rnd.more(k + 1);
-        hb_compare(lt, und, o0, tb(k));
-        hb_compare(lt, und, o1, tb(k + 1));
-    }
-    if (k <= kmax && any4(und)) hb_compare(lt, und, rnd.more(k), tb(k));
-    return lt;
-}
-
 struct TbScalar {
     uint32_t t;
     TL_DEV uint4 operator()(int k) const
@@ -626,24 +581,6 @@ TL_DEV void word_count_sliced(uint32_t w, int64_t i, int64_t plane_words, uint32
         const uint32_t c = *p;
         *p = c ^ carry;
         carry &= c;
-    }
-}
-
-// The same add for four consecutive words (index i a multiple of 4): one
-// 16-byte read and write per counter plane, the four carries rippling
-// together, so a thread's counter update is one chain of dependent accesses
-// per four words instead of per word.
-TL_DEV void word_count_sliced4(uint4 w, int64_t i, int64_t plane_words, uint32_t* cplanes)
-{
-#ifdef TL_DEBUG
-    if (!TL_IN(i + 3, plane_words, 107)) return;
-#endif
-    uint4 carry = w;
-    for (int b = 0; b < 32 && any4(carry); ++b) {
-        uint4* p = reinterpret_cast<uint4*>(cplanes + (int64_t)b * plane_words + i);
-        const uint4 c = *p;
-        *p = x4(c, carry);
-        carry = make_uint4(carry.x & c.x, carry.y & c.y, carry.z & c.z, carry.w & c.w);
     }
 }
 

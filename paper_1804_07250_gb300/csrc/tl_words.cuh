@@ -129,15 +129,6 @@ TL_DEV void anf_products(uint32_t tl, uint32_t tr, uint32_t br, uint32_t bl, uin
     m[14] = m[6] & bl;
     m[15] = m[7] & bl;
 }
-template <int NM>
-TL_DEV uint32_t anf_bit(const uint32_t (&c)[16], const uint32_t (&m)[16])
-{
-    uint32_t t = c[0];
-#pragma unroll
-    for (int i = 1; i < NM; ++i) t ^= c[i] & m[i];
-    return t;
-}
-
 // Bits [lo, hi] of a word, clipped to it (lo, hi any integers).
 TL_DEV uint32_t span_mask(int lo, int hi)
 {
