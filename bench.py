@@ -347,6 +347,8 @@ def run_ours(args):
     peak, peak_kind = peaks()
     achieved = alg_bytes_launch / (k_ms / 1e3) / 1e9
     kname, ksrc = RESIDENT_KERNELS.get(plan["kernel"], ("pass_global_kernel", KERNEL_SOURCES))
+    if kname == "regdom_kernel" and wl["size"][0] <= 127 and not wl["density"]:
+        kname = "small_kernel"  # plain runs of small domains take the one-block kernel
     # the recorded traffic is of the workload's own launches: none for
     # another sweep count or plan
     traffic = recorded_traffic(wl["name"], ksrc, {"kernel": plan["kernel"]}) \
