@@ -197,10 +197,16 @@ __global__ void __launch_bounds__(NT, 512 / NT) batch_kernel(const BatchChain* _
     if (tid == 0) mbar_init(&s_bar, 1);
     __syncthreads();
     uint32_t parity = 0;
-    for (;;) {
+    // a block's first tile is its own index, and a grid that covers the tiles
+    // asks for no second one
+    for (bool own = true;; own = false) {
+        if (!own && (int)gridDim.x >= ntiles) break;
         // a raised status word (a wait that gave up elsewhere, or raised by
         // the host) stops the block before it issues another copy
-        if (tid == 0) s_tile = *(volatile int*)status ? ntiles : (int)atomicAdd(cursor, 1u);
+        if (tid == 0)
+            s_tile = *(volatile int*)status ? ntiles
+                     : own                  ? (int)blockIdx.x
+                                            : (int)(gridDim.x + atomicAdd(cursor, 1u));
         __syncthreads();
         const int t = s_tile;
         __syncthreads();

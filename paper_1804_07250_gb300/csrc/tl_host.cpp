@@ -3079,7 +3079,11 @@ static int batch_launch(tl_batch* b, int r, uint32_t off, int slot, void* stream
 {
     unsigned int* cur = b->d_cursor + (slot % b->ncursor);
     if (!per_chain) {
-        CUDA_TRY(cudaMemsetAsync(cur, 0, 4, SS(stream)));
+        // cursors of the launches to come, cleared together (a clear before each
+        // launch cost 1 us and a gap each); a grid that covers
+        // the tiles reads none
+        if (slot % b->ncursor == 0 && b->grid < b->ntiles)
+            CUDA_TRY(cudaMemsetAsync(b->d_cursor, 0, sizeof(unsigned int) * b->ncursor, SS(stream)));
         const int e = launch_batch(b->d_chains, b->d_tiles_lpt, b->ntiles, r, off, b->src, cur, b->grid, b->run_threads,
                                    b->smem, b->d_status, stream);
         if (e) return fail(TL_ECUDA, "batch kernel: %s", cudaGetErrorString((cudaError_t)e));

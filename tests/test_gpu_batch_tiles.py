@@ -60,3 +60,24 @@ def test_plans_of_other_batches_leave_a_batch_runnable(T):
     small.set_plan(8, 1, -1)
     big.run(8)
     assert len(big.hashes()) == 1
+
+
+@pytest.mark.parametrize("graph_block", [-1, 1026])
+def test_more_launches_than_tile_cursors(T, graph_block):
+    # 1,024 cursors are cleared together: launches beyond them, with more tiles
+    # than blocks so that the blocks read them
+    ctx = T.Context(0)
+    cs = [T.Chain(ctx, T.Domain.aztec(8 + i % 5), seed=3, stream_id=i, th=T.thresholds(scalar=3 << 29))
+          for i in range(320)]
+    b = T.Batch(ctx, cs)
+    b.set_plan(8, 1, graph_block, 256)
+    p = b.plan()
+    assert p["ntiles"] > p["grid"]
+    import torch
+    stream = torch.cuda.Stream()
+    b.run(1030, stream=stream)
+    got = b.hashes(stream=stream)
+    for i in (0, 1, 158, 317, 318, 319):
+        alone = T.Chain(ctx, T.Domain.aztec(8 + i % 5), seed=3, stream_id=i, th=T.thresholds(scalar=3 << 29))
+        alone.run(1030)
+        assert int(got[i]) == alone.state_hash(), i
