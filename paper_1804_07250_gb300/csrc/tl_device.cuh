@@ -544,6 +544,44 @@ TL_DEV void group_update(uint32_t* row, int64_t RW, const Geom& g, int y, int m,
     else sixv_update(row, RW, g.K, g.N, y, m, pass, rnd, th, ttab, ctab, nflip);
 }
 
+// Write-back order of the resident kernels.  A stripe loads its halo rows from
+// the buffer its neighbours write back to.  A launch with an exchange orders
+// the two (a stripe publishes only after it has loaded); one that ends before
+// its first exchange does not, and blocks that start late would load rows
+// already updated.  Such launches mark each stripe loaded with the launch's
+// epoch (thread 0, after a barrier that follows the loads), and a stripe waits
+// for its neighbours' marks before it stores.  The marks are long there by then:
+// the wait costs a read of the L2.
+TL_DEV void stripe_mark_loaded(unsigned int* loaded, unsigned int epoch)
+{
+    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(loaded + blockIdx.x), "r"(epoch) : "memory");
+}
+// Thread 0: false if a wait ran for two seconds, or another block's did.
+TL_DEV bool stripe_neighbours_loaded(const unsigned int* loaded, unsigned int epoch, int* status)
+{
+    const int c = blockIdx.x, C = gridDim.x;
+    uint64_t t_wait = 0;
+    for (int d = -1; d <= 1; d += 2) {
+        if (c + d < 0 || c + d >= C) continue;
+        for (unsigned spin = 1;; ++spin) {
+            unsigned int v;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(loaded + c + d) : "memory");
+            if (v == epoch) break;
+            if ((spin & 15u) == 0u) {
+                uint64_t now;
+                asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+                if (!t_wait) t_wait = now;
+                if (*(volatile int*)status || now - t_wait > 2000000000ull) {
+                    atomicExch(status, 1);
+                    return false;
+                }
+            }
+            __nanosleep(32);
+        }
+    }
+    return true;
+}
+
 // splitmix64 output for state x (Steele, Lea & Flood 2014).
 TL_DEV uint64_t mix64(uint64_t x)
 {

@@ -981,7 +981,7 @@ struct tl_chain {
     ResidentPlan res{};
     int* stripe_d = nullptr;
     unsigned long long* xbuf_d = nullptr;
-    int* status_d = nullptr;
+    int* status_d = nullptr;           // error word, then a word per stripe (ResidentPlan::loaded)
     int threads_req = 0, npre_req = 0;
     int random_order = 0;   // colours of the pass slots drawn per sweep
     uint8_t* colours = nullptr;   // device colours of one resident launch's slots
@@ -1588,12 +1588,12 @@ static int plan_regdom(tl_chain* c, const RegHull& rh, int h, int max_threads)
     if ((rc = dev_alloc(&c->stripe_d, (size_t)C + 1, "stripes")) ||
         (rc = dev_alloc(&c->hull_d, (size_t)npairs, "pair hulls")) ||
         (rc = dev_alloc(&c->xbuf_d, (size_t)C * 4 * h * g.row_words, "exchange buffer")) ||
-        (rc = dev_alloc(&c->status_d, 1, "status")))
+        (rc = dev_alloc(&c->status_d, 1 + (size_t)C, "status")))
         return rc;
     CUDA_TRY(cudaMemcpy(c->stripe_d, rows_lo.data(), sizeof(int) * (C + 1), cudaMemcpyHostToDevice));
     CUDA_TRY(cudaMemcpy(c->hull_d, hull.data(), sizeof(int2) * npairs, cudaMemcpyHostToDevice));
     CUDA_TRY(cudaMemset(c->xbuf_d, 0, sizeof(unsigned long long) * C * 4 * h * g.row_words));
-    CUDA_TRY(cudaMemset(c->status_d, 0, sizeof(int)));
+    CUDA_TRY(cudaMemset(c->status_d, 0, sizeof(int) * (1 + (size_t)C)));
     c->reg.ctas = C;
     c->reg.threads = threads;
     c->reg.halo = h;
@@ -1602,6 +1602,7 @@ static int plan_regdom(tl_chain* c, const RegHull& rh, int h, int max_threads)
     c->reg.hull = c->hull_d;
     c->reg.xbuf = c->xbuf_d;
     c->reg.status = c->status_d;
+    c->reg.loaded = reinterpret_cast<unsigned int*>(c->status_d + 1);
     // the common fields, for reporting and the launch loop
     c->res = ResidentPlan{};
     c->res.ctas = C;
@@ -1613,6 +1614,7 @@ static int plan_regdom(tl_chain* c, const RegHull& rh, int h, int max_threads)
     c->res.stripe_lo = c->stripe_d;
     c->res.xbuf = c->xbuf_d;
     c->res.status = c->status_d;
+    c->res.loaded = reinterpret_cast<unsigned int*>(c->status_d + 1);
     c->use_reg = true;
     c->res_ready = true;
     // domains of at most 1,024 words of sites: plain runs take the one-block
@@ -1640,16 +1642,17 @@ static int alloc_resident(tl_chain* c, const std::vector<int>& lo, int h)
     int rc;
     if ((rc = dev_alloc(&c->stripe_d, (size_t)C + 1, "stripes")) ||
         (rc = dev_alloc(&c->xbuf_d, (size_t)C * 4 * h * g.row_words, "exchange buffer")) ||
-        (rc = dev_alloc(&c->status_d, 1, "status")))
+        (rc = dev_alloc(&c->status_d, 1 + (size_t)C, "status")))
         return rc;
     CUDA_TRY(cudaMemcpy(c->stripe_d, lo.data(), sizeof(int) * (C + 1), cudaMemcpyHostToDevice));
     CUDA_TRY(cudaMemset(c->xbuf_d, 0, sizeof(unsigned long long) * C * 4 * h * g.row_words));
-    CUDA_TRY(cudaMemset(c->status_d, 0, sizeof(int)));
+    CUDA_TRY(cudaMemset(c->status_d, 0, sizeof(int) * (1 + (size_t)C)));
     c->res.ctas = C;
     c->res.halo = h;
     c->res.stripe_lo = c->stripe_d;
     c->res.xbuf = c->xbuf_d;
     c->res.status = c->status_d;
+    c->res.loaded = reinterpret_cast<unsigned int*>(c->status_d + 1);
     c->res_ready = true;
     return TL_OK;
 }

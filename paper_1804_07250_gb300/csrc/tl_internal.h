@@ -137,6 +137,7 @@ struct ResidentPlan {
     const int* stripe_lo;          // device [ctas + 1]
     unsigned long long* xbuf;      // device [ctas][2][2][halo][row_words] tagged words
     int* status;                   // device error word: 0 ok, 1 a bounded wait gave up
+    unsigned int* loaded;          // device [ctas], zeroed with the plan
 };
 
 // Shared-memory attribute and occupancy: blocks that fit on one SM (0 if none).
@@ -175,6 +176,7 @@ struct RegPlan {
     const int2* hull;              // device [pairs]
     unsigned long long* xbuf;      // device [ctas][2][2][halo / 2][16][Kg][2]
     int* status;
+    unsigned int* loaded;          // device [ctas], zeroed with the plan
 };
 size_t regdom_smem_bytes(int threads, int max_local_pairs);
 int regdom_prepare(int threads, size_t smem_bytes, int* blocks_per_sm);

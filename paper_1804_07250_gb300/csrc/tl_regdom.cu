@@ -45,6 +45,7 @@ struct RegParams {
     DevRng rng;
     unsigned long long* xbuf;   // [C][2][2][halo / 2][16][Kg][2] tagged words
     int* status;
+    unsigned int* loaded;       // [C] epoch of the last launch without an exchange that a stripe has loaded in
     unsigned long long* ring;
     uint32_t* counts;
     uint64_t burn;
@@ -308,6 +309,11 @@ __global__ void __launch_bounds__(NT, 1) regdom_kernel(const RegParams P)
     const uint32_t grp1 = grp0 + (uint32_t)Kg;
 
     const uint64_t total = (uint64_t)P.nsweeps * 2;
+    if (gridDim.x > 1 && (uint64_t)P.nsweeps * 2 <= (uint64_t)P.halo) {
+        __threadfence();   // the loads into registers
+        __syncthreads();
+        if (tid == 0) stripe_mark_loaded(P.loaded, P.epoch);
+    }
     const size_t side_words = (size_t)(h >> 1) * 32 * Kg;   // u64 per side
     uint64_t done = 0;
     uint32_t nflip = 0;   // accepted flips of this thread's owned sites
@@ -581,6 +587,9 @@ __global__ void __launch_bounds__(NT, 1) regdom_kernel(const RegParams P)
         }
         ++cyc;
     }
+    if (gridDim.x > 1 && (uint64_t)P.nsweeps * 2 <= (uint64_t)P.halo &&
+        !__syncthreads_and(tid != 0 || stripe_neighbours_loaded(P.loaded, P.epoch, P.status)))
+        return;
     if (COUNT && nflip) atomicAdd(P.flips, (unsigned long long)nflip);
     if (owned && inb) {
         uint32_t* b0 = P.rows0 + (int64_t)y0 * RW + k0;
@@ -657,6 +666,7 @@ int launch_regdom(const Geom& g, uint32_t* rows, const RegPlan& plan, uint32_t s
     P.rng = rng;
     P.xbuf = plan.xbuf;
     P.status = plan.status;
+    P.loaded = plan.loaded;
     P.ring = ring;
     P.counts = counts;
     P.burn = burn;

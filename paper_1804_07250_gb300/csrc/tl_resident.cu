@@ -38,6 +38,7 @@ struct ResParams {
     const int2* grange;
     unsigned long long* xbuf;   // tagged exchange words
     int* status;
+    unsigned int* loaded;       // [C] epoch of the last launch without an exchange that a stripe has loaded in
     unsigned long long* ring;
     uint32_t* counts;           // bit-sliced density counter planes, or nullptr
     uint64_t burn;
@@ -176,6 +177,7 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResParams P)
 
     const int passes = g.passes;
     const uint64_t total = (uint64_t)P.nsweeps * passes;
+    if (total <= (uint64_t)h && tid == 0) stripe_mark_loaded(P.loaded, P.epoch);
     const size_t side_words = (size_t)h * RW;
 #ifdef TL_DEBUG
     const int cap = P.cap_cycle;
@@ -405,6 +407,7 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResParams P)
         hc = hc_next;
         ++cyc;
     }
+    if (cyc == 0 && !__syncthreads_and(tid != 0 || stripe_neighbours_loaded(P.loaded, P.epoch, P.status))) return;
     copy_rows_to_global(P.rows0 + (int64_t)lo * RW, srow0 + (int64_t)lo * RW, (int64_t)(hi - lo) * RW, tid, NT);
     if (P.flips && nflip) atomicAdd(P.flips, (unsigned long long)nflip);
 }
@@ -449,6 +452,7 @@ int launch_resident(const Geom& g, uint32_t* rows, const ResidentPlan& plan, uin
     P.grange = grange;
     P.xbuf = plan.xbuf;
     P.status = plan.status;
+    P.loaded = plan.loaded;
     P.ring = ring;
     P.counts = counts;
     P.burn = burn;

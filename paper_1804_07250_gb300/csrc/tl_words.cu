@@ -63,6 +63,7 @@ int launch_words(const Geom& g, uint32_t* rows, const ResidentPlan& plan, uint32
     P.grange = grange;
     P.xbuf = plan.xbuf;
     P.status = plan.status;
+    P.loaded = plan.loaded;
     P.ring = ring;
     P.counts = counts;
     P.burn = burn;

@@ -50,6 +50,7 @@ struct WordParams {
     const int2* grange;
     unsigned long long* xbuf;   // [C][2][2][halo row_words] tagged exchange words
     int* status;
+    unsigned int* loaded;       // [C] epoch of the last launch without an exchange that a stripe has loaded in
     unsigned long long* ring;
     uint32_t* counts;           // bit-sliced density counter planes, or nullptr
     uint64_t burn;
@@ -202,6 +203,7 @@ __global__ void __launch_bounds__(MAXT, 1) words_kernel(const __grid_constant__ 
 
     const int passes = g.passes;
     const uint64_t total = (uint64_t)P.nsweeps * passes;
+    if (C > 1 && total <= (uint64_t)h && tid == 0) stripe_mark_loaded(P.loaded, P.epoch);
     // the next density sample: sweeps s (counted after the sweep, 1-based)
     // with s >= burn and (s - burn) % stride == 0, tracked incrementally
     uint64_t next_sample = ~0ull;
@@ -542,6 +544,9 @@ __global__ void __launch_bounds__(MAXT, 1) words_kernel(const __grid_constant__ 
         if (!__syncthreads_and(ok)) return;   // the state is undefined; the host reports TL_ETIMEOUT
         ++cyc;
     }
+    if (gridDim.x > 1 && cyc == 0 &&
+        !__syncthreads_and(tid != 0 || stripe_neighbours_loaded(P.loaded, P.epoch, P.status)))
+        return;
     {
         uint4* d = reinterpret_cast<uint4*>(P.rows0 + (int64_t)lo * RW);
         const uint4* s = smem4 + (size_t)(lo - slo) * (RW / 4);
