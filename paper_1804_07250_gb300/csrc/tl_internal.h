@@ -140,6 +140,11 @@ struct ResidentPlan {
     unsigned int* loaded;          // device [ctas], zeroed with the plan
 };
 
+// Dynamic shared memory up to what the device has left beside the kernel's
+// static: the limit belongs to the kernel, not to a plan, so a plan that set
+// only its own need would take it from the chains planned before.
+int set_smem_limit(const void* kernel);
+
 // Shared-memory attribute and occupancy: blocks that fit on one SM (0 if none).
 int resident_prepare(int threads, size_t smem_bytes, int* blocks_per_sm);
 

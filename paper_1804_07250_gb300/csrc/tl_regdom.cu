@@ -636,15 +636,9 @@ int regdom_prepare(int threads, size_t smem_bytes, int* blocks_per_sm)
 {
     *blocks_per_sm = 0;
     const void* k = reg_pick(threads, false, false);
-    cudaError_t e = cudaSuccess;
-    for (int v = 0; v < 4 && e == cudaSuccess; ++v)
-        e = cudaFuncSetAttribute(reg_pick(threads, (v & 1) != 0, (v & 2) != 0),
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        return (int)e;
-    }
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, threads, smem_bytes);
+    for (int v = 0; v < 4; ++v)
+        if (const int e = set_smem_limit(reg_pick(threads, (v & 1) != 0, (v & 2) != 0))) return e;
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, threads, smem_bytes);
     if (e != cudaSuccess) cudaGetLastError();
     return (int)e;
 }
