@@ -456,8 +456,9 @@ int tl_read_domino_nsew(tl_chain* c, double* out, size_t cap, void* stream);
  * depend on the plan: the random numbers are keyed by site and sweep.
  *  kernel:            1 one launch per pass over global memory; 2 the
  *                     shared-memory resident multi-sweep kernels (cooperative
- *                     launch; a thread per 32 sites, for dominoes at t = 2^31
- *                     a thread per 128; TL_EUNSUPPORTED if the domain does not
+ *                     launch; a thread per 32 sites, or per 128 for dominoes at
+ *                     t = 2^31 and for large stripes with one threshold of
+ *                     few bits; TL_EUNSUPPORTED if the domain does not
  *                     fit); 3 the register-resident multi-sweep kernel for
  *                     dominoes at t = 2^31 (every 128-site group of a row
  *                     pair held in one thread's registers; the automatic

@@ -1677,22 +1677,28 @@ static std::vector<int> even_stripes(const std::vector<double>& pre, int C, int 
     return lo;
 }
 
-// Dominoes at t = 2^31 on the shared-memory kernel with the single-plane
-// update: 1024 threads and 6 passes per exchange run fastest on the Aztec
-// diamond of order 2048.
-static int plan_fast(tl_chain* c)
+// Kernels of a thread per 128-site group (tl_resident.cu).  `fast`: dominoes at
+// t = 2^31 with the single-plane update, 1024 threads and 6 passes per exchange
+// (fastest on the Aztec diamond of order 2048).  Else 512 threads, 8 (dominoes)
+// or 6 (lozenges) passes.
+static int plan_groups(tl_chain* c, bool fast)
 {
     const Geom& g = c->g;
     const tl_domain& d = c->dom_copy;
-    const int h = c->halo_req > 0 ? c->halo_req : 6;
-    const int threads = c->threads_req > 0 ? c->threads_req : 1024;
+    const bool half = fast_candidate(c);
+    const int h = c->halo_req > 0 ? c->halo_req : half || g.lattice == LAT_LOZENGE ? 6 : 8;
+    const int threads = c->threads_req > 0 && g.lattice == LAT_DOMINO ? c->threads_req : half ? 1024 : 512;
+    const int planes = c->th.kind == THR_SITE ? 32 : std::max(1, c->th.kmax + 1);
+    const int npre = fast ? 1 : c->npre_req > 0 ? c->npre_req : std::min(8, planes);
     std::vector<int> pre(g.H + 1, 0);
     std::vector<double> w(g.H + 1, 0.0);
     for (int y = 0; y < g.H; ++y) {
-        // and the group left of them, which writes the word they share
+        // fast: and the group left of them, which writes the word they share
+        // (it counts in the weights of both forms: rows of few groups cost
+        // shared memory, and the outer stripes have many of them)
         const int2 gr = d.grange[y];
         const int act = gr.y > gr.x ? gr.y - std::max(0, gr.x - 1) : 0;
-        pre[y + 1] = pre[y] + act;
+        pre[y + 1] = pre[y] + (fast || act == 0 ? act : gr.y - gr.x);
         w[y + 1] = w[y] + 0.1 + act;
     }
     auto items_in = [&](int a, int b) {
@@ -1720,23 +1726,37 @@ static int plan_fast(tl_chain* c)
         }
         cap_cycle = std::max(cap_cycle, cyc);
     }
-    const size_t smem = (size_t)max_nloc * g.row_words * 4 + (size_t)cap_cycle * 16 + (size_t)cap_items * 12 +
-                        (size_t)(max_nloc + 1) * 4 + 24;
+    size_t smem = (size_t)max_nloc * g.row_words * 4 + (size_t)npre * cap_cycle * 16 + (size_t)cap_items * 4 +
+                  (size_t)(max_nloc + 1) * 4 + 16;
+    if (fast) smem += (size_t)cap_items * 8 + 8;
     int bps = 0;
-    if (max_pass > fast_capacity(threads) || (long)smem > (long)c->ctx->smem_optin ||
-        resident_prepare(threads, smem, &bps) != 0 || bps < 1 || C > bps * c->ctx->sms) {
-        c->res_why = "a pass does not fit the single-plane update";
+    if ((fast && max_pass > fast_capacity(threads)) || (long)smem > (long)c->ctx->smem_optin ||
+        resident_prepare(g, c->th.kind, threads, fast, smem, &bps) != 0 || bps < 1 || C > bps * c->ctx->sms) {
+        c->res_why = fast ? "a pass does not fit the single-plane update" : "stripe does not fit in shared memory";
         return TL_EUNSUPPORTED;
     }
     c->res = ResidentPlan{};
     c->res.threads = threads;
-    c->res.slots = 1;
-    c->res.npre = 1;
+    c->res.npre = npre;
     c->res.cap_items = cap_items;
     c->res.cap_cycle = cap_cycle;
-    c->res.fast = true;
+    c->res.fast = fast;
     c->res.smem_bytes = smem;
     return alloc_resident(c, lo, h);
+}
+
+// Words a stripe of the word kernel holds from which the group form is the
+// better one (tl_resident.cu has the figures).  The word kernel's cost goes by
+// blocks of four planes, the group form's by planes.
+static int group_form_from(const tl_chain* c)
+{
+    const bool dom = c->g.lattice == LAT_DOMINO;
+    if (c->th.kind == THR_SITE && c->g.lattice == LAT_LOZENGE) return 801;
+    if (c->th.kind != THR_SCALAR || c->g.lattice == LAT_SIXV) return 1 << 30;
+    const int planes = c->th.kmax + 1;
+    if (planes > 6) return 1 << 30;
+    if (planes == 5 || planes <= (dom ? 2 : 1)) return 513;
+    return planes == 6 ? 881 : dom ? 641 : 801;
 }
 
 // The word kernel: stripes, passes per exchange, threads and words per thread.
@@ -1797,6 +1817,7 @@ static int plan_words(tl_chain* c)
     cand.push_back(Cand{model(pre[U], 0, 0), c->halo_req > 0 ? c->halo_req : 60, 1});
     std::stable_sort(cand.begin(), cand.end(), [](const Cand& a, const Cand& b) { return a.t < b.t; });
     c->res_why = "stripe does not fit in shared memory";
+    bool groups_tried = false;
     for (const Cand& cd : cand) {
         const int h = cd.h, C = cd.C;
         const std::vector<int> lo = even_stripes(w, C, h, step);
@@ -1810,6 +1831,11 @@ static int plan_words(tl_chain* c)
         const int lanes = std::max(32, 4 * items);
         const size_t smem = words_smem_bytes(g, max_nloc);
         if (smem > (size_t)c->ctx->smem_optin || lanes > 4096) continue;
+        if (!groups_tried && lanes >= group_form_from(c)) {
+            groups_tried = true;
+            if (plan_groups(c, false) == TL_OK) return TL_OK;
+            free_resident(c);
+        }
         // `threads` asks for at most that many; results never depend on it
         const int cap = c->threads_req == 512 && lanes <= 2048 ? 512 : 1024;
         int slots = 1;
@@ -1830,6 +1856,8 @@ static int plan_words(tl_chain* c)
         c->res.smem_bytes = smem;
         return alloc_resident(c, lo, h);
     }
+    // stripes of more words than the word kernel takes
+    if (c->th.kind == THR_SCALAR && !sixv && !groups_tried) return plan_groups(c, false);
     return TL_EUNSUPPORTED;
 }
 
@@ -1876,7 +1904,7 @@ static int plan_resident(tl_chain* c)
         return TL_EUNSUPPORTED;
     }
     if (fast_candidate(c)) {
-        if (plan_fast(c) == TL_OK) return TL_OK;
+        if (plan_groups(c, true) == TL_OK) return TL_OK;
         free_resident(c);
     }
     return plan_words(c);
@@ -1947,8 +1975,8 @@ static int run_resident(tl_chain* c, uint64_t k, unsigned long long* ring, void*
                                 ring ? ring + done : nullptr, dens ? c->cplanes : nullptr, c->burn,
                                 dens ? c->stride : 0, c->random_order ? c->colours : nullptr,
                                 c->count_flips ? c->flips_d : nullptr, stream)
-            : c->res.fast
-                ? launch_resident(c->g, c->rows, c->res, (uint32_t)c->sweep, (uint32_t)n, c->rng, c->grange,
+            : c->res.slots == 0
+                ? launch_resident(c->g, c->rows, c->res, (uint32_t)c->sweep, (uint32_t)n, c->rng, c->th, c->grange,
                                   ++c->epoch, ring ? ring + done : nullptr, dens ? c->cplanes : nullptr, c->burn,
                                   dens ? c->stride : 0, c->random_order ? c->colours : nullptr,
                                   c->count_flips ? c->flips_d : nullptr, stream)

@@ -127,12 +127,12 @@ int launch_height_noalloc(const Geom& g, const uint32_t* rows, const int* seg, i
 struct ResidentPlan {
     int ctas;                      // cooperative grid size
     int threads;                   // threads per CTA
-    int slots;                     // words per thread (the word kernel)
+    int slots;                     // words per thread (the word kernel; 0: a thread per group, tl_resident.cu)
     int halo;                      // passes per exchange cycle (= halo rows per side)
     int npre;                      // random planes generated ahead per group
-    int cap_items;                 // `fast`: item-table capacity per CTA
-    int cap_cycle;                 // `fast`: groups touched per cycle, per CTA (upper bound)
-    bool fast;                     // dominoes at t = 2^31: branch-free single-plane update (tl_resident.cu)
+    int cap_items;                 // slots 0: item-table capacity per CTA
+    int cap_cycle;                 // slots 0: groups touched per cycle, per CTA (upper bound)
+    bool fast;                     // dominoes at t = 2^31: branch-free single-plane update
     size_t smem_bytes;             // dynamic shared memory per CTA
     const int* stripe_lo;          // device [ctas + 1]
     unsigned long long* xbuf;      // device [ctas][2][2][halo][row_words] tagged words
@@ -146,13 +146,13 @@ struct ResidentPlan {
 int set_smem_limit(const void* kernel);
 
 // Shared-memory attribute and occupancy: blocks that fit on one SM (0 if none).
-int resident_prepare(int threads, size_t smem_bytes, int* blocks_per_sm);
+int resident_prepare(const Geom& g, int thr_kind, int threads, bool fast, size_t smem_bytes, int* blocks_per_sm);
 
 // ring: per-sweep hashes (nullptr = off; must be zeroed).  counts: density
 // counters sampled after every sweep s with s + 1 >= burn and
 // (s + 1 - burn) % stride == 0 (nullptr or stride 0 = off).
 int launch_resident(const Geom& g, uint32_t* rows, const ResidentPlan& plan, uint32_t sweep0,
-                    uint32_t nsweeps, const DevRng& rng, const int2* grange,
+                    uint32_t nsweeps, const DevRng& rng, const ThrView& th, const int2* grange,
                     unsigned int epoch, unsigned long long* ring, uint32_t* counts, uint64_t burn,
                     uint32_t stride, const uint8_t* colours, unsigned long long* flips, void* stream);
 

@@ -1,6 +1,7 @@
-// Shared-memory resident multi-sweep kernel for dominoes at t = 2^31 whose
-// stripes do not fit the register-resident kernel, or when a plan asks for it
-// (cooperative launch).
+// Shared-memory resident multi-sweep kernels with a thread per 128-site group
+// (cooperative launch), in two forms: FAST for dominoes at t = 2^31 when a plan
+// asks for it, and the group form for dominoes and lozenges with one threshold
+// of few set bits, and lozenges with one a site, and many groups a stripe.
 //
 // Each CTA keeps a horizontal stripe of the packed state plus `halo` rows
 // above and below it in shared memory for a whole launch.  A pass updates
@@ -11,8 +12,21 @@
 // refreshes its halos from its two neighbours.
 //
 // Half the warps update the current pass, from an item table of the active
-// 128-site groups, while the other half generate the random plane of the
-// next: at t = 2^31 one plane decides every site.
+// 128-site groups, while the other half generate the random planes of the
+// next: one where the threshold has one bit (t = 2^31), else `npre`.
+//
+// Where the group form is the better one: the word kernel (tl_words_kernel.cuh)
+// draws four planes at a time whether the threshold has one bit or four, and
+// above 128 groups a stripe it runs with 80, then 64 registers a thread and
+// then with several words a thread.  The bound here is the issue of the updates
+// and draws, so the work per group decides.
+// us a sweep, word kernel -> this one: squares at t = 1/4 1200 1.86 -> 1.90, 1400
+// 2.20 -> 1.96, 2000 2.55 -> 2.17, 2800 4.44 -> 3.10, 4000 9.93 -> 4.49, and at
+// t = 1/2 6000 (a launch per pass) 12.4 -> 7.39; hexagons at t = 1/2 1100 3.29 ->
+// 3.37, 1200 3.90 -> 3.50, 1400 4.27 -> 3.56, 2000 7.26 -> 5.38, 2800 13.5 -> 7.05;
+// squares 2000 by planes 2 2.55 -> 2.17, 3 2.54 -> 2.41, 4 2.54 -> 2.54, 5 3.18 ->
+// 2.84, 6 3.19 -> 3.18, 7 3.21 -> 3.46, 32 3.67 -> 4.71; hexagons with a threshold
+// a site 1400 5.95 -> 5.66.
 //
 // Exchange: every boundary word travels with a 32-bit tag (launch epoch,
 // cycle) in one 64-bit store; the reader polls the 64-bit words until the
@@ -29,12 +43,13 @@ struct ResParams {
     uint32_t* rows0;            // global row 0 (after the pad row)
     Geom g;
     const int* stripe_lo;
-    int halo;
+    int halo, npre;
     const uint8_t* colours;     // random pass order: colour of every slot of the launch, else nullptr
     int cap_items;              // item-table capacity per CTA
     int cap_cycle;              // random-plane buffer capacity (groups per cycle)
     uint32_t sweep0, nsweeps;
     DevRng rng;
+    ThrView th;
     const int2* grange;
     unsigned long long* xbuf;   // tagged exchange words
     int* status;
@@ -103,9 +118,50 @@ TL_DEV PassRange pass_range(const Geom& g, int i, int slo, int shi, bool bot, bo
     return PassRange{off[a - slo], off[b - slo]};
 }
 
-// Branch-free, atomic-free group update; every updater thread handles at most
-// two groups per pass.
-template <int NT>
+// The first `npre` planes from shared memory (plane-major, `stride` uint4s
+// apart), the rest computed on the spot.
+struct RndPre {
+    const uint4* pre;
+    int npre, stride;
+    RndPhilox more;
+};
+// Two loops, so that the Philox of later planes is never evaluated for the
+// planes generated ahead.
+template <class TB>
+TL_DEV uint4 heat_bath(uint4 f, int kmax, const RndPre& rnd, const TB& tb)
+{
+    uint4 und = f;
+    uint4 lt = make_uint4(0u, 0u, 0u, 0u);
+    const int kp = (kmax + 1) < rnd.npre ? (kmax + 1) : rnd.npre;
+    int k = 0;
+    // planes compared four at a time, their loads issued together (a plane
+    // compared after every site is decided changes nothing)
+    for (; k + 4 <= kp; k += 4) {
+        if (!any4(und)) return lt;
+        const uint4 p0 = rnd.pre[(size_t)k * rnd.stride], p1 = rnd.pre[(size_t)(k + 1) * rnd.stride],
+                    p2 = rnd.pre[(size_t)(k + 2) * rnd.stride], p3 = rnd.pre[(size_t)(k + 3) * rnd.stride];
+        hb_compare(lt, und, p0, tb(k));
+        hb_compare(lt, und, p1, tb(k + 1));
+        hb_compare(lt, und, p2, tb(k + 2));
+        hb_compare(lt, und, p3, tb(k + 3));
+    }
+    for (; k < kp; ++k) {
+        if (!any4(und)) return lt;
+        hb_compare(lt, und, rnd.pre[(size_t)k * rnd.stride], tb(k));
+    }
+    for (; k + 1 <= kmax; k += 2) {
+        if (!any4(und)) return lt;
+        const uint4 o0 = rnd.more(k), o1 = rnd.more(k + 1);
+        hb_compare(lt, und, o0, tb(k));
+        hb_compare(lt, und, o1, tb(k + 1));
+    }
+    if (k <= kmax && any4(und)) hb_compare(lt, und, rnd.more(k), tb(k));
+    return lt;
+}
+
+// FAST: dominoes at t = 2^31 with the branch-free, atomic-free group update;
+// every updater thread handles at most two groups per pass.
+template <int LAT, int TK, int NT, bool FAST>
 __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResParams P)
 {
     extern __shared__ uint4 smem4[];
@@ -129,18 +185,18 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResParams P)
     uint32_t* sm = reinterpret_cast<uint32_t*>(smem4);
     uint32_t* srow0 = sm - (int64_t)slo * RW;   // srow0 + y * RW is global row y
     uint4* rbuf = reinterpret_cast<uint4*>(sm + (int64_t)nloc * RW);
-    uint32_t* items = reinterpret_cast<uint32_t*>(rbuf + P.cap_cycle);
+    uint32_t* items = reinterpret_cast<uint32_t*>(rbuf + (size_t)P.npre * P.cap_cycle);
     int* off = reinterpret_cast<int*>(items + P.cap_items);
-    // 8-byte aligned after the offsets
+    // FAST only: 8-byte aligned after the offsets
     uint2* fitems = reinterpret_cast<uint2*>((reinterpret_cast<uintptr_t>(off + nloc + 1) + 7) & ~(uintptr_t)7);
 
     copy_rows_from_global(sm, P.rows0 + (int64_t)slo * RW, (int64_t)nloc * RW, tid, NT);
 
-    // item table: active groups of each local row and the one left of them
-    // (it writes the word they share), prefix offsets
+    // item table: active groups of each local row (FAST: and the one left of
+    // them, which writes the word they share), prefix offsets
     auto row_groups = [&](int y) {
         int2 gr = P.grange[y];
-        if (gr.y > gr.x && gr.x > 0) --gr.x;
+        if (FAST && gr.y > gr.x && gr.x > 0) --gr.x;
         return gr;
     };
     for (int r = tid; r < nloc; r += NT) {
@@ -168,8 +224,9 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResParams P)
             if (!TL_IN(o, P.cap_items, 201)) break;
 #endif
             // word offset of (row y, plane 0, word 4m) and whether m+1 follows in this row
-            fitems[o] = make_uint2((uint32_t)((int64_t)r * RW + 4 * m),
-                                   (uint32_t)y | ((uint32_t)m << 16) | (m + 1 < gr.y ? 0x80000000u : 0u));
+            if (FAST)
+                fitems[o] = make_uint2((uint32_t)((int64_t)r * RW + 4 * m),
+                                       (uint32_t)y | ((uint32_t)m << 16) | (m + 1 < gr.y ? 0x80000000u : 0u));
             items[o++] = ((uint32_t)r << 8) | (uint32_t)m;
         }
     }
@@ -179,9 +236,7 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResParams P)
     const uint64_t total = (uint64_t)P.nsweeps * passes;
     if (total <= (uint64_t)h && tid == 0) stripe_mark_loaded(P.loaded, P.epoch);
     const size_t side_words = (size_t)h * RW;
-#ifdef TL_DEBUG
     const int cap = P.cap_cycle;
-#endif
     // warp roles: the first half updates the current pass, the second half
     // generates the random planes of the next pass
     constexpr int HALF = NT / 2;
@@ -218,7 +273,9 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResParams P)
         s_next_sweep = sweep;
         s_next_pass = pass;
     };
-    // random plane of one pass (generator warps)
+    // random planes of one pass (generator warps), of a group four at a time:
+    // independent Philox chains in flight together (all four even where fewer
+    // are kept: guarded they take registers the update needs)
     auto gen = [&](int i) {
         const int4 e = s_ptab[i];
         const uint32_t sweep = s_psweep[i], pass = (uint32_t)e.w & 255u;   // slot
@@ -228,8 +285,20 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResParams P)
 #endif
             const uint32_t item = items[e.x + it];
             const int y = slo + (int)(item >> 8), m = (int)(item & 255u);
-            rbuf[e.z + it] =
-                philox10((uint32_t)(y * g.Kg + m), sweep, pass, P.rng.stream, P.rng.k0, P.rng.k1);
+            const uint32_t grp = (uint32_t)(y * g.Kg + m);
+            if constexpr (FAST) {
+                rbuf[e.z + it] = philox10(grp, sweep, pass, P.rng.stream, P.rng.k0, P.rng.k1);
+            } else {
+                for (int k0 = 0; k0 < P.npre; k0 += 4) {
+                    uint4 o[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        o[q] = philox10(grp, sweep, ((uint32_t)(k0 + q) << 16) | pass, P.rng.stream, P.rng.k0, P.rng.k1);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        if (k0 + q < P.npre) rbuf[(size_t)(k0 + q) * cap + e.z + it] = o[q];
+                }
+            }
         }
     };
     // the first cycle's table and random planes; later cycles get theirs from
@@ -244,7 +313,7 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResParams P)
         for (int i = 0; i < hc; ++i) {
             const int4 e = s_ptab[i];
             const uint32_t slot = (uint32_t)e.w & 255u, pass = (uint32_t)e.w >> 8, sweep = s_psweep[i];
-            if (upd_role) {
+            if (FAST && upd_role) {
                 // read and decide every group of the pass, then store: groups
                 // read their neighbours' boundary words
                 constexpr int MAXI = NT >= 1024 ? 1 : 2;
@@ -278,6 +347,20 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResParams P)
 #pragma unroll
                 for (int q = 0; q < MAXI; ++q)
                     if (has[q]) domino_fast_store(r[q]);
+            } else if (upd_role) {
+                for (int it = rtid; it < e.y; it += HALF) {
+#ifdef TL_DEBUG
+                    if (!TL_IN(e.x + it, P.cap_items, 207) || !TL_IN(e.z + it, cap, 203)) continue;
+                    // the update reads rows y - 1 and y of the local rows
+                    if (!TL_IN((int)(items[e.x + it] >> 8) - 1, nloc - 1, 208)) continue;
+#endif
+                    const uint32_t item = items[e.x + it];
+                    const int y = slo + (int)(item >> 8), m = (int)(item & 255u);
+                    const RndPre rnd{rbuf + e.z + it, P.npre, cap,
+                                     RndPhilox{(uint32_t)(y * g.Kg + m), sweep, slot, P.rng}};
+                    group_update<LAT, TK>(srow0 + (int64_t)y * RW, RW, g, y, m, pass, rnd, P.th, nullptr,
+                                                  nullptr, (P.flips && y >= lo && y < hi) ? &nflip : nullptr);
+                }
             } else if (i + 1 < hc) {
                 gen(i + 1);
             }
@@ -412,10 +495,16 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResParams P)
     if (P.flips && nflip) atomicAdd(P.flips, (unsigned long long)nflip);
 }
 
-static const void* pick(int threads)
+static const void* pick(int lattice, int tk, int threads, bool fast)
 {
-    return threads > 512 ? reinterpret_cast<const void*>(&resident_kernel<1024>)
-                         : reinterpret_cast<const void*>(&resident_kernel<512>);
+    if (fast)
+        return threads > 512 ? reinterpret_cast<const void*>(&resident_kernel<LAT_DOMINO, THR_SCALAR, 1024, true>)
+                             : reinterpret_cast<const void*>(&resident_kernel<LAT_DOMINO, THR_SCALAR, 512, true>);
+    if (lattice == LAT_LOZENGE)
+        return tk == THR_SITE ? reinterpret_cast<const void*>(&resident_kernel<LAT_LOZENGE, THR_SITE, 512, false>)
+                              : reinterpret_cast<const void*>(&resident_kernel<LAT_LOZENGE, THR_SCALAR, 512, false>);
+    return threads > 512 ? reinterpret_cast<const void*>(&resident_kernel<LAT_DOMINO, THR_SCALAR, 1024, false>)
+                         : reinterpret_cast<const void*>(&resident_kernel<LAT_DOMINO, THR_SCALAR, 512, false>);
 }
 
 int set_smem_limit(const void* kernel)
@@ -431,10 +520,10 @@ int set_smem_limit(const void* kernel)
     return (int)e;
 }
 
-int resident_prepare(int threads, size_t smem_bytes, int* blocks_per_sm)
+int resident_prepare(const Geom& g, int thr_kind, int threads, bool fast, size_t smem_bytes, int* blocks_per_sm)
 {
     *blocks_per_sm = 0;
-    const void* k = pick(threads);
+    const void* k = pick(g.lattice, thr_kind, threads, fast);
     if (const int e = set_smem_limit(k)) return e;
     const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, threads, smem_bytes);
     if (e != cudaSuccess) cudaGetLastError();
@@ -442,7 +531,7 @@ int resident_prepare(int threads, size_t smem_bytes, int* blocks_per_sm)
 }
 
 int launch_resident(const Geom& g, uint32_t* rows, const ResidentPlan& plan, uint32_t sweep0,
-                    uint32_t nsweeps, const DevRng& rng, const int2* grange,
+                    uint32_t nsweeps, const DevRng& rng, const ThrView& th, const int2* grange,
                     unsigned int epoch, unsigned long long* ring, uint32_t* counts, uint64_t burn,
                     uint32_t stride, const uint8_t* colours, unsigned long long* flips, void* stream)
 {
@@ -452,12 +541,14 @@ int launch_resident(const Geom& g, uint32_t* rows, const ResidentPlan& plan, uin
     P.g = g;
     P.stripe_lo = plan.stripe_lo;
     P.halo = plan.halo;
+    P.npre = plan.npre;
     P.colours = colours;
     P.cap_items = plan.cap_items;
     P.cap_cycle = plan.cap_cycle;
     P.sweep0 = sweep0;
     P.nsweeps = nsweeps;
     P.rng = rng;
+    P.th = th;
     P.grange = grange;
     P.xbuf = plan.xbuf;
     P.status = plan.status;
@@ -468,7 +559,7 @@ int launch_resident(const Geom& g, uint32_t* rows, const ResidentPlan& plan, uin
     P.stride = stride;
     P.epoch = epoch;
     void* args[] = {&P};
-    const void* k = pick(plan.threads);
+    const void* k = pick(g.lattice, th.kind, plan.threads, plan.fast);
     return (int)cudaLaunchCooperativeKernel(k, dim3(plan.ctas), dim3(plan.threads), args, plan.smem_bytes,
                                             reinterpret_cast<cudaStream_t>(stream));
 }
