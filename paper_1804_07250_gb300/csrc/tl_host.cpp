@@ -1759,6 +1759,25 @@ static int group_form_from(const tl_chain* c)
     return planes == 6 ? 881 : dom ? 641 : 801;
 }
 
+// Words a stripe of the word kernel may hold for it to beat a launch per pass.
+// Over 2,048 a thread owns four, with 64 registers and spills.  us a sweep, four
+// words / per pass, at the words a stripe: six-vertex 13.4 / 33.9 (2,304) and 13.1 /
+// 40.8 (3,456); dominoes with one threshold 8.3 / 12.3 (2,176, 2 to 4 planes), 12.6 /
+// 13.2 (3,968), 18.6 / 24.6 (32 planes), but with 5 planes 10.6 / 12.3 (2,176),
+// 12.6 / 12.3 (2,432), 14.4 / 12.3 (3,328); with one a site 16.7 / 19.4 (2,176),
+// 19.3 / 20.3 (2,432), 16.8 / 14.1 (3,072); lozenges of 2 to 4 planes 14.4 / 18.5
+// (2,176), 15.6 / 18.5 (2,432), 21.6 / 18.5 (2,688), of more 17.3 / 18.5, 19.0 / 18.5
+// and 24.5 / 18.5, with one a site 25.3 / 19.0 (2,176).
+static int word_form_to(const tl_chain* c)
+{
+    if (c->g.lattice == LAT_SIXV) return 4096;
+    const bool dom = c->g.lattice == LAT_DOMINO;
+    if (c->th.kind == THR_SITE) return dom ? 2432 : 2048;
+    const int planes = c->th.kmax + 1;
+    if (dom) return planes == 5 ? 2176 : 4096;
+    return planes <= 4 ? 2432 : 2176;
+}
+
 // The word kernel: stripes, passes per exchange, threads and words per thread.
 //
 // A pass is modelled as a fixed chain (update and barrier), a cost per
@@ -1835,6 +1854,10 @@ static int plan_words(tl_chain* c)
             groups_tried = true;
             if (plan_groups(c, false) == TL_OK) return TL_OK;
             free_resident(c);
+        }
+        if (c->kernel != 2 && lanes > word_form_to(c)) {
+            c->res_why = "a launch per pass is the faster one";
+            continue;
         }
         // `threads` asks for at most that many; results never depend on it
         const int cap = c->threads_req == 512 && lanes <= 2048 ? 512 : 1024;
