@@ -1840,11 +1840,12 @@ static int plan_words(tl_chain* c)
     for (const Cand& cd : cand) {
         const int h = cd.h, C = cd.C;
         const std::vector<int> lo = even_stripes(w, C, h, step);
-        int max_nloc = 0, items = 0;
+        int max_nloc = 0, max_own = 0, items = 0;
         for (int k = 0; k < C; ++k) {
             int slo, shi;
             stripe_local(lo[k], lo[k + 1], k, C, h, g.H, &slo, &shi);
             max_nloc = std::max(max_nloc, shi - slo);
+            max_own = std::max(max_own, lo[k + 1] - lo[k]);
             items = std::max(items, items_in(slo, shi));
         }
         const int lanes = std::max(32, 4 * items);
@@ -1872,6 +1873,7 @@ static int plan_words(tl_chain* c)
         c->res = ResidentPlan{};
         c->res.threads = threads;
         c->res.slots = slots;
+        c->res.max_words = (int)std::min<int64_t>(max_own * g.row_words, 1 << 30);
         // six-vertex words carry 8 or 4 planes by their build
         c->res.npre = sixv ? (slots <= 2 ? 8 : 4)
                            : c->npre_req > 0 ? c->npre_req
@@ -2159,7 +2161,24 @@ TL_API int tl_run_sweeps_hashed(tl_chain* c, uint64_t k, uint64_t* ring, void* s
         rc = zero_counts_if_needed(c, stream);
         cudaError_t e = cudaMemsetAsync(dring, 0, k * 8, SS(stream));
         if (rc == TL_OK && e != cudaSuccess) rc = fail(TL_ECUDA, "hash ring: %s", cudaGetErrorString(e));
-        if (rc == TL_OK) rc = run_resident(c, k, reinterpret_cast<unsigned long long*>(dring), stream);
+        // A stripe hashes its own words.  The outer stripes of large diamonds
+        // hold many rows of few, full words each, a lane's work and not a warp's:
+        // there a launch per sweep and a hash over the whole chip are faster (us a
+        // sweep: Aztec 1200 with a threshold a site 39.9 -> 28.2, 1600 42.3 -> 32.5;
+        // 900, 6,700 words a stripe, 18.5 as it is).  Rows of lozenges and faces are
+        // denser, and their stripes hash themselves faster (hexagon 1100 27.1, 34.7
+        // apart).
+        if (!c->use_reg && c->res.slots > 0 && c->g.lattice == LAT_DOMINO && c->res.max_words > 9600) {
+            for (uint64_t i = 0; i < k && rc == TL_OK; ++i) {
+                rc = run_resident(c, 1, nullptr, stream);
+                if (rc != TL_OK) break;
+                const int eh = launch_hash(c->g, c->rows, reinterpret_cast<unsigned long long*>(dring + i), stream);
+                c->launches += 1;
+                if (eh) rc = fail(TL_ECUDA, "hash kernel: %s", cudaGetErrorString((cudaError_t)eh));
+            }
+        } else if (rc == TL_OK) {
+            rc = run_resident(c, k, reinterpret_cast<unsigned long long*>(dring), stream);
+        }
         k = rc == TL_OK ? k : 0;
         goto copy_back;
     }

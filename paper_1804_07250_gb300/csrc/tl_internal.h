@@ -130,6 +130,7 @@ struct ResidentPlan {
     int slots;                     // words per thread (the word kernel; 0: a thread per group, tl_resident.cu)
     int halo;                      // passes per exchange cycle (= halo rows per side)
     int npre;                      // random planes generated ahead per group
+    int max_words;                 // words of the largest stripe, without halos (the word kernel)
     int cap_items;                 // slots 0: item-table capacity per CTA
     int cap_cycle;                 // slots 0: groups touched per cycle, per CTA (upper bound)
     bool fast;                     // dominoes at t = 2^31: branch-free single-plane update

@@ -1,6 +1,8 @@
 // Launches of the word kernel (tl_words_kernel.cuh).
 #include "tl_words_kernel.cuh"
 
+#include <numeric>
+
 namespace tl {
 
 // ---- host side ----
@@ -14,6 +16,21 @@ static const void* pick(int lattice, int tk, int cpol, int threads, int slots, b
     if (lattice == LAT_DOMINO) return words_kernel_domino(tk, threads, slots, fixed);
     if (lattice == LAT_LOZENGE) return words_kernel_lozenge(tk, threads, slots, fixed);
     return words_kernel_sixv(cpol >= 0, threads, slots, fixed);
+}
+
+// Threads of a launch with a hash after every sweep: up to 512, whatever the
+// passes need, share the words, in a number of warps that does not divide the
+// 32-word runs of a row (or the same warps would take the same planes, the full
+// ones, in every row).  us a sweep with the plan's threads -> these: Aztec 40 6.4
+// -> 4.7, 300 8.3 -> 5.9, hexagon 200 12.7 -> 8.5, domain-wall square 30 12.7 ->
+// 5.0, 500 12.2 -> 7.0; Aztec 900 (128 words a row) 17 with 480 threads, 42 with 512.
+static int hash_threads(const Geom& g, const ResidentPlan& plan)
+{
+    if (plan.slots != 1 || plan.threads >= 512) return plan.threads;
+    const int runs = g.row_words % 32 ? 1 : (int)(g.row_words / 32);
+    for (int w = 16; 32 * w > plan.threads && w > 12; --w)
+        if (std::gcd(w, runs) == 1) return 32 * w;
+    return plan.threads;
 }
 
 size_t words_smem_bytes(const Geom& g, int local_rows) { return (size_t)local_rows * g.row_words * 4 + (size_t)(local_rows + 2) * 4; }
@@ -91,8 +108,8 @@ int launch_words(const Geom& g, uint32_t* rows, const ResidentPlan& plan, uint32
     void* args[] = {&P};
     const bool fixed = !colours && plan.halo % g.passes == 0;
     const void* k = pick(g.lattice, th.kind, th.cpol, plan.threads, plan.slots, fixed);
-    return (int)cudaLaunchCooperativeKernel(k, dim3(plan.ctas), dim3(plan.threads), args, plan.smem_bytes,
-                                            reinterpret_cast<cudaStream_t>(stream));
+    return (int)cudaLaunchCooperativeKernel(k, dim3(plan.ctas), dim3(ring ? hash_threads(g, plan) : plan.threads), args,
+                                            plan.smem_bytes, reinterpret_cast<cudaStream_t>(stream));
 }
 
 }  // namespace tl
