@@ -428,9 +428,17 @@ __global__ void hash_kernel(const uint32_t* __restrict__ rows0, Geom g, unsigned
     if ((threadIdx.x & 31) == 0 && acc) atomicAdd(out, (unsigned long long)acc);
 }
 
-// The same in one block, writing the result itself (small states: one launch
-// instead of a clear and a launch).
-constexpr int64_t kSmallHashWords = 8192;
+// The same in one block, writing the result itself: one launch instead of a
+// clear and a launch, where a thread takes one word.  A word is a chain of up
+// to 32 mixes, and one SM has room for 32 warps of them: us a hash in one block
+// / in two launches, Aztec diamonds 8 3.6 / 5.1, 24 5.2 / 5.8, 32 (1,040 words)
+// 6.2 / 6.2, 40 7.2 / 6.3, 127 20.7 / 8.3; domain-wall squares (denser) 30 5.6 /
+// 6.3, 40 (672 words) 6.3 / 6.4, 50 7.9 / 6.8, 180 20.8 / 8.2; hexagons 10 4.3 /
+// 5.0, 20 6.3 / 6.1, 40 11.5 / 6.4.
+static bool small_hash(const Geom& g)
+{
+    return (int64_t)g.H * g.row_words <= (g.lattice == LAT_SIXV ? 704 : 1040);
+}
 __global__ void __launch_bounds__(1024) hash_small_kernel(const uint32_t* __restrict__ rows0, Geom g,
                                                           unsigned long long* out)
 {
@@ -455,7 +463,7 @@ __global__ void __launch_bounds__(1024) hash_small_kernel(const uint32_t* __rest
 
 int launch_hash(const Geom& g, const uint32_t* rows, unsigned long long* out, void* stream)
 {
-    if ((int64_t)g.H * g.row_words <= kSmallHashWords) {
+    if (small_hash(g)) {
         hash_small_kernel<<<1, 1024, 0, S(stream)>>>(rows + g.row_words, g, out);
         return (int)cudaGetLastError();
     }
