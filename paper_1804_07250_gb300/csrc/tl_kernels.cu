@@ -795,8 +795,8 @@ __global__ void __launch_bounds__(1024) height_link_kernel(const uint32_t* __res
     link_segments<LAT>(rows0, g, seg, nseg, hw, rel, base, val, up);
 }
 
-// All of it in one block, for grids so small that four launches take longer.
-constexpr int64_t kSmallHeights = 32768;
+// All of it in one block, for grids so small that four launches take longer:
+// its 32 warps take the segments in turn, 32 vertices at a time.
 template <int LAT>
 __global__ void __launch_bounds__(1024) height_small_kernel(const uint32_t* __restrict__ rows0, Geom g,
                                                             const int* __restrict__ seg, int nseg, int hw, int n,
@@ -829,9 +829,15 @@ __global__ void __launch_bounds__(256) height_add_kernel(int32_t* __restrict__ o
     for (int x = lo + threadIdx.x; x <= hi; x += 256) o[x] += b;
 }
 
+// One block or four launches.  us in one block / four launches: Aztec diamonds 32
+// 8.3 / 17.6, 64 12.5 / 17.8, 100 (40,401 heights) 19.6 / 18.2, 127 28.0 / 18.6;
+// domain-wall squares 100 12.7 / 17.5, 140 (19,881) 17.8 / 17.6, 180 23.7 / 17.5;
+// squares of 11 columns 300 (301 segments) 15.3 / 18.5, 1000 36.7 / 18.5; flat ones
+// 1000 x 4 (32 turns a segment) 12.5 / 17.5, 2000 x 4 20.7 / 19.7, 15000 x 1 119 / 37.
 int height_launches(int nseg, int hw, int hh)
 {
-    return nseg <= 0 || ((int64_t)hw * hh <= kSmallHeights && nseg <= 1024) ? 1 : 4;
+    const int64_t turns = (int64_t)((nseg + 31) / 32) * ((hw + 31) / 32);
+    return nseg <= 0 || ((int64_t)hw * hh <= 20000 && nseg <= 320 && turns <= 32) ? 1 : 4;
 }
 
 int launch_height(const Geom& g, const uint32_t* rows, const int* seg, int nseg, int hw, int hh, int32_t* out,
