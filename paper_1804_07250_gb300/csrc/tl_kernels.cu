@@ -93,35 +93,62 @@ int launch_pass_global(const Geom& g, uint32_t* rows, uint32_t pass, uint32_t sl
 // ---------------------------------------------------------------------------
 // Layout conversion.  Canonical: uint8 [ntype][H][W].
 // ---------------------------------------------------------------------------
-// A warp per (row, plane): lane l looks at the byte of bit l of a word, and a
-// ballot is the word.
+// A thread per word, for planes of one group a row (at most 128 columns each): the
+// rows are too short for a warp.
+__global__ void pack_narrow_kernel(const uint8_t* __restrict__ canon, uint32_t* __restrict__ rows, Geom g)
+{
+    const uint32_t n = (uint32_t)g.H * (uint32_t)g.row_words;
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const uint32_t y = i / (uint32_t)g.row_words, rem = i - y * (uint32_t)g.row_words;
+        const int pl = (int)rem / g.K, k = (int)rem - pl * g.K, type = pl / g.npar, res = pl - type * g.npar;
+        const uint8_t* src = canon + ((size_t)type * g.H + y) * g.W;
+        uint32_t w = 0;
+        for (int b = 0; b < 32; ++b) {
+            const int x = g.npar * (32 * k + b) + res;
+            if (x < g.W && src[x]) w |= 1u << b;
+        }
+        rows[g.row_words + i] = w;
+    }
+}
+
+// A warp per 32 words of a (row, plane): lane l looks at the byte of bit l of a
+// word, and a ballot is the word.  (Indices fit 32 bits: at most 65,536 rows of
+// 9 planes of 32 such runs.)
+// us: square 2048 18 with a thread a word, 9.4 with a warp a row, 10 so; 60000 x 4
+// 4.0, 52, 3.4; 12000 x 60 5.9, 13, 4.1.
 __global__ void pack_kernel(const uint8_t* __restrict__ canon, uint32_t* __restrict__ rows, Geom g)
 {
     const int lane = threadIdx.x & 31;
-    const int64_t nr = (int64_t)g.H * g.P, nw = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t r = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); r < nr; r += nw) {
-        const int y = (int)(r / g.P), pl = (int)(r - (int64_t)y * g.P);
+    const uint32_t runs = (uint32_t)(g.K + 31) >> 5, n = (uint32_t)g.H * (uint32_t)g.P * runs,
+                   step = gridDim.x * (blockDim.x >> 5);
+    for (uint32_t u = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); u < n; u += step) {
+        const uint32_t r = runs == 1u ? u : u / runs, y = r / (uint32_t)g.P;
+        const int pl = (int)(r - y * (uint32_t)g.P), k0 = 32 * (int)(u - r * runs);
         const int type = pl / g.npar, res = pl - type * g.npar;
         const uint8_t* src = canon + ((size_t)type * g.H + y) * g.W;
         uint32_t* dst = rows + g.row_words + (int64_t)y * g.row_words + (int64_t)pl * g.K;
-        for (int k0 = 0; k0 < g.K; k0 += 32) {
-            const int n = g.K - k0 < 32 ? g.K - k0 : 32;   // a multiple of 4
-            uint32_t keep = 0;
-            for (int k = 0; k < n; k += 8) {
-                uint32_t w[8];
+        const int nk = g.K - k0 < 32 ? g.K - k0 : 32;   // a multiple of 4
+        uint32_t keep = 0;
+        auto words = [&](int k, auto cnt) {
+            constexpr int N = decltype(cnt)::value;
+            uint32_t w[N];
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const int x = g.npar * (32 * (k0 + k + j) + lane) + res;
-                    w[j] = x < g.W ? src[x] : 0u;
-                }
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const uint32_t v = __ballot_sync(0xFFFFFFFFu, w[j] != 0u);
-                    if (lane == k + j) keep = v;
-                }
+            for (int j = 0; j < N; ++j) {
+                const int x = g.npar * (32 * (k0 + k + j) + lane) + res;
+                w[j] = x < g.W ? src[x] : 0u;
             }
-            if (lane < n) dst[k0 + lane] = keep;
-        }
+#pragma unroll
+            for (int j = 0; j < N; ++j) {
+                const uint32_t v = __ballot_sync(0xFFFFFFFFu, w[j] != 0u);
+                if (lane == k + j) keep = v;
+            }
+        };
+        // the words that hold columns of the domain's box
+        const int nw = (g.W + 32 * g.npar - 1) / (32 * g.npar) - k0, nv = nk < nw ? nk : nw;
+        int k = 0;
+        for (; k + 8 <= nv; k += 8) words(k, std::integral_constant<int, 8>{});
+        for (; k < nv; k += 2) words(k, std::integral_constant<int, 2>{});
+        if (lane < nk) dst[k0 + lane] = keep;
     }
 }
 
@@ -149,42 +176,43 @@ TL_DEV uint32_t spread3(uint32_t x)
     return (x | (x << 2)) & 0x00249249u;
 }
 
-// A warp per canonical row, 16 bytes a lane: the bits of 16 neighbouring edges
+// 16 bytes a thread: the bits of 16 neighbouring edges of a canonical row
 // interleaved from the row's planes, four bits at a time spread into bytes by
 // a product, and one aligned 16-byte store (the row's ragged ends by bytes).
-// 33.6 MB of the Aztec diamond 2048: 121 us with a thread and three divisions
-// a byte.
+// A row's units at its own alignment (at most `units`) are consecutive threads,
+// whatever the shape: with a warp a row, few wide rows leave the chip idle and
+// narrow ones the lanes.
+// us: square 2048 36 with a thread a byte, 6.0 with a warp a row, 5.9 so; 60000 x 4
+// 5.7, 39, 1.9; 200 x 20000 35, 15, 7.9; 2 x 30000 2.9, 20, 3.1.
 __global__ void unpack_kernel(const uint32_t* __restrict__ rows, uint8_t* __restrict__ canon, Geom g)
 {
-    const int lane = threadIdx.x & 31;
-    const int64_t nr = (int64_t)g.ntype * g.H, nw = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t r = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); r < nr; r += nw) {
-        const int type = (int)(r / g.H), y = (int)(r - (int64_t)type * g.H);
+    const uint32_t units = (uint32_t)(g.W + 30) >> 4, n = (uint32_t)(g.ntype * g.H) * units;
+    for (uint32_t u = blockIdx.x * blockDim.x + threadIdx.x; u < n; u += gridDim.x * blockDim.x) {
+        const uint32_t r = u / units;
+        const int type = (int)(r / (uint32_t)g.H), y = (int)(r - (uint32_t)type * (uint32_t)g.H);
         const uint32_t* p = rows + g.row_words + (int64_t)y * g.row_words + (int64_t)type * g.npar * g.K;
         uint8_t* o = canon + (size_t)r * g.W;
         const int lead = (int)(reinterpret_cast<uintptr_t>(o) & 15u);
-        const int chunks = (lead + g.W + 15) >> 4;
-        for (int c = lane; c < chunks; c += 32) {
-            const int x0 = 16 * c - lead;   // may be negative: those bits are not stored
-            uint32_t v;
-            if (g.npar == 2) {
-                const int j0 = x0 >> 1;
-                v = (spread2(plane_bits(p, g.K, j0)) | spread2(plane_bits(p + g.K, g.K, j0)) << 1) >> (x0 & 1);
-            } else {
-                const int j0 = (x0 + 18) / 3 - 6;   // floor, x0 > -16
-                v = (spread3(plane_bits(p, g.K, j0)) | spread3(plane_bits(p + g.K, g.K, j0)) << 1 |
-                     spread3(plane_bits(p + 2 * g.K, g.K, j0)) << 2) >>
-                    (x0 - 3 * j0);
-            }
-            const uint32_t b0 = ((v & 15u) * 0x00204081u) & 0x01010101u, b1 = (((v >> 4) & 15u) * 0x00204081u) & 0x01010101u,
-                           b2 = (((v >> 8) & 15u) * 0x00204081u) & 0x01010101u,
-                           b3 = (((v >> 12) & 15u) * 0x00204081u) & 0x01010101u;
-            if (x0 >= 0 && x0 + 16 <= g.W) {
-                *reinterpret_cast<uint4*>(o + x0) = make_uint4(b0, b1, b2, b3);
-            } else {
-                for (int t = 0; t < 16; ++t)
-                    if (x0 + t >= 0 && x0 + t < g.W) o[x0 + t] = (uint8_t)((v >> t) & 1u);
-            }
+        const int x0 = 16 * (int)(u - r * units) - lead;   // may be negative: those bits are not stored
+        if (x0 >= g.W) continue;
+        uint32_t v;
+        if (g.npar == 2) {
+            const int j0 = x0 >> 1;
+            v = (spread2(plane_bits(p, g.K, j0)) | spread2(plane_bits(p + g.K, g.K, j0)) << 1) >> (x0 & 1);
+        } else {
+            const int j0 = (x0 + 18) / 3 - 6;   // floor, x0 > -16
+            v = (spread3(plane_bits(p, g.K, j0)) | spread3(plane_bits(p + g.K, g.K, j0)) << 1 |
+                 spread3(plane_bits(p + 2 * g.K, g.K, j0)) << 2) >>
+                (x0 - 3 * j0);
+        }
+        const uint32_t b0 = ((v & 15u) * 0x00204081u) & 0x01010101u, b1 = (((v >> 4) & 15u) * 0x00204081u) & 0x01010101u,
+                       b2 = (((v >> 8) & 15u) * 0x00204081u) & 0x01010101u,
+                       b3 = (((v >> 12) & 15u) * 0x00204081u) & 0x01010101u;
+        if (x0 >= 0 && x0 + 16 <= g.W) {
+            *reinterpret_cast<uint4*>(o + x0) = make_uint4(b0, b1, b2, b3);
+        } else {
+            for (int t = 0; t < 16; ++t)
+                if (x0 + t >= 0 && x0 + t < g.W) o[x0 + t] = (uint8_t)((v >> t) & 1u);
         }
     }
 }
@@ -201,13 +229,14 @@ int launch_pack(const Geom& g, const uint8_t* canon_dev, uint32_t* rows, void* s
 {
     cudaError_t e = cudaMemsetAsync(rows, 0, (size_t)g.total_words * 4, S(stream));
     if (e != cudaSuccess) return (int)e;
-    pack_kernel<<<grid_for((int64_t)g.H * g.P * 32, 256), 256, 0, S(stream)>>>(canon_dev, rows, g);
+    if (g.K == 4) pack_narrow_kernel<<<grid_for((int64_t)g.H * g.row_words, 256), 256, 0, S(stream)>>>(canon_dev, rows, g);
+    else pack_kernel<<<grid_for((int64_t)g.H * g.P * ((g.K + 31) / 32) * 32, 256), 256, 0, S(stream)>>>(canon_dev, rows, g);
     return (int)cudaGetLastError();
 }
 
 int launch_unpack(const Geom& g, const uint32_t* rows, uint8_t* canon_dev, void* stream)
 {
-    unpack_kernel<<<grid_for((int64_t)g.ntype * g.H * 32, 256), 256, 0, S(stream)>>>(rows, canon_dev, g);
+    unpack_kernel<<<grid_for((int64_t)g.ntype * g.H * ((g.W + 30) / 16), 256), 256, 0, S(stream)>>>(rows, canon_dev, g);
     return (int)cudaGetLastError();
 }
 
@@ -291,20 +320,20 @@ __global__ void validate_bytes_kernel(const uint8_t* __restrict__ s, size_t n, u
 // The lattice checks: a warp per 256 columns of a row.
 constexpr int kCheckCols = 256;
 struct WarpSpan {
-    int64_t u, n, step;
-    int segs, cols;
+    uint32_t u, n, step;   // 32 bits: at most 65,537 rows of 257 spans
+    uint32_t segs;
+    int cols;
     TL_DEV WarpSpan(int rows, int cols_)
-        : u(blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5)), step((int64_t)gridDim.x * (blockDim.x >> 5)),
-          cols(cols_)
+        : u(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)), step(gridDim.x * (blockDim.x >> 5)), cols(cols_)
     {
-        segs = (cols + kCheckCols - 1) / kCheckCols;
-        n = (int64_t)rows * segs;
+        segs = (uint32_t)(cols + kCheckCols - 1) / kCheckCols;
+        n = (uint32_t)rows * segs;
     }
-    TL_DEV int row() const { return (int)(u / segs); }
+    TL_DEV int row() const { return (int)(segs == 1u ? u : u / segs); }
     // this lane's first column and the end of the span
     TL_DEV void span(int row, int& x0, int& x1) const
     {
-        const int c = (int)(u - (int64_t)row * segs) * kCheckCols;
+        const int c = (int)(u - (uint32_t)row * segs) * kCheckCols;
         x0 = c + (int)(threadIdx.x & 31);
         x1 = c + kCheckCols < cols ? c + kCheckCols : cols;
     }
