@@ -637,7 +637,7 @@ __global__ void __launch_bounds__(256) nsew_kernel(const uint32_t* __restrict__ 
     }
 }
 
-// Rows too wide for shared memory: from canonical counters in memory.
+// Few wide rows, or many narrow ones: from canonical counters in memory.
 __global__ void nsew_counts_kernel(const uint32_t* __restrict__ counts, Geom g, double inv, int kappa,
                                    double* __restrict__ out)
 {
@@ -663,7 +663,13 @@ int launch_nsew(const Geom& g, const uint32_t* cplanes, uint32_t* counts, uint64
 {
     const double inv = samples ? 1.0 / (double)samples : 0.0;
     const size_t smem = sizeof(double) * kNsewTable + 3 * sizeof(uint32_t) * (size_t)g.W;
-    if (smem <= (size_t)smem_optin) {
+    // A block per row leaves the chip idle where a domain has few rows, and
+    // spends 3 us a row however narrow it is where a block takes several.  us
+    // fused / through memory: 16000 x 2 27 / 8, 8000 x 8 17 / 10, 2000 x 8 10 / 8,
+    // 8000 x 31 17 / 17, 12000 x 60 21 / 33; 20 x 20000 68 / 23, 100 x 20000 100 /
+    // 78, 200 x 20000 107 / 148, 30 x 900 9.8 / 8.5.
+    const bool flat = g.H <= 32 && g.W > 1600, narrow = g.W < 160 && g.H > 880;
+    if (!flat && !narrow && smem <= (size_t)smem_optin) {
         int nbits = 0;
         while (nbits < 32 && (samples >> nbits)) ++nbits;
         cudaError_t e = cudaFuncSetAttribute(nsew_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin);
