@@ -1955,11 +1955,18 @@ static bool small_run(const tl_chain* c)
     return c->use_reg && c->small_threads > 0 && !c->density_on && !c->random_order && !c->count_flips;
 }
 
+// Sweeps of one resident launch at most: exchange tags carry 16 bits of cycle
+// and 16 bits of launch epoch, and a launch ends in a time that a user can wait
+// for (well under a second).
+static uint64_t max_launch_sweeps(const tl_chain* c)
+{
+    return std::max<uint64_t>(1, 60000ull * c->res.halo / c->g.passes);
+}
+
 // Resident launches over [c->sweep, c->sweep + k), at most spl sweeps each.
 static int run_resident(tl_chain* c, uint64_t k, unsigned long long* ring, void* stream)
 {
-    // exchange tags carry 16 bits of cycle and 16 bits of launch epoch
-    const uint64_t max_sweeps = std::max<uint64_t>(1, 60000ull * c->res.halo / c->g.passes);
+    const uint64_t max_sweeps = max_launch_sweeps(c);
     uint64_t done = 0;
     while (done < k) {
         uint64_t n = c->spl > 0 ? std::min<uint64_t>((uint64_t)c->spl, k - done) : k - done;
@@ -2697,13 +2704,16 @@ TL_API int tl_cftp(tl_ctx* ctx, const tl_domain* d, uint64_t seed, uint32_t stre
             if (rc == TL_OK) rc = tl_chain_seek(c, 0x100000000ull - T);
         }
         if (pair) {
-            const int e = rc == TL_OK ? launch_small(top->g, top->rows, bot->rows, top->small_threads,
-                                                     (uint32_t)top->sweep, (uint32_t)T, top->rng, top->grange, stream)
-                                      : 0;
-            if (e) rc = fail(TL_ECUDA, "tl_cftp: %s", cudaGetErrorString((cudaError_t)e));
-            for (tl_chain* c : {top, bot}) {
-                c->sweep += T;
-                c->launches += 1;
+            for (uint64_t done = 0; rc == TL_OK && done < T;) {
+                const uint64_t n = std::min(T - done, max_launch_sweeps(top));
+                const int e = launch_small(top->g, top->rows, bot->rows, top->small_threads, (uint32_t)top->sweep,
+                                           (uint32_t)n, top->rng, top->grange, stream);
+                if (e) rc = fail(TL_ECUDA, "tl_cftp: %s", cudaGetErrorString((cudaError_t)e));
+                for (tl_chain* c : {top, bot}) {
+                    c->sweep += n;
+                    c->launches += 1;
+                }
+                done += n;
             }
         } else if (side) {
             cudaError_t e = cudaEventRecord(ready, SS(stream));   // the resets
