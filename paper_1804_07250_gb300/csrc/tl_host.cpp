@@ -2911,6 +2911,7 @@ struct tl_batch {
     int tile_rows = 64, R = 2, block = 100, grid = 0;
     int threads = 256;                    // threads per tile (faces per thread)
     int run_threads = 256;                // threads per tile of the launches: more where tiles are few
+    int run_rows = 64, run_R = 2;         // rows per tile and sweeps per launch: fewer where tiles are few or wide
     size_t smem = 0;
     int ntiles = 0;
     int src = 0;                          // buffer holding the current state
@@ -2974,33 +2975,47 @@ static int batch_plan(tl_batch* b, int tile_rows, int R, int threads)
         return n;
     };
     while (rows >= 128 && count(rows) < (size_t)b->ctx->sms) rows = (rows + 3) / 4 * 2;
-    for (size_t i = 0; i < b->chains.size(); ++i) {
-        const tl_chain* c = b->chains[i];
-        const Geom& g = c->g;
-        const int halo = g.passes * R, step = g.lattice == LAT_SIXV ? 2 : 1;
-        const std::vector<int2> unit = unit_groups(c->dom_copy);
-        std::vector<int> pre(unit.size() + 1, 0);
-        for (size_t r = 0; r < unit.size(); ++r) pre[r + 1] = pre[r] + std::max(0, unit[r].y - unit[r].x);
-        first.push_back((int)tiles.size());
-        for (int lo = 0; lo < g.H; lo += rows) {
-            const int hi = std::min(g.H, lo + rows);
-            tiles.push_back(BatchTile{(int)i, lo, hi});
-            const int slo = std::max(lo - halo, -1), shi = std::min(hi + halo, g.H + 1);
-            const int ra = std::max(slo, 0) / step, rb = (std::min(shi, g.H) + step - 1) / step;
-            const int items = pre[rb] - pre[ra];
-            // rows, then the item table
-            smem = std::max(smem, (size_t)(shi - slo) * (size_t)g.row_words * 4 + 4 * (size_t)(rb - ra + 1 + items));
-            work.push_back((0.1 * (rb - ra) + items) * R);
+    // the rows of a tile and its halos alone
+    size_t need = 0;
+    for (const tl_chain* c : b->chains)
+        need = std::max(need, (size_t)std::min(rows + 2 * c->g.passes * R, c->g.H + 2) * (size_t)c->g.row_words * 4);
+    if ((long)need > (long)b->ctx->smem_optin) return fail(TL_EUNSUPPORTED, "batch plan: a tile needs %zu B of shared memory", need);
+    int bps = 0, run_threads = threads, run_R = R;
+    // where the rows fit and the item table beside them does not, lower tiles do
+    // (and below one row, whose halo is then the tile, fewer sweeps a launch)
+    for (const int asked = rows;; rows > 1 ? rows = (rows + 1) / 2 : (rows = asked, run_R = (run_R + 1) / 2)) {
+        tiles.clear();
+        work.clear();
+        first.clear();
+        smem = 0;
+        for (size_t i = 0; i < b->chains.size(); ++i) {
+            const tl_chain* c = b->chains[i];
+            const Geom& g = c->g;
+            const int halo = g.passes * run_R, step = g.lattice == LAT_SIXV ? 2 : 1;
+            const std::vector<int2> unit = unit_groups(c->dom_copy);
+            std::vector<int> pre(unit.size() + 1, 0);
+            for (size_t r = 0; r < unit.size(); ++r) pre[r + 1] = pre[r] + std::max(0, unit[r].y - unit[r].x);
+            first.push_back((int)tiles.size());
+            for (int lo = 0; lo < g.H; lo += rows) {
+                const int hi = std::min(g.H, lo + rows);
+                tiles.push_back(BatchTile{(int)i, lo, hi});
+                const int slo = std::max(lo - halo, -1), shi = std::min(hi + halo, g.H + 1);
+                const int ra = std::max(slo, 0) / step, rb = (std::min(shi, g.H) + step - 1) / step;
+                const int items = pre[rb] - pre[ra];
+                // rows, then the item table
+                smem = std::max(smem, (size_t)(shi - slo) * (size_t)g.row_words * 4 + 4 * (size_t)(rb - ra + 1 + items));
+                work.push_back((0.1 * (rb - ra) + items) * run_R);
+            }
         }
-    }
-    first.push_back((int)tiles.size());
-    if ((long)smem > (long)b->ctx->smem_optin) return fail(TL_EUNSUPPORTED, "batch plan: a tile needs %zu B of shared memory", smem);
-    int bps = 0;
-    int run_threads = tiles.size() <= (size_t)b->ctx->sms ? 512 : tiles.size() <= 2 * (size_t)b->ctx->sms ? 256 : threads;
-    if (batch_prepare(smem, run_threads, &bps) != 0 || bps < 1) {
-        run_threads = threads;
-        if (batch_prepare(smem, threads, &bps) != 0 || bps < 1)
-            return fail(TL_EUNSUPPORTED, "batch plan: tile kernel does not fit");
+        first.push_back((int)tiles.size());
+        const size_t sms = (size_t)b->ctx->sms;
+        run_threads = tiles.size() <= sms ? 512 : tiles.size() <= 2 * sms ? 256 : threads;
+        if ((long)smem <= (long)b->ctx->smem_optin) {
+            if (batch_prepare(smem, run_threads, &bps) == 0 && bps > 0) break;
+            run_threads = threads;
+            if (batch_prepare(smem, run_threads, &bps) == 0 && bps > 0) break;
+        }
+        if (rows == 1 && run_R == 1) return fail(TL_EUNSUPPORTED, "batch plan: a tile needs %zu B of shared memory", smem);
     }
     std::vector<int> order(tiles.size());
     for (size_t i = 0; i < order.size(); ++i) order[i] = (int)i;
@@ -3020,6 +3035,8 @@ static int batch_plan(tl_batch* b, int tile_rows, int R, int threads)
     b->R = R;
     b->threads = threads;
     b->run_threads = run_threads;
+    b->run_rows = rows;
+    b->run_R = run_R;
     b->smem = smem;
     b->grid = std::min(bps * b->ctx->sms, b->ntiles);
     return TL_OK;
@@ -3222,12 +3239,12 @@ static std::vector<int> batch_launch_sizes(uint64_t k, int R)
 // Graph of one block of `block` sweeps: the launches plus the counter advance.
 static int batch_build_graph(tl_batch* b, void* stream)
 {
-    if (b->graph && b->graph_block == b->block && b->graph_R == b->R) return TL_OK;
+    if (b->graph && b->graph_block == b->block && b->graph_R == b->run_R) return TL_OK;
     if (b->graph) cudaGraphExecDestroy(b->graph);
     b->graph = nullptr;
     cudaStream_t s = SS(stream);
     if (!s) return TL_OK;   // the legacy stream cannot be captured: run without a graph
-    const std::vector<int> sizes = batch_launch_sizes((uint64_t)b->block, b->R);
+    const std::vector<int> sizes = batch_launch_sizes((uint64_t)b->block, b->run_R);
     if (sizes.size() % 2) return TL_OK;   // cannot keep the buffers aligned: no graph
     const int src0 = b->src;
     const uint64_t l0 = b->launches;
@@ -3255,7 +3272,7 @@ static int batch_build_graph(tl_batch* b, void* stream)
     cudaGraphDestroy(graph);
     if (ie != cudaSuccess) return fail(TL_ECUDA, "batch graph instantiate: %s", cudaGetErrorString(ie));
     b->graph_block = b->block;
-    b->graph_R = b->R;
+    b->graph_R = b->run_R;
     b->graph_launches = (int)sizes.size();
     return TL_OK;
 }
@@ -3274,7 +3291,7 @@ static int batch_run(tl_batch* b, uint64_t k, void* stream, bool per_chain)
     }
     // the rest: offsets relative to the counters after the last advance
     const uint64_t rest_start = done;
-    const std::vector<int> sizes = batch_launch_sizes(k - done, b->R);
+    const std::vector<int> sizes = batch_launch_sizes(k - done, b->run_R);
     uint32_t off = 0;
     for (size_t j = 0; j < sizes.size(); ++j) {
         TL_TRY(batch_launch(b, sizes[j], off, (int)j, stream, per_chain));

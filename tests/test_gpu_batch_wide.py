@@ -18,8 +18,8 @@ def T():
 
 
 # 232,448 bytes a block: 72 rows of 3,136 bytes leave no room for their table; nor
-# do one row and 64 halo rows of 3,456
-@pytest.mark.parametrize("width,height,rows,R", [(12500, 300, 64, 2), (12500, 300, 0, 0), (13700, 200, 1, 16)])
+# do one row and its 68 halo rows
+@pytest.mark.parametrize("width,height,rows,R", [(12500, 300, 64, 2), (12500, 300, 0, 0), (12500, 200, 1, 17)])
 def test_wide_chain(T, width, height, rows, R):
     ctx = T.Context(0)
     th = T.thresholds(scalar=3 << 29)
