@@ -547,9 +547,15 @@ int tl_debug_build(void);
 int tl_debug_checks(int clear, uint64_t* failures, int* first_id, int64_t* index, int64_t* bound);
 int tl_debug_selftest(void);
 
+/* Plan of a batch: what was asked for, and (out) what it comes to.  Launches
+ * can differ from tile_rows, sweeps_per_launch and threads; tl_batch_get_launch
+ * says what they take. */
 typedef struct {
-    int tile_rows;          /* rows per tile (0 = keep) */
-    int sweeps_per_launch;  /* R (0 = keep) */
+    int tile_rows;          /* rows per tile (0 = keep; fewer where the batch has
+                               fewer tiles than the GPU has SMs, or where the
+                               rows leave no shared memory for a tile's table) */
+    int sweeps_per_launch;  /* R (0 = keep; fewer where one row and its halos
+                               leave no room) */
     int graph_block;        /* sweeps per CUDA-graph block (0 = keep; default 100;
                                -1 = never capture graphs, e.g. while other threads
                                use the legacy stream) */
@@ -561,7 +567,9 @@ typedef struct {
                                group of a pass, so this sets the faces per
                                thread (128 threads: twice as many, with more
                                tiles resident per SM where shared memory
-                               allows) */
+                               allows).  Launches take 512 where the batch has
+                               no more tiles than the GPU has SMs, 256 up to
+                               twice as many tiles */
 } tl_batch_plan;
 
 int tl_batch_create(tl_ctx* ctx, tl_chain* const* chains, size_t n, tl_batch** out);
@@ -582,6 +590,9 @@ int tl_batch_run_per_chain(tl_batch* b, uint64_t k, void* stream);
 int tl_batch_hashes(tl_batch* b, uint64_t* out, size_t n, void* stream);
 int tl_batch_set_plan(tl_batch* b, const tl_batch_plan* plan);
 int tl_batch_get_plan(tl_batch* b, tl_batch_plan* plan);
+/* Rows per tile, sweeps per launch and threads per tile of the batch's launches
+ * (each pointer may be NULL). */
+int tl_batch_get_launch(tl_batch* b, int* tile_rows, int* sweeps, int* threads);
 /* Time every tile height in {32, 64, 128} x R in {1, 2, 4, 8} x threads per
  * tile in {256, 128} (the faces per thread) on the batch itself for
  * `trial_sweeps` sweeps (rounded up to a multiple of R), twice

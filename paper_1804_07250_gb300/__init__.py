@@ -140,6 +140,7 @@ _SIG = {
     "tl_batch_hashes": (_i, [_vp, _vp, ctypes.c_size_t, _vp]),
     "tl_batch_set_plan": (_i, [_vp, ctypes.POINTER(BatchPlan)]),
     "tl_batch_get_plan": (_i, [_vp, ctypes.POINTER(BatchPlan)]),
+    "tl_batch_get_launch": (_i, [_vp, ctypes.POINTER(_i), ctypes.POINTER(_i), ctypes.POINTER(_i)]),
     "tl_batch_autotune": (_i, [_vp, _u64, _vp, ctypes.POINTER(BatchPlan)]),
     "tl_batch_launches": (_u64, [_vp]),
     "tl_batch_add": (_i, [_vp, _vp]),
@@ -592,6 +593,12 @@ class Batch:
         p = BatchPlan()
         _check(_lib.tl_batch_get_plan(self._h, ctypes.byref(p)))
         return p.as_dict()
+
+    def launch_shape(self) -> dict:
+        """What the launches take (the plan holds what was asked for)."""
+        v = [_i() for _ in range(3)]
+        _check(_lib.tl_batch_get_launch(self._h, *[ctypes.byref(x) for x in v]))
+        return dict(zip(("tile_rows", "sweeps_per_launch", "threads"), (x.value for x in v)))
 
     def autotune(self, trial_sweeps: int = 8, stream=None) -> dict:
         p = BatchPlan()

@@ -3373,6 +3373,15 @@ TL_API int tl_batch_get_plan(tl_batch* b, tl_batch_plan* p)
     return TL_OK;
 }
 
+TL_API int tl_batch_get_launch(tl_batch* b, int* tile_rows, int* sweeps, int* threads)
+{
+    if (!b) return fail(TL_EINVAL, "tl_batch_get_launch: NULL batch");
+    if (tile_rows) *tile_rows = b->run_rows;
+    if (sweeps) *sweeps = b->run_R;
+    if (threads) *threads = b->run_threads;
+    return TL_OK;
+}
+
 // Try tile heights x sweeps per launch on the batch itself, keep the fastest.
 // The chains' states and sweep counters are restored afterwards, so tuning
 // does not change any result.
