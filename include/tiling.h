@@ -596,11 +596,13 @@ int tl_batch_get_launch(tl_batch* b, int* tile_rows, int* sweeps, int* threads);
 /* Time every tile height in {32, 64, 128} x R in {1, 2, 4, 8} x threads per
  * tile in {256, 128} (the faces per thread) on the batch itself for
  * `trial_sweeps` sweeps (rounded up to a multiple of R), twice
- * each from the same states, and keep the plan with the fastest run; states
- * and sweep counters are restored afterwards.  The result is cached per
- * (lattices present, threshold kinds present, total rows rounded down to a
- * power of two, SM count): a later batch with the same key takes the cached
- * plan at once, without trials.  tl_autotune_cache_clear empties the cache. */
+ * each from the same states, and keep the plan with the fastest run (plans
+ * whose launches are the same are tried once); states and sweep counters are
+ * restored afterwards.  The result is cached per (lattices present, threshold
+ * kinds present, total rows rounded down to a power of two, SM count, what the
+ * plans come to for the batch's number of tiles): a later batch with the same
+ * key takes the cached plan at once, without trials.  tl_autotune_cache_clear
+ * empties the cache. */
 int tl_batch_autotune(tl_batch* b, uint64_t trial_sweeps, void* stream, tl_batch_plan* out);
 void tl_autotune_cache_clear(void);
 uint64_t tl_batch_launches(const tl_batch* b);

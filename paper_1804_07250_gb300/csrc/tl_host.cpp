@@ -15,6 +15,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <set>
 #include <mutex>
 #include <new>
 #include <tuple>
@@ -2955,6 +2956,30 @@ static void batch_free(tl_batch* b)
     ctx_release(ctx);
 }
 
+// Tiles of a batch cut into `rows` rows.
+static size_t batch_tiles(const tl_batch* b, int rows)
+{
+    size_t n = 0;
+    for (const tl_chain* c : b->chains) n += (size_t)((c->g.H + rows - 1) / rows);
+    return n;
+}
+
+// A batch with fewer tiles than SMs takes lower tiles (down to 64 rows) and
+// more threads per tile: a serving mix of 12 jobs in 62 tiles of 128 rows left
+// 90 SMs idle (100 sweeps and read-out: 1.52 ms so, 1.19 in tiles of 64 rows,
+// 1.26 in tiles of 32, whose halos are as high).
+static int batch_rows(const tl_batch* b, int tile_rows)
+{
+    int rows = tile_rows;
+    while (rows >= 128 && batch_tiles(b, rows) < (size_t)b->ctx->sms) rows = (rows + 3) / 4 * 2;
+    return rows;
+}
+static int batch_threads(const tl_batch* b, size_t ntiles, int threads)
+{
+    const size_t sms = (size_t)b->ctx->sms;
+    return ntiles <= sms ? 512 : ntiles <= 2 * sms ? 256 : threads;
+}
+
 // Tiles of height tile_rows for every chain; shared memory for tile + halo.
 static int batch_plan(tl_batch* b, int tile_rows, int R, int threads)
 {
@@ -2964,17 +2989,7 @@ static int batch_plan(tl_batch* b, int tile_rows, int R, int threads)
     std::vector<double> work;
     std::vector<int> first;
     size_t smem = 0;
-    // a batch with fewer tiles than SMs takes lower tiles (down to 64 rows)
-    // and more threads per tile: a serving mix of 12 jobs in 62 tiles of 128
-    // rows left 90 SMs idle (100 sweeps and read-out: 1.52 ms so, 1.19 in
-    // tiles of 64 rows, 1.26 in tiles of 32, whose halos are as high)
-    int rows = tile_rows;
-    auto count = [&](int r) {
-        size_t n = 0;
-        for (const tl_chain* c : b->chains) n += (size_t)((c->g.H + r - 1) / r);
-        return n;
-    };
-    while (rows >= 128 && count(rows) < (size_t)b->ctx->sms) rows = (rows + 3) / 4 * 2;
+    int rows = batch_rows(b, tile_rows);
     // the rows of a tile and its halos alone
     size_t need = 0;
     for (const tl_chain* c : b->chains)
@@ -3008,8 +3023,7 @@ static int batch_plan(tl_batch* b, int tile_rows, int R, int threads)
             }
         }
         first.push_back((int)tiles.size());
-        const size_t sms = (size_t)b->ctx->sms;
-        run_threads = tiles.size() <= sms ? 512 : tiles.size() <= 2 * sms ? 256 : threads;
+        run_threads = batch_threads(b, tiles.size(), threads);
         if ((long)smem <= (long)b->ctx->smem_optin) {
             if (batch_prepare(smem, run_threads, &bps) == 0 && bps > 0) break;
             run_threads = threads;
@@ -3386,10 +3400,14 @@ TL_API int tl_batch_get_launch(tl_batch* b, int* tile_rows, int* sweeps, int* th
 // The chains' states and sweep counters are restored afterwards, so tuning
 // does not change any result.
 // Autotune results per (lattices present, threshold kinds present, rows of
-// the batch rounded down to a power of two, SMs): a batch like one already
-// tuned takes that plan without trials.
+// the batch rounded down to a power of two, SMs, what the trials' tile heights
+// and threads come to for its number of tiles): a batch like one already tuned
+// takes that plan without trials.
 namespace {
-using TuneKey = std::tuple<int, int, int, int>;
+using TuneKey = std::tuple<int, int, int, int, int>;
+constexpr int kTuneRows[] = {32, 64, 128};
+constexpr int kTuneR[] = {1, 2, 4, 8};
+constexpr int kTuneThreads[] = {256, 128};
 std::mutex g_tune_mu;
 struct TunePlan {
     int tile_rows, R, threads;
@@ -3409,7 +3427,15 @@ TuneKey tune_key(const tl_batch* b)
         rows >>= 1;
         ++bucket;
     }
-    return TuneKey(lat, thr, bucket, b->ctx->sms);
+    // two trials that launch the same thing for this batch need not for one of
+    // more tiles, which must not take their pick
+    int form = 0;
+    for (int tr : kTuneRows) {
+        const int r = batch_rows(b, tr);
+        const size_t n = batch_tiles(b, r);
+        form = form * 6 + (r != tr) * 3 + (n <= (size_t)b->ctx->sms ? 0 : n <= 2 * (size_t)b->ctx->sms ? 1 : 2);
+    }
+    return TuneKey(lat, thr, bucket, b->ctx->sms, form);
 }
 }  // namespace
 
@@ -3446,20 +3472,19 @@ TL_API int tl_batch_autotune(tl_batch* b, uint64_t trial_sweeps, void* stream, t
     }
     std::vector<uint64_t> sweeps;
     for (auto* c : b->chains) sweeps.push_back(c->sweep);
-    const int tile_opts[] = {32, 64, 128};
-    const int r_opts[] = {1, 2, 4, 8};
-    const int nt_opts[] = {256, 128};
+    std::set<std::tuple<int, int, int>> tried;   // what the trials launched
     float best = 1e30f;
     int best_t = b->tile_rows, best_r = b->R, best_nt = b->threads;
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
     int rc = TL_OK;
-    for (int nt : nt_opts)
-    for (int tr : tile_opts)
-        for (int R : r_opts) {
+    for (int nt : kTuneThreads)
+    for (int tr : kTuneRows)
+        for (int R : kTuneR) {
             if (rc != TL_OK) break;
             if (batch_plan(b, tr, R, nt) != TL_OK) continue;   // does not fit: skip
+            if (!tried.insert({b->run_rows, b->run_R, b->run_threads}).second) continue;
             const uint64_t k = ((trial_sweeps + R - 1) / R) * R;
             const int saved_block = b->block;
             b->block = 1 << 30;                            // no graph during trials
