@@ -2036,6 +2036,16 @@ static int zero_counts_if_needed(tl_chain* c, void* stream)
     return TL_OK;
 }
 
+static bool is_capturing(void* stream)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(SS(stream), &st) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
+
 TL_API int tl_run_sweeps(tl_chain* c, uint64_t k, void* stream)
 {
     NvtxRange nvtx_("tl_run_sweeps");
@@ -2044,7 +2054,10 @@ TL_API int tl_run_sweeps(tl_chain* c, uint64_t k, void* stream)
     CUDA_TRY(cudaSetDevice(c->ctx->device));
     TL_TRY(zero_counts_if_needed(c, stream));
     if (k == 0) return TL_OK;
-    if (want_resident(c)) return run_resident(c, k, nullptr, stream);
+    // planning allocates and copies, which a capture does not take: a chain not
+    // planned yet is captured as one launch per pass
+    const bool planned = c->kernel == 1 || c->res_ready || c->res_failed;
+    if ((planned || !is_capturing(stream)) && want_resident(c)) return run_resident(c, k, nullptr, stream);
     if (c->kernel == 2) return fail(TL_EUNSUPPORTED, "resident kernel unavailable: %s", c->res_why.c_str());
     const uint64_t end = c->sweep + k;
     while (c->sweep < end) {
