@@ -2479,6 +2479,7 @@ TL_API int tl_aztec_shuffle(tl_ctx* ctx, int n, uint64_t seed, uint32_t stream_i
                           ? launch_shuffle(sc.seg.data(), (int)sc.seg.size(), n, sc.g.K, (size_t)sc.g.total_words,
                                            sc.xbuf_words, sc.rows, rng, stream)
                           : launch_shuffle_global(n, sc.g.K, (size_t)sc.g.total_words, sc.rows, sc.alt, rng, stream));
+    if (e == cudaSuccess) e = (cudaError_t)launch_shuffle_check(n, sc.g.K, sc.rows, sc.status, stream);
     if (e == cudaSuccess) e = (cudaError_t)launch_unpack(sc.g, sc.rows, dev ? canon : sc.canon, stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&hstatus, sc.status, sizeof(int), cudaMemcpyDeviceToHost, SS(stream));
     if (e == cudaSuccess && !dev) e = cudaMemcpyAsync(canon, sc.canon, ncanon, cudaMemcpyDeviceToHost, SS(stream));
@@ -2486,6 +2487,7 @@ TL_API int tl_aztec_shuffle(tl_ctx* ctx, int n, uint64_t seed, uint32_t stream_i
     if (e != cudaSuccess) return fail(TL_ECUDA, "tl_aztec_shuffle: %s", cudaGetErrorString(e));
     if (hstatus) {
         CUDA_TRY(cudaMemset(sc.status, 0, sizeof(int)));
+        if (hstatus == 2) return fail(TL_ECUDA, "tl_aztec_shuffle: the result is not a tiling");
         return fail(TL_ETIMEOUT, "tl_aztec_shuffle: a bounded wait gave up");
     }
     return TL_OK;

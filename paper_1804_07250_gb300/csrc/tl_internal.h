@@ -91,7 +91,7 @@ struct ShufflePlan {
     size_t smem_bytes;             // dynamic shared memory per CTA
     const int* stripe_lo;          // device [ctas + 1]
     unsigned long long* xbuf;      // device [ctas][2][2][4 halo Kw] tagged words, shared by the launches
-    int* status;                   // device error word: 0 ok, 1 a bounded wait gave up
+    int* status;                   // device error word: 0 ok, 1 a bounded wait gave up, 2 not a tiling
 };
 size_t shuffle_smem_bytes(int local_rows, int Kw);
 size_t shuffle_static_smem(int threads);
@@ -101,6 +101,8 @@ int launch_shuffle(const ShufflePlan* seg, int nseg, int n, int Kw, size_t total
 // One launch per step over two global buffers of total_words words each; the
 // sample ends in A.
 int launch_shuffle_global(int n, int Kw, size_t total_words, uint32_t* A, uint32_t* B, const DevRng& rng, void* stream);
+// Raises the status word to 2 unless the sample is a tiling of the diamond.
+int launch_shuffle_check(int n, int Kw, const uint32_t* rows, int* status, void* stream);
 // seg: [nseg][6] height segments (y, lo, hi, parent, xs, dir); base_scratch: nseg ints.
 int launch_height(const Geom& g, const uint32_t* rows, const int* seg, int nseg, int hw, int hh,
                   int32_t* out, int* base_scratch, void* stream);
