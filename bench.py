@@ -58,10 +58,16 @@ WORKLOADS = {
 UNIFORM_T = 1 << 31
 KERNEL_SOURCES = ["paper_1804_07250_gb300/csrc/tl_words_kernel.cuh", "paper_1804_07250_gb300/csrc/tl_words.cuh",
                   "paper_1804_07250_gb300/csrc/tl_device.cuh"]
-REG_SOURCES = ["paper_1804_07250_gb300/csrc/tl_regdom.cu", "paper_1804_07250_gb300/csrc/tl_words.cuh",
-               "paper_1804_07250_gb300/csrc/tl_device.cuh"]
-# plan kernel -> (ncu kernel name, sources whose hash keys the recorded traffic)
-RESIDENT_KERNELS = {2: ("words_kernel", KERNEL_SOURCES), 3: ("regdom_kernel", REG_SOURCES)}
+# the kernel a chain runs on -> sources whose hash keys the recorded traffic
+CHAIN_KERNELS = {
+    "words_kernel": KERNEL_SOURCES,
+    "regdom_kernel": ["paper_1804_07250_gb300/csrc/tl_regdom.cu", "paper_1804_07250_gb300/csrc/tl_words.cuh",
+                      "paper_1804_07250_gb300/csrc/tl_device.cuh"],
+    "small_kernel": ["paper_1804_07250_gb300/csrc/tl_small.cu", "paper_1804_07250_gb300/csrc/tl_words.cuh",
+                     "paper_1804_07250_gb300/csrc/tl_device.cuh"],
+    "resident_kernel": ["paper_1804_07250_gb300/csrc/tl_resident.cu", "paper_1804_07250_gb300/csrc/tl_device.cuh"],
+    "pass_global_kernel": ["paper_1804_07250_gb300/csrc/tl_kernels.cu", "paper_1804_07250_gb300/csrc/tl_device.cuh"],
+}
 BATCH_SOURCES = ["paper_1804_07250_gb300/csrc/tl_batch.cu", "paper_1804_07250_gb300/csrc/tl_words.cuh",
                  "paper_1804_07250_gb300/csrc/tl_device.cuh"]
 
@@ -332,7 +338,9 @@ def run_ours(args):
     # dominant kernel: the sweep launches of each step, timed with CUDA
     # events on their stream
     plan = chain.plan()
-    if plan["kernel"] in RESIDENT_KERNELS:
+    kname = chain.kernel
+    ksrc, resident = CHAIN_KERNELS[kname], kname != "pass_global_kernel"
+    if resident:
         # the library splits a run into launches of at most spl sweeps and at
         # most 60000 * halo / passes sweeps (16-bit exchange tags)
         per = max(1, 60000 * plan["halo"] // info.passes)
@@ -346,13 +354,10 @@ def run_ours(args):
     alg_bytes_launch = bytes_per_sweep * SWEEPS / k_launches_per_run
     peak, peak_kind = peaks()
     achieved = alg_bytes_launch / (k_ms / 1e3) / 1e9
-    kname, ksrc = RESIDENT_KERNELS.get(plan["kernel"], ("pass_global_kernel", KERNEL_SOURCES))
-    if kname == "regdom_kernel" and wl["size"][0] <= 127 and not wl["density"]:
-        kname = "small_kernel"  # plain runs of small domains take the one-block kernel
     # the recorded traffic is of the workload's own launches: none for
     # another sweep count or plan
     traffic = recorded_traffic(wl["name"], ksrc, {"kernel": plan["kernel"]}) \
-        if plan["kernel"] in RESIDENT_KERNELS and SWEEPS == wl["sweeps"] else None
+        if resident and SWEEPS == wl["sweeps"] else None
 
     # end to end through the C-ABI: every step copies its start state in from
     # page-locked host memory and its results (state, heights and, with

@@ -486,6 +486,11 @@ typedef struct {
 
 int tl_chain_set_plan(tl_chain* c, const tl_plan* plan);
 int tl_chain_get_plan(tl_chain* c, tl_plan* plan);
+/* Name of the kernel that tl_run_sweeps launches for the chain as it is set up
+ * (plan, pass order, densities, flip counts): "small_kernel", "regdom_kernel",
+ * "resident_kernel" (shared memory, a thread per 128 sites), "words_kernel" (a
+ * thread per 32) or "pass_global_kernel".  A static string; NULL for NULL. */
+const char* tl_chain_kernel(tl_chain* c);
 
 /* Wait for the chain's work on `stream` and report a failure of the
  * resident kernel's bounded waits (TL_ETIMEOUT; the state is then

@@ -113,6 +113,7 @@ _SIG = {
     "tl_chain_launches": (_u64, [_vp]),
     "tl_chain_set_plan": (_i, [_vp, ctypes.POINTER(Plan)]),
     "tl_chain_get_plan": (_i, [_vp, ctypes.POINTER(Plan)]),
+    "tl_chain_kernel": (ctypes.c_char_p, [_vp]),
     "tl_chain_sync": (_i, [_vp, _vp]),
     "tl_debug_raise_status": (_i, [_vp, _vp]),
     "tl_debug_build": (_i, []),
@@ -437,6 +438,11 @@ class Chain:
         p = Plan()
         _check(_lib.tl_chain_get_plan(self._h, ctypes.byref(p)))
         return p.as_dict()
+
+    @property
+    def kernel(self) -> str:
+        """Name of the kernel that `run` launches as the chain is set up."""
+        return _lib.tl_chain_kernel(self._h).decode()
 
     def sync(self, stream=None):
         _check(_lib.tl_chain_sync(self._h, _stream(stream)))

@@ -2026,6 +2026,14 @@ static int run_resident(tl_chain* c, uint64_t k, unsigned long long* ring, void*
     return TL_OK;
 }
 
+TL_API const char* tl_chain_kernel(tl_chain* c)
+{
+    if (!c || cudaSetDevice(c->ctx->device) != cudaSuccess) return nullptr;
+    if (!want_resident(c)) return "pass_global_kernel";
+    if (small_run(c)) return "small_kernel";
+    return c->use_reg ? "regdom_kernel" : c->res.slots == 0 ? "resident_kernel" : "words_kernel";
+}
+
 static int zero_counts_if_needed(tl_chain* c, void* stream)
 {
     if (c->counts_dirty) {
