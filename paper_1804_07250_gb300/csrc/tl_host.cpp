@@ -1575,7 +1575,7 @@ static int plan_regdom(tl_chain* c, const RegHull& rh, int h, int max_threads)
         return TL_EUNSUPPORTED;
     }
     int bps = 0;
-    if (regdom_prepare(threads, smem, &bps) != 0 || bps < 1) {
+    if (regdom_prepare(threads, smem, c->ctx->smem_optin, &bps) != 0 || bps < 1) {
         c->res_why = "register-resident kernel does not fit on an SM";
         return TL_EUNSUPPORTED;
     }
@@ -1732,7 +1732,7 @@ static int plan_groups(tl_chain* c, bool fast)
     if (fast) smem += (size_t)cap_items * 8 + 8;
     int bps = 0;
     if ((fast && max_pass > fast_capacity(threads)) || (long)smem > (long)c->ctx->smem_optin ||
-        resident_prepare(g, c->th.kind, threads, fast, smem, &bps) != 0 || bps < 1 || C > bps * c->ctx->sms) {
+        resident_prepare(g, c->th.kind, threads, fast, smem, c->ctx->smem_optin, &bps) != 0 || bps < 1 || C > bps * c->ctx->sms) {
         c->res_why = fast ? "a pass does not fit the single-plane update" : "stripe does not fit in shared memory";
         return TL_EUNSUPPORTED;
     }

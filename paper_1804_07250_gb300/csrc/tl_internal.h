@@ -143,13 +143,9 @@ struct ResidentPlan {
     unsigned int* loaded;          // device [ctas], zeroed with the plan
 };
 
-// Dynamic shared memory up to what the device has left beside the kernel's
-// static: the limit belongs to the kernel, not to a plan, so a plan that set
-// only its own need would take it from the chains planned before.
-int set_smem_limit(const void* kernel);
-
 // Shared-memory attribute and occupancy: blocks that fit on one SM (0 if none).
-int resident_prepare(const Geom& g, int thr_kind, int threads, bool fast, size_t smem_bytes, int* blocks_per_sm);
+int resident_prepare(const Geom& g, int thr_kind, int threads, bool fast, size_t smem_bytes, int smem_optin,
+                     int* blocks_per_sm);
 
 // ring: per-sweep hashes (nullptr = off; must be zeroed).  counts: density
 // counters sampled after every sweep s with s + 1 >= burn and
@@ -187,7 +183,10 @@ struct RegPlan {
     unsigned int* loaded;          // device [ctas], zeroed with the plan
 };
 size_t regdom_smem_bytes(int threads, int max_local_pairs);
-int regdom_prepare(int threads, size_t smem_bytes, int* blocks_per_sm);
+// smem_optin: the most a block can have.  The limit set belongs to the kernel, not
+// to a plan: a plan that set only its own need would lower it under the chains
+// planned before.
+int regdom_prepare(int threads, size_t smem_bytes, int smem_optin, int* blocks_per_sm);
 int launch_regdom(const Geom& g, uint32_t* rows, const RegPlan& plan, uint32_t sweep0, uint32_t nsweeps,
                   const DevRng& rng, unsigned int epoch, unsigned long long* ring, uint32_t* counts, uint64_t burn,
                   uint32_t stride, const uint8_t* colours, unsigned long long* flips, void* stream);

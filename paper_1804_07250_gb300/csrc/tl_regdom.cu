@@ -632,13 +632,17 @@ size_t regdom_smem_bytes(int threads, int max_local_pairs)
     return b;
 }
 
-int regdom_prepare(int threads, size_t smem_bytes, int* blocks_per_sm)
+int regdom_prepare(int threads, size_t smem_bytes, int smem_optin, int* blocks_per_sm)
 {
     *blocks_per_sm = 0;
     const void* k = reg_pick(threads, false, false);
-    for (int v = 0; v < 4; ++v)
-        if (const int e = set_smem_limit(reg_pick(threads, (v & 1) != 0, (v & 2) != 0))) return e;
-    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, threads, smem_bytes);
+    // the kernels' limit, not this plan's need: all of a block's shared memory but
+    // 1 KB, where their static (at most 128 bytes) lies
+    cudaError_t e = cudaSuccess;
+    for (int v = 0; v < 4 && e == cudaSuccess; ++v)
+        e = cudaFuncSetAttribute(reg_pick(threads, (v & 1) != 0, (v & 2) != 0),
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin - 1024);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, threads, smem_bytes);
     if (e != cudaSuccess) cudaGetLastError();
     return (int)e;
 }

@@ -504,25 +504,17 @@ static const void* pick(int lattice, int tk, int threads, bool fast)
                          : reinterpret_cast<const void*>(&resident_kernel<LAT_DOMINO, THR_SCALAR, 512, false>);
 }
 
-int set_smem_limit(const void* kernel)
-{
-    int dev = 0, optin = 0;
-    cudaFuncAttributes fa{};
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kernel);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
-    if (e != cudaSuccess) cudaGetLastError();
-    return (int)e;
-}
-
-int resident_prepare(const Geom& g, int thr_kind, int threads, bool fast, size_t smem_bytes, int* blocks_per_sm)
+int resident_prepare(const Geom& g, int thr_kind, int threads, bool fast, size_t smem_bytes, int smem_optin,
+                     int* blocks_per_sm)
 {
     *blocks_per_sm = 0;
     const void* k = pick(g.lattice, thr_kind, threads, fast);
-    if (const int e = set_smem_limit(k)) return e;
-    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, threads, smem_bytes);
+    // the kernel's limit, not this plan's need
+    cudaFuncAttributes fa{};
+    cudaError_t e = cudaFuncGetAttributes(&fa, k);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin - (int)fa.sharedSizeBytes);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, threads, smem_bytes);
     if (e != cudaSuccess) cudaGetLastError();
     return (int)e;
 }
