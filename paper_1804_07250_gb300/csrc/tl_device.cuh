@@ -327,7 +327,7 @@ TL_DEV void domino_update(uint32_t* row, int64_t RW, int K, int y, int m, uint32
 // the next group's first site from `onext` (bit 0 of that group's first
 // random word; 0 if that group holds no domain site).  This group therefore
 // never writes bit 31 of word k0-1: the group to its left does, which is why
-// the planner lists one extra group left of every active range.  Because a
+// the kernel lists one extra group left of every active range.  Because a
 // group reads its neighbours' boundary words, all groups of a pass must
 // finish domino_fast_compute before any of them runs domino_fast_store.
 struct DominoFast {

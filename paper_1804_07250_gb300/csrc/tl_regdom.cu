@@ -196,8 +196,11 @@ TL_DEV void pair_count_sliced(const PairWords& pw, int j0, int64_t i0, int64_t R
 // COUNT: the chain counts its accepted flips (a separate instantiation, so
 // the default path carries no counter).  RND: the colour of every pass slot
 // comes from the host's table (random order) instead of slot s updating
-// colour s.
-template <int NT, bool COUNT, bool RND>
+// colour s.  SHORT: launches that end before their first exchange, which mark
+// their stripes loaded and wait for the neighbours' marks before they write back
+// (its own build: the few instructions take a register of the long launches', 1.41
+// -> 1.42 us a sweep of Aztec 2048).
+template <int NT, bool COUNT, bool RND, bool SHORT>
 __global__ void __launch_bounds__(NT, 1) regdom_kernel(const RegParams P)
 {
     extern __shared__ uint4 rsm[];
@@ -309,7 +312,7 @@ __global__ void __launch_bounds__(NT, 1) regdom_kernel(const RegParams P)
     const uint32_t grp1 = grp0 + (uint32_t)Kg;
 
     const uint64_t total = (uint64_t)P.nsweeps * 2;
-    if (gridDim.x > 1 && (uint64_t)P.nsweeps * 2 <= (uint64_t)P.halo) {
+    if constexpr (SHORT) {
         __threadfence();   // the loads into registers
         __syncthreads();
         if (tid == 0) stripe_mark_loaded(P.loaded, P.epoch);
@@ -464,7 +467,7 @@ __global__ void __launch_bounds__(NT, 1) regdom_kernel(const RegParams P)
             }
         }
         done += (uint64_t)hc;
-        if (done >= total) break;
+        if (SHORT || done >= total) break;
 
         // ---- exchange of boundary rows with the neighbouring stripes ----
         const int par = cyc & 1;
@@ -587,9 +590,8 @@ __global__ void __launch_bounds__(NT, 1) regdom_kernel(const RegParams P)
         }
         ++cyc;
     }
-    if (gridDim.x > 1 && (uint64_t)P.nsweeps * 2 <= (uint64_t)P.halo &&
-        !__syncthreads_and(tid != 0 || stripe_neighbours_loaded(P.loaded, P.epoch, P.status)))
-        return;
+    if constexpr (SHORT)
+        if (!__syncthreads_and(tid != 0 || stripe_neighbours_loaded(P.loaded, P.epoch, P.status))) return;
     if (COUNT && nflip) atomicAdd(P.flips, (unsigned long long)nflip);
     if (owned && inb) {
         uint32_t* b0 = P.rows0 + (int64_t)y0 * RW + k0;
@@ -607,18 +609,24 @@ __global__ void __launch_bounds__(NT, 1) regdom_kernel(const RegParams P)
     }
 }
 
-template <bool COUNT, bool RND>
+template <bool COUNT, bool RND, bool SHORT>
 static const void* reg_pick_nt(int threads)
 {
-    if (threads > 384) return reinterpret_cast<const void*>(&regdom_kernel<512, COUNT, RND>);
-    if (threads > 256) return reinterpret_cast<const void*>(&regdom_kernel<384, COUNT, RND>);
-    return reinterpret_cast<const void*>(&regdom_kernel<256, COUNT, RND>);
+    if (threads > 384) return reinterpret_cast<const void*>(&regdom_kernel<512, COUNT, RND, SHORT>);
+    if (threads > 256) return reinterpret_cast<const void*>(&regdom_kernel<384, COUNT, RND, SHORT>);
+    return reinterpret_cast<const void*>(&regdom_kernel<256, COUNT, RND, SHORT>);
 }
 
-static const void* reg_pick(int threads, bool count, bool rnd)
+template <bool SHORT>
+static const void* reg_pick_form(int threads, bool count, bool rnd)
 {
-    if (count) return rnd ? reg_pick_nt<true, true>(threads) : reg_pick_nt<true, false>(threads);
-    return rnd ? reg_pick_nt<false, true>(threads) : reg_pick_nt<false, false>(threads);
+    if (count) return rnd ? reg_pick_nt<true, true, SHORT>(threads) : reg_pick_nt<true, false, SHORT>(threads);
+    return rnd ? reg_pick_nt<false, true, SHORT>(threads) : reg_pick_nt<false, false, SHORT>(threads);
+}
+
+static const void* reg_pick(int threads, bool count, bool rnd, bool shrt)
+{
+    return shrt ? reg_pick_form<true>(threads, count, rnd) : reg_pick_form<false>(threads, count, rnd);
 }
 
 size_t regdom_smem_bytes(int threads, int max_local_pairs)
@@ -635,12 +643,12 @@ size_t regdom_smem_bytes(int threads, int max_local_pairs)
 int regdom_prepare(int threads, size_t smem_bytes, int smem_optin, int* blocks_per_sm)
 {
     *blocks_per_sm = 0;
-    const void* k = reg_pick(threads, false, false);
+    const void* k = reg_pick(threads, false, false, false);
     // the kernels' limit, not this plan's need: all of a block's shared memory but
     // 1 KB, where their static (at most 128 bytes) lies
     cudaError_t e = cudaSuccess;
-    for (int v = 0; v < 4 && e == cudaSuccess; ++v)
-        e = cudaFuncSetAttribute(reg_pick(threads, (v & 1) != 0, (v & 2) != 0),
+    for (int v = 0; v < 8 && e == cudaSuccess; ++v)
+        e = cudaFuncSetAttribute(reg_pick(threads, (v & 1) != 0, (v & 2) != 0, (v & 4) != 0),
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin - 1024);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, threads, smem_bytes);
     if (e != cudaSuccess) cudaGetLastError();
@@ -671,8 +679,10 @@ int launch_regdom(const Geom& g, uint32_t* rows, const RegPlan& plan, uint32_t s
     P.stride = stride;
     P.epoch = epoch;
     void* args[] = {&P};
-    return (int)cudaLaunchCooperativeKernel(reg_pick(plan.threads, flips != nullptr, colours != nullptr), dim3(plan.ctas), dim3(plan.threads), args,
-                                            plan.smem_bytes, reinterpret_cast<cudaStream_t>(stream));
+    const bool shrt = plan.ctas > 1 && (uint64_t)nsweeps * 2 <= (uint64_t)plan.halo;   // no exchange
+    return (int)cudaLaunchCooperativeKernel(reg_pick(plan.threads, flips != nullptr, colours != nullptr, shrt),
+                                            dim3(plan.ctas), dim3(plan.threads), args, plan.smem_bytes,
+                                            reinterpret_cast<cudaStream_t>(stream));
 }
 
 // This file's debug word (failures, then the id, index and bound of the

@@ -1,5 +1,5 @@
-// Resident multi-sweep kernel of every chain but the dominoes at t = 2^31
-// (cooperative launch, one CTA per SM).
+// Resident multi-sweep kernel of every chain but the dominoes at t = 2^31 and
+// large stripes with thresholds of few bits (cooperative launch, one CTA per SM).
 //
 // The paper launches Rotate and Update once per half-step and moves the whole
 // tiling through device memory every time (Sec. 2.2).  Here one launch runs
