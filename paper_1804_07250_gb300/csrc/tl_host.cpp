@@ -1599,6 +1599,7 @@ static int plan_regdom(tl_chain* c, const RegHull& rh, int h, int max_threads)
     c->reg.threads = threads;
     c->reg.halo = h;
     c->reg.smem_bytes = smem;
+    c->reg.smem_optin = c->ctx->smem_optin;
     c->reg.stripe_lo = c->stripe_d;
     c->reg.hull = c->hull_d;
     c->reg.xbuf = c->xbuf_d;
@@ -2487,8 +2488,8 @@ TL_API int tl_aztec_shuffle(tl_ctx* ctx, int n, uint64_t seed, uint32_t stream_i
                           ? launch_shuffle(sc.seg.data(), (int)sc.seg.size(), n, sc.g.K, (size_t)sc.g.total_words,
                                            sc.xbuf_words, sc.rows, rng, stream)
                           : launch_shuffle_global(n, sc.g.K, (size_t)sc.g.total_words, sc.rows, sc.alt, rng, stream));
-    if (e == cudaSuccess) e = (cudaError_t)launch_shuffle_check(n, sc.g.K, sc.rows, sc.status, stream);
-    if (e == cudaSuccess) e = (cudaError_t)launch_unpack(sc.g, sc.rows, dev ? canon : sc.canon, stream);
+    if (e == cudaSuccess)
+        e = (cudaError_t)launch_unpack_diamond(sc.g, sc.rows, dev ? canon : sc.canon, n, sc.status, stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&hstatus, sc.status, sizeof(int), cudaMemcpyDeviceToHost, SS(stream));
     if (e == cudaSuccess && !dev) e = cudaMemcpyAsync(canon, sc.canon, ncanon, cudaMemcpyDeviceToHost, SS(stream));
     if (e == cudaSuccess) e = cudaStreamSynchronize(SS(stream));

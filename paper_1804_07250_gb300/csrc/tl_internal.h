@@ -63,6 +63,9 @@ struct HeightPlan {
 // ---- kernel launchers (tl_kernels.cu); all return cudaError_t as int ----
 int launch_pack(const Geom& g, const uint8_t* canon_dev, uint32_t* rows, void* stream);
 int launch_unpack(const Geom& g, const uint32_t* rows, uint8_t* canon_dev, void* stream);
+// The same of a diamond of order n, raising the status word to 2 unless the edges
+// are a tiling of it.
+int launch_unpack_diamond(const Geom& g, const uint32_t* rows, uint8_t* canon_dev, int n, int* status, void* stream);
 // `pass`: the colour class updated; `slot`: the pass slot that keys the
 // random numbers (equal unless the pass order is random).
 // flips: accepted-flip counter (nullptr = not counted).
@@ -101,8 +104,6 @@ int launch_shuffle(const ShufflePlan* seg, int nseg, int n, int Kw, size_t total
 // One launch per step over two global buffers of total_words words each; the
 // sample ends in A.
 int launch_shuffle_global(int n, int Kw, size_t total_words, uint32_t* A, uint32_t* B, const DevRng& rng, void* stream);
-// Raises the status word to 2 unless the sample is a tiling of the diamond.
-int launch_shuffle_check(int n, int Kw, const uint32_t* rows, int* status, void* stream);
 // seg: [nseg][6] height segments (y, lo, hi, parent, xs, dir); base_scratch: nseg ints.
 int launch_height(const Geom& g, const uint32_t* rows, const int* seg, int nseg, int hw, int hh,
                   int32_t* out, int* base_scratch, void* stream);
@@ -176,6 +177,7 @@ struct RegPlan {
     int threads;                   // threads per CTA (<= 512, multiple of 32)
     int halo;                      // even
     size_t smem_bytes;
+    int smem_optin;                // the most shared memory a block can have
     const int* stripe_lo;          // device [ctas + 1], even
     const int2* hull;              // device [pairs]
     unsigned long long* xbuf;      // device [ctas][2][2][halo / 2][16][Kg][2]

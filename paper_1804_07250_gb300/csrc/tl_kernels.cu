@@ -159,6 +159,13 @@ TL_DEV uint32_t plane_bits(const uint32_t* p, int K, int j0)
     const uint32_t a = k >= 0 && k < K ? p[k] : 0u, b = k + 1 >= 0 && k + 1 < K ? p[k + 1] : 0u;
     return __funnelshift_r(a, b, j0 & 31);
 }
+// Bits [lo, hi] of 16, clipped to them.
+TL_DEV uint32_t cell_span(int lo, int hi)
+{
+    lo = lo > 0 ? lo : 0;
+    hi = hi < 15 ? hi : 15;
+    return hi < lo ? 0u : (2u << hi) - (1u << lo);
+}
 // Bit i of the low 16 to position 2 i; of the low 8 to position 3 i.
 TL_DEV uint32_t spread2(uint32_t x)
 {
@@ -167,6 +174,12 @@ TL_DEV uint32_t spread2(uint32_t x)
     x = (x | (x << 4)) & 0x0F0F0F0Fu;
     x = (x | (x << 2)) & 0x33333333u;
     return (x | (x << 1)) & 0x55555555u;
+}
+// Edges x0 .. x0 + 16 (at least) of a row from its planes of even and odd x.
+TL_DEV uint32_t bits2(const uint32_t* p, int K, int x0)
+{
+    const int j0 = x0 >> 1;
+    return (spread2(plane_bits(p, K, j0)) | spread2(plane_bits(p + K, K, j0)) << 1) >> (x0 & 1);
 }
 TL_DEV uint32_t spread3(uint32_t x)
 {
@@ -184,7 +197,14 @@ TL_DEV uint32_t spread3(uint32_t x)
 // narrow ones the lanes.
 // us: square 2048 36 with a thread a byte, 6.0 with a warp a row, 5.9 so; 60000 x 4
 // 5.7, 39, 1.9; 200 x 20000 35, 15, 7.9; 2 x 30000 2.9, 20, 3.1.
-__global__ void unpack_kernel(const uint32_t* __restrict__ rows, uint8_t* __restrict__ canon, Geom g)
+//
+// CHECK: dominoes, the units of horizontal edges also look at the other edges of
+// their 16 cells: exactly one domino on every cell of the diamond of order n and
+// none elsewhere, or the status word is raised (domino shuffling's steps look at
+// edges only and would not notice; a launch of its own took 4 us, a check of every
+// block the steps read 1 to 3% of a sample).
+template <bool CHECK>
+__global__ void unpack_kernel(const uint32_t* __restrict__ rows, uint8_t* __restrict__ canon, Geom g, int order, int* status)
 {
     const uint32_t units = (uint32_t)(g.W + 30) >> 4, n = (uint32_t)(g.ntype * g.H) * units;
     for (uint32_t u = blockIdx.x * blockDim.x + threadIdx.x; u < n; u += gridDim.x * blockDim.x) {
@@ -196,9 +216,15 @@ __global__ void unpack_kernel(const uint32_t* __restrict__ rows, uint8_t* __rest
         const int x0 = 16 * (int)(u - r * units) - lead;   // may be negative: those bits are not stored
         if (x0 >= g.W) continue;
         uint32_t v;
-        if (g.npar == 2) {
-            const int j0 = x0 >> 1;
-            v = (spread2(plane_bits(p, g.K, j0)) | spread2(plane_bits(p + g.K, g.K, j0)) << 1) >> (x0 & 1);
+        if (CHECK || g.npar == 2) {
+            v = bits2(p, g.K, x0);
+            if (CHECK && type == 0 && y < 2 * order) {
+                const uint32_t b = bits2(p + g.row_words, g.K, x0), c = bits2(p + 2 * g.K, g.K, x0), d = c >> 1;
+                const int w = y < order ? y + 1 : 2 * order - y;   // cells order - w .. order + w - 1 of the row
+                const uint32_t in = cell_span(order - w - x0, order + w - 1 - x0);
+                const uint32_t one = (v ^ b ^ c ^ d) & ~((v & b) | (c & d)), any = v | b | c | d;
+                if (((one ^ in) | (any & ~in)) & 0xFFFFu) atomicCAS(status, 0, 2);
+            }
         } else {
             const int j0 = (x0 + 18) / 3 - 6;   // floor, x0 > -16
             v = (spread3(plane_bits(p, g.K, j0)) | spread3(plane_bits(p + g.K, g.K, j0)) << 1 |
@@ -236,7 +262,15 @@ int launch_pack(const Geom& g, const uint8_t* canon_dev, uint32_t* rows, void* s
 
 int launch_unpack(const Geom& g, const uint32_t* rows, uint8_t* canon_dev, void* stream)
 {
-    unpack_kernel<<<grid_for((int64_t)g.ntype * g.H * ((g.W + 30) / 16), 256), 256, 0, S(stream)>>>(rows, canon_dev, g);
+    unpack_kernel<false><<<grid_for((int64_t)g.ntype * g.H * ((g.W + 30) / 16), 256), 256, 0, S(stream)>>>(rows, canon_dev, g, 0,
+                                                                                                          nullptr);
+    return (int)cudaGetLastError();
+}
+
+int launch_unpack_diamond(const Geom& g, const uint32_t* rows, uint8_t* canon_dev, int n, int* status, void* stream)
+{
+    unpack_kernel<true><<<grid_for((int64_t)g.ntype * g.H * ((g.W + 30) / 16), 256), 256, 0, S(stream)>>>(rows, canon_dev, g, n,
+                                                                                                         status);
     return (int)cudaGetLastError();
 }
 

@@ -647,8 +647,8 @@ int regdom_prepare(int threads, size_t smem_bytes, int smem_optin, int* blocks_p
     // the kernels' limit, not this plan's need: all of a block's shared memory but
     // 1 KB, where their static (at most 128 bytes) lies
     cudaError_t e = cudaSuccess;
-    for (int v = 0; v < 8 && e == cudaSuccess; ++v)
-        e = cudaFuncSetAttribute(reg_pick(threads, (v & 1) != 0, (v & 2) != 0, (v & 4) != 0),
+    for (int v = 0; v < 4 && e == cudaSuccess; ++v)
+        e = cudaFuncSetAttribute(reg_pick(threads, (v & 1) != 0, (v & 2) != 0, false),
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin - 1024);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, threads, smem_bytes);
     if (e != cudaSuccess) cudaGetLastError();
@@ -680,8 +680,12 @@ int launch_regdom(const Geom& g, uint32_t* rows, const RegPlan& plan, uint32_t s
     P.epoch = epoch;
     void* args[] = {&P};
     const bool shrt = plan.ctas > 1 && (uint64_t)nsweeps * 2 <= (uint64_t)plan.halo;   // no exchange
-    return (int)cudaLaunchCooperativeKernel(reg_pick(plan.threads, flips != nullptr, colours != nullptr, shrt),
-                                            dim3(plan.ctas), dim3(plan.threads), args, plan.smem_bytes,
+    const void* k = reg_pick(plan.threads, flips != nullptr, colours != nullptr, shrt);
+    if (shrt) {   // its limit is set here: plans need not pay for it
+        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, plan.smem_optin - 1024);
+        if (e != cudaSuccess) return (int)e;
+    }
+    return (int)cudaLaunchCooperativeKernel(k, dim3(plan.ctas), dim3(plan.threads), args, plan.smem_bytes,
                                             reinterpret_cast<cudaStream_t>(stream));
 }
 

@@ -391,40 +391,6 @@ __global__ void shuffle_plain_kernel(const uint32_t* __restrict__ B, uint32_t* _
     }
 }
 
-// The finished sample: exactly one domino on every cell of the diamond and no
-// edge elsewhere, 32 cells of one column parity a thread and turn.  (The steps
-// look at edges only; a check of every block they read costs 1 to 3% of a
-// sample, this one 4 us at order 2048.)
-__global__ void shuffle_check_kernel(const uint32_t* __restrict__ rows, int n, int Kw, int* status)
-{
-    const int64_t RW = 4 * (int64_t)Kw, total = 2 * (int64_t)n * Kw;
-    bool bad = false;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        const int y = (int)(i / Kw), k = (int)(i - (int64_t)y * Kw);
-        const uint32_t* p = rows + y * RW + k;   // row y: He, Ho, Ve, Vo
-        const int w = y < n ? y + 1 : 2 * n - y;  // cells n - w .. n + w - 1 of this row
-        const uint32_t ve1 = k + 1 < Kw ? p[2 * Kw + 1] : 0u;
-#pragma unroll
-        for (int r = 0; r < 2; ++r) {
-            const uint32_t a = p[r * Kw], b = p[RW + r * Kw], c = p[(2 + r) * Kw],
-                           d = r ? (p[2 * Kw] >> 1) | (ve1 << 31) : p[3 * Kw];
-            const uint32_t in = span_mask(((n - w + 1 - r) >> 1) - 32 * k, ((n + w - 1 - r) >> 1) - 32 * k);
-            const uint32_t one = (a ^ b ^ c ^ d) & ~((a & b) | (c & d));
-            bad |= one != in || ((a | b | c | d) & ~in) != 0u;
-        }
-    }
-    if (bad) atomicCAS(status, 0, 2);
-}
-
-int launch_shuffle_check(int n, int Kw, const uint32_t* rows, int* status, void* stream)
-{
-    const int64_t total = 2 * (int64_t)n * Kw;
-    const int64_t blocks = (total + 255) / 256;
-    shuffle_check_kernel<<<(unsigned)(blocks < 4864 ? blocks : 4864), 256, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
-        rows + 4 * (size_t)Kw, n, Kw, status);
-    return (int)cudaGetLastError();
-}
-
 static inline cudaStream_t SS_(void* s) { return reinterpret_cast<cudaStream_t>(s); }
 
 size_t shuffle_smem_bytes(int nloc, int Kw) { return (size_t)nloc * 4 * Kw * 4 * 2; }
