@@ -2055,6 +2055,14 @@ static bool is_capturing(void* stream)
     return st != cudaStreamCaptureStatusNone;
 }
 
+// Planning allocates and copies, which a capture does not take: a chain not
+// planned yet is captured as one launch per pass.
+static bool want_resident_on(tl_chain* c, void* stream)
+{
+    const bool planned = c->kernel == 1 || c->res_ready || c->res_failed;
+    return (planned || !is_capturing(stream)) && want_resident(c);
+}
+
 TL_API int tl_run_sweeps(tl_chain* c, uint64_t k, void* stream)
 {
     NvtxRange nvtx_("tl_run_sweeps");
@@ -2063,10 +2071,7 @@ TL_API int tl_run_sweeps(tl_chain* c, uint64_t k, void* stream)
     CUDA_TRY(cudaSetDevice(c->ctx->device));
     TL_TRY(zero_counts_if_needed(c, stream));
     if (k == 0) return TL_OK;
-    // planning allocates and copies, which a capture does not take: a chain not
-    // planned yet is captured as one launch per pass
-    const bool planned = c->kernel == 1 || c->res_ready || c->res_failed;
-    if ((planned || !is_capturing(stream)) && want_resident(c)) return run_resident(c, k, nullptr, stream);
+    if (want_resident_on(c, stream)) return run_resident(c, k, nullptr, stream);
     if (c->kernel == 2) return fail(TL_EUNSUPPORTED, "resident kernel unavailable: %s", c->res_why.c_str());
     const uint64_t end = c->sweep + k;
     while (c->sweep < end) {
@@ -2187,7 +2192,7 @@ TL_API int tl_run_sweeps_hashed(tl_chain* c, uint64_t k, uint64_t* ring, void* s
         dring = tmp;
     }
     int rc = TL_OK;
-    if (k && want_resident(c)) {
+    if (k && want_resident_on(c, stream)) {
         rc = zero_counts_if_needed(c, stream);
         cudaError_t e = cudaMemsetAsync(dring, 0, k * 8, SS(stream));
         if (rc == TL_OK && e != cudaSuccess) rc = fail(TL_ECUDA, "hash ring: %s", cudaGetErrorString(e));

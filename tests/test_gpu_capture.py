@@ -38,3 +38,19 @@ def test_captured_sweeps(T, kind, size, t, planned):
     ch.run(10)
     ref.run(10)
     assert ch.state_hash() == ref.state_hash()
+
+
+@pytest.mark.parametrize("planned", [False, True])
+def test_captured_hashed_run(T, planned):
+    import torch
+    ctx, dom, th = T.Context(0), T.Domain.aztec(3), T.thresholds(scalar=3 << 29)
+    ch, ref = (T.Chain(ctx, dom, seed=6, th=th) for _ in range(2))
+    if planned:
+        ch.plan()
+    ring = torch.zeros(12, dtype=torch.int64, device="cuda")
+    stream, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        ch.run_hashed(12, ring, stream=stream)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert np.array_equal(ring.cpu().numpy().view(np.uint64), ref.run_hashed(12))
